@@ -417,8 +417,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
         __syncwarp();
     } else {
         // ------------------------------------- MMA issuers: warp 8 -> slot 0, warp 10 -> slot 1
-        if (elect_one()) {
-            const int slot = warp == 8 ? 0 : 1;
+        // The whole warp walks the loop and every value in it is warp-uniform (broadcasts and votes
+        // tell the compiler so); only the tensor-core instructions are issued by one lane.  Their
+        // descriptors and addresses then live in uniform registers: a loop run by a single elected
+        // lane has to move six operands there for every MMA.
+        {
+            const bool leader = elect_one();
+            const int slot = __shfl_sync(0xffffffffu, warp, 0) == 8 ? 0 : 1;
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
             const uint32_t idesc_qk = make_idesc_bf16(kBM, kBN, false, false);
             const uint32_t idesc_pv = make_idesc_bf16(kBM, kD, false, true);
             // Descriptors differ from tile to tile only in the 14-bit start-address field, so the
@@ -426,30 +432,38 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             const uint64_t desc_k = make_smem_desc_sw128(0, 16, 1024);             // K-major Q / K
             const uint64_t desc_v = make_smem_desc_sw128(0, kHalfBytes, 1024);     // MN-major V
             const uint64_t desc_q = desc_k + ((sQ + slot * kQBytes) >> 4);
-            const uint32_t tSslot = tmem + slot * 128;
-            const uint32_t tOslot = tmem + 256 + slot * kD;
+            const uint32_t tSslot = tm + slot * 128;
+            const uint32_t tOslot = tm + 256 + slot * kD;
             auto issue_qk = [&](int buf, int stage) {          // S[buf] = Q K^T, N = 64 keys
                 const uint64_t b = desc_k + ((sKV + stage * kTileBytes) >> 4);
+                if (leader) {
+                    if constexpr (GATHER) fence_proxy_async_smem();     // the tile came through the generic proxy
 #pragma unroll
-                for (int kk = 0; kk < kD / 16; ++kk) {
-                    const uint32_t qoff = ((kk >> 2) * kQHalf + (kk & 3) * 32) >> 4;
-                    const uint32_t koff = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
-                    umma_ss(tSslot + buf * kBN, desc_q + qoff, b + koff, idesc_qk, kk > 0);
+                    for (int kk = 0; kk < kD / 16; ++kk) {
+                        const uint32_t qoff = ((kk >> 2) * kQHalf + (kk & 3) * 32) >> 4;
+                        const uint32_t koff = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
+                        umma_ss(tSslot + buf * kBN, desc_q + qoff, b + koff, idesc_qk, kk > 0);
+                    }
+                    umma_commit(s_full(slot, buf));
+                    umma_commit(kv_empty(stage));
                 }
+                __syncwarp();
             };
             auto issue_pv = [&](int buf, int stage, bool first) {   // O += P[buf] V, K = 64 keys
                 const uint64_t b = desc_v + ((sKV + stage * kTileBytes) >> 4);
+                if (leader) {
+                    if constexpr (GATHER) fence_proxy_async_smem();
 #pragma unroll
-                for (int kk = 0; kk < kBN / 16; ++kk)
-                    umma_ts(tOslot, tSslot + buf * kBN + kk * 8, b + kk * (2048 >> 4), idesc_pv,
-                            !(first && kk == 0));
+                    for (int kk = 0; kk < kBN / 16; ++kk)
+                        umma_ts(tOslot, tSslot + buf * kBN + kk * 8, b + kk * (2048 >> 4), idesc_pv,
+                                !(first && kk == 0));
+                    umma_commit(kv_empty(stage));
+                }
+                __syncwarp();
             };
-            // The issuing thread shares its scheduler with two softmax warps, so its own
-            // instruction count per tile matters: ring positions are advanced incrementally (no
-            // division), and the abort flag is only looked at when a wait fails.
             bool ok = true;
             auto wait = [&](uint32_t bar, uint32_t ph, int code) {
-                if (!mbar_wait(bar, ph)) { fail(code); ok = false; }
+                if (!mbar_wait_warp(bar, ph)) { if (leader) fail(code); ok = false; }
             };
             struct Cursor {                      // position of a ring entry: stage and phase bit
                 uint32_t st, ph;
@@ -463,12 +477,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             Cursor cur{0u, 0u};                  // first ring entry of the next run
             uint32_t qcnt = 0, tc = 0;           // tc: tiles this slot has processed so far
             while (ok && iter.next(p, g)) {
-                const int n = g.t1 - g.t0;
-                if (slot >= g.n_slots) {
+                const int n = __shfl_sync(0xffffffffu, g.t1 - g.t0, 0);
+                if (slot >= __shfl_sync(0xffffffffu, g.n_slots, 0)) {
                     // nothing to compute for this slot, but every K/V stage is released by both issuers
                     for (int e = 0; e < 2 * n && ok; ++e) {
                         wait(kv_full(cur.st), cur.ph, 206);
-                        if (ok) mbar_arrive(kv_empty(cur.st));
+                        if (ok && leader) mbar_arrive(kv_empty(cur.st));
                         cur.step(1);
                     }
                     continue;
@@ -481,11 +495,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 for (int i = 0; i < 2 && i < n && ok; ++i) {        // S(0), S(1)
                     wait(kv_full(ck.st), ck.ph, 202);
                     if (!ok) break;
-                    if constexpr (GATHER) fence_proxy_async_smem();   // the tile came through the generic proxy
                     tc_fence_after_sync();
                     issue_qk((tc + i) & 1, ck.st);
-                    umma_commit(s_full(slot, (tc + i) & 1));
-                    umma_commit(kv_empty(ck.st));
                     ck.step(2);
                 }
                 if (n == 1) ck.step(2);                              // keep ck two tiles ahead of cv
@@ -494,22 +505,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     const int buf = (tc + i) & 1;
                     wait(kv_full(cv.st), cv.ph, 203);
                     if (!ok) break;
-                    if (!mbar_wait_spin(p_full(slot, buf), ((tc + i) >> 1) & 1u)) { fail(205); ok = false; break; }
-                    if constexpr (GATHER) fence_proxy_async_smem();
+                    wait(p_full(slot, buf), ((tc + i) >> 1) & 1u, 205);
+                    if (!ok) break;
                     tc_fence_after_sync();
                     issue_pv(buf, cv.st, i == 0);
-                    umma_commit(kv_empty(cv.st));
                     if (i + 2 < n) {                                // S(i+2) reuses the buffer P(i) was read from
                         wait(kv_full(ck.st), ck.ph, 204);
                         if (!ok) break;
-                        if constexpr (GATHER) fence_proxy_async_smem();
                         issue_qk(buf, ck.st);
-                        umma_commit(s_full(slot, buf));
-                        umma_commit(kv_empty(ck.st));
                     } else if (i + 2 == n) {
-                        umma_commit(pv_done(slot));                 // lets the last tile's softmax know O is at rest
+                        if (leader) umma_commit(pv_done(slot));     // lets the last tile's softmax know O is at rest
                     }
-                    if (i == n - 1) { umma_commit(o_done(slot)); umma_commit(q_empty(slot)); }
+                    if (i == n - 1 && leader) { umma_commit(o_done(slot)); umma_commit(q_empty(slot)); }
+                    __syncwarp();
                     cv.step(2);
                     ck.step(2);
                 }

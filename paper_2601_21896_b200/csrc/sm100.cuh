@@ -84,6 +84,20 @@ __device__ __forceinline__ bool mbar_wait_spin(uint32_t bar, uint32_t parity) {
     return mbar_wait(bar, parity);
 }
 
+// The bounded wait of a whole warp: all 32 lanes poll and leave together with one answer, which the
+// vote makes warp-uniform for the compiler.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+#pragma unroll 1
+    for (int i = 0; i < 2048; ++i)
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const uint64_t t0 = global_timer_ns();
+#pragma unroll 1
+    while (true) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, global_timer_ns() - t0 > kWaitLimitNs)) return false;
+    }
+}
+
 // ------------------------------------------------------------------------------- fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
