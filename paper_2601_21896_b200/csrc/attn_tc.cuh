@@ -9,7 +9,7 @@
 // grid is persistent: one CTA per SM.  Items go out whole, round by round, while no CTA exceeds its
 // even share of the work; the key tiles of the items that are left are laid end to end and cut
 // into contiguous shares, one per CTA, so that every CTA ends with the same total whatever the item
-// count (a tile with both slots live costs 8 units, with one slot 6: a lone slot has no partner to
+// count (a tile with both slots live costs 8 units, with one slot 7: a lone slot has no partner to
 // hide its softmax behind).  A CTA whose share covers only
 // part of an item's keys writes an unnormalised partial (O, running max, row sum) to the
 // workspace; a second small kernel merges the partials of each split item in key order, which
@@ -98,7 +98,8 @@ struct Seg {
                          // earlier CTA; 1: begins an item that a later CTA continues
 };
 
-constexpr int kCost2 = 8, kCost1 = 6;   // cost of one key tile with two / one live slots (best of 5..7 on every measured workload)
+constexpr int kCost2 = 8, kCost1 = 7;   // cost of one key tile with two / one live slots (with 6 the CTAs that got a
+                                        // one-slot item ended 20 to 30 us after the others)
 
 struct StreamCost {
     int64_t nqp, nt, head_cost;
@@ -310,8 +311,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
     auto p_full = [&](int s, int b) { return bar0 + 8 * (8 + 2 * s + b); };
     auto pv_done = [&](int s) { return bar0 + 8 * (12 + s); };
     auto o_done = [&](int s) { return bar0 + 8 * (14 + s); };
-    auto kv_full = [&](int st) { return bar0 + 8 * (16 + st); };
-    auto kv_empty = [&](int st) { return bar0 + 8 * (16 + kStages + st); };
+    auto turn = [&](int s) { return bar0 + 8 * (16 + s); };
+    auto kv_full = [&](int st) { return bar0 + 8 * (18 + st); };
+    auto kv_empty = [&](int st) { return bar0 + 8 * (18 + kStages + st); };
     __shared__ uint32_t tmem_base_sh;
     __shared__ volatile int abort_flag;
 
@@ -323,6 +325,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             mbar_init(s_full(s, 0), 1); mbar_init(s_full(s, 1), 1);
             mbar_init(p_full(s, 0), 4); mbar_init(p_full(s, 1), 4);   // one arrival per softmax warp
             mbar_init(pv_done(s), 1); mbar_init(o_done(s), 1);
+            mbar_init(turn(s), 1);
         }
         for (int st = 0; st < kStages; ++st) {
             mbar_init(kv_full(st), GATHER ? 32 : 1);    // gather: every lane of the loader warp arrives
@@ -500,35 +503,26 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             // constant part is built once and the address (in 16-byte units) is added per MMA.
             const uint64_t desc_k = make_smem_desc_sw128(0, 16, 1024);             // K-major Q / K
             const uint64_t desc_v = make_smem_desc_sw128(0, kHalfBytes, 1024);     // MN-major V
-            const uint64_t desc_q = desc_k + ((sQ + slot * kQBytes) >> 4);
+            const uint32_t hi = (uint32_t)(desc_k >> 32);                          // the same for both
+            const uint32_t lo_q = (uint32_t)desc_k + ((sQ + slot * kQBytes) >> 4);
+            const uint32_t lo_k = (uint32_t)desc_k + (sKV >> 4), lo_v = (uint32_t)desc_v + (sKV >> 4);
             const uint32_t tSslot = tm + slot * 128;
             const uint32_t tOslot = tm + 256 + slot * kD;
-            auto issue_qk = [&](int buf, int stage) {          // S[buf] = Q K^T, N = 64 keys
-                const uint64_t b = desc_k + ((sKV + stage * kTileBytes) >> 4);
-                if (leader) {
-                    if constexpr (GATHER) fence_proxy_async_smem();     // the tile came through the generic proxy
+            auto issue_qk = [&](int buf, int stage, bool pass) {     // S[buf] = Q K^T, N = 64 keys; `pass`: hand the turn on
+                if constexpr (GATHER) fence_proxy_async_smem();     // the tile came through the generic proxy
 #pragma unroll
-                    for (int kk = 0; kk < kD / 16; ++kk) {
-                        const uint32_t qoff = ((kk >> 2) * kQHalf + (kk & 3) * 32) >> 4;
-                        const uint32_t koff = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
-                        umma_ss(tSslot + buf * kBN, desc_q + qoff, b + koff, idesc_qk, kk > 0);
-                    }
-                    umma_commit(s_full(slot, buf));
-                    umma_commit(kv_empty(stage));
+                for (int c = 0; c < kD / 64; ++c) {
+                    if (c == kD / 64 - 1 && pass) elect_arrive(turn(slot ^ 1));
+                    umma_ss_x4(tSslot + buf * kBN, lo_q + c * (kQHalf >> 4),
+                               lo_k + stage * (kTileBytes >> 4) + c * (kHalfBytes >> 4), idesc_qk, hi, c > 0);
                 }
-                __syncwarp();
+                elect_commit(s_full(slot, buf));
+                elect_commit(kv_empty(stage));
             };
             auto issue_pv = [&](int buf, int stage, bool first) {   // O += P[buf] V, K = 64 keys
-                const uint64_t b = desc_v + ((sKV + stage * kTileBytes) >> 4);
-                if (leader) {
-                    if constexpr (GATHER) fence_proxy_async_smem();
-#pragma unroll
-                    for (int kk = 0; kk < kBN / 16; ++kk)
-                        umma_ts(tOslot, tSslot + buf * kBN + kk * 8, b + kk * (2048 >> 4), idesc_pv,
-                                !(first && kk == 0));
-                    umma_commit(kv_empty(stage));
-                }
-                __syncwarp();
+                if constexpr (GATHER) fence_proxy_async_smem();
+                umma_ts_x4(tOslot, tSslot + buf * kBN, lo_v + stage * (kTileBytes >> 4), idesc_pv, hi, !first);
+                elect_commit(kv_empty(stage));
             };
             bool ok = true;
             auto wait = [&](uint32_t bar, uint32_t ph, int code) {
@@ -545,9 +539,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             Seg g;
             Cursor cur{0u, 0u};                  // first ring entry of the next run
             uint32_t qcnt = 0, tc = 0;           // tc: tiles this slot has processed so far
+            uint32_t turns = 0;                  // turns this slot has taken
             while (ok && iter.next(p, g)) {
                 const int n = __shfl_sync(0xffffffffu, g.t1 - g.t0, 0);
-                if (slot >= __shfl_sync(0xffffffffu, g.n_slots, 0)) {
+                const bool two = __shfl_sync(0xffffffffu, g.n_slots, 0) == 2;
+                if (slot == 1 && !two) {
                     // nothing to compute for this slot, but every K/V stage is released by both issuers
                     for (int e = 0; e < 2 * n && ok; ++e) {
                         wait(kv_full(cur.st), cur.ph, 206);
@@ -565,26 +561,34 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     wait(kv_full(ck.st), ck.ph, 202);
                     if (!ok) break;
                     tc_fence_after_sync();
-                    issue_qk((tc + i) & 1, ck.st);
+                    issue_qk((tc + i) & 1, ck.st, false);
                     ck.step(2);
                 }
                 if (n == 1) ck.step(2);                              // keep ck two tiles ahead of cv
 #pragma unroll 1
                 for (int i = 0; i < n && ok; ++i) {
                     const int buf = (tc + i) & 1;
+                    const bool more = i + 2 < n;
                     wait(kv_full(cv.st), cv.ph, 203);
+                    if (!ok) break;
+                    if (more) wait(kv_full(ck.st), ck.ph, 204);
                     if (!ok) break;
                     wait(p_full(slot, buf), ((tc + i) >> 1) & 1u, 205);
                     if (!ok) break;
+                    // The slots take turns at the tensor core, a tile's P V and the next Q K^T at a time: left
+                    // alone they fall into step, their MMAs interleave one by one and then both wait (some CTAs
+                    // 690k clocks, most 800k; with turns 727k on all).  The turn is handed on before the
+                    // last block of Q K^T so that the other slot's MMAs queue up behind it without a gap.
+                    if (two) {
+                        wait(turn(slot), (turns & 1u) ^ (slot == 0 ? 1u : 0u), 207);
+                        if (!ok) break;
+                        ++turns;
+                    }
                     tc_fence_after_sync();
                     issue_pv(buf, cv.st, i == 0);
-                    if (i + 2 < n) {                                // S(i+2) reuses the buffer P(i) was read from
-                        wait(kv_full(ck.st), ck.ph, 204);
-                        if (!ok) break;
-                        issue_qk(buf, ck.st);
-                    } else if (i + 2 == n) {
-                        if (leader) umma_commit(pv_done(slot));     // lets the last tile's softmax know O is at rest
-                    }
+                    if (more) issue_qk(buf, ck.st, two);            // S(i+2) reuses the buffer P(i) was read from
+                    else if (two) elect_arrive(turn(slot ^ 1));
+                    if (i + 2 == n && leader) umma_commit(pv_done(slot));     // lets the last tile's softmax know O is at rest
                     if (i == n - 1 && leader) { umma_commit(o_done(slot)); umma_commit(q_empty(slot)); }
                     __syncwarp();
                     cv.step(2);

@@ -184,6 +184,49 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// Series of MMAs over one 64-wide block of the reduction, executed by a whole warp in uniform control
+// flow: the elected lane issues them as predicated instructions (the same lane every time, so its
+// commits cover them).  Only the low word of a descriptor (start address and leading offset, in
+// 16-byte units) differs between MMAs; the high word is a constant, and so are the steps along K.
+#define PAFU_MMA_SS(n, acc)                                                                          \
+    "add.u32 al, %1, " n "; add.u32 bl, %2, " n "; mov.b64 a, {al, %4}; mov.b64 b, {bl, %4};\n\t"      \
+    "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, " acc ";\n\t"
+// D = A B^T, both K-major in shared memory: four K = 16 slices of one swizzled block; `accumulate`
+// applies to the first slice.
+__device__ __forceinline__ void umma_ss_x4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                           uint32_t desc_hi, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred e, t, f;\n\t.reg .b32 al, bl;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 f, %5, 0;\n\tsetp.eq.u32 t, 0, 0;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        PAFU_MMA_SS("0", "f") PAFU_MMA_SS("2", "t") PAFU_MMA_SS("4", "t") PAFU_MMA_SS("6", "t") "}\n"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(desc_hi), "r"(accumulate) : "memory");
+}
+#define PAFU_MMA_TS(na, nb, acc)                                                                     \
+    "add.u32 al, %1, " na "; add.u32 bl, %2, " nb "; mov.b64 b, {bl, %4};\n\t"                        \
+    "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [al], b, %3, " acc ";\n\t"
+// D (+)= A B over 64 rows of K: A bf16 in tensor memory (8 columns per slice), B MN-major in shared
+// memory (2048 bytes per slice).
+__device__ __forceinline__ void umma_ts_x4(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
+                                           uint32_t desc_hi, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred e, t, f;\n\t.reg .b32 al, bl;\n\t.reg .b64 b;\n\t"
+        "setp.ne.b32 f, %5, 0;\n\tsetp.eq.u32 t, 0, 0;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        PAFU_MMA_TS("0", "0", "f") PAFU_MMA_TS("8", "128", "t") PAFU_MMA_TS("16", "256", "t") PAFU_MMA_TS("24", "384", "t") "}\n"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(desc_hi), "r"(accumulate) : "memory");
+}
+// Warp-wide forms: the elected lane commits / arrives.
+__device__ __forceinline__ void elect_commit(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void elect_arrive(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}\n" ::"r"(bar) : "memory");
+}
 // Arrive on `bar` once every tcgen05 operation this thread issued so far has completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
