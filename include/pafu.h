@@ -385,8 +385,8 @@ pafu_status pafu_cache_update(pafu_cache* cache, const pafu_head* head,
  * L < 2 * block_len).  P is never written: the kernel needs only each row's log-sum-exp.
  *   Q, K      device bf16 [L, n_heads, d_head]
  *   LSE       device fp32 [n_heads, L]: log-sum-exp of scale * q_i . k_j over all L keys, as
- *             pafu_chunk_attn writes it for the same Q, K and scale; NULL = computed here with the
- *             attention kernel (costs a full attention pass and scratch for its output)
+ *             pafu_chunk_attn writes it for the same Q, K and scale; NULL = computed here (the same
+ *             bits; a pass over all logits without the P V half of the attention)
  *   s         device fp32 [L], out
  *   comp      device fp32 [3, L], out: low, diag, up; or NULL
  *   gmax      device fp32 [L], out, or NULL: mean over heads of max_i P[n,i,j] over ALL queries -

@@ -5,6 +5,7 @@
 #include "common.cuh"
 #include "attn_mma.cuh"
 #include "attn_tc.cuh"
+#include "attn_stats.cuh"
 
 namespace pafu {
 
@@ -34,6 +35,14 @@ pafu_status launch_attn_indexed(const uint16_t* Q, const uint16_t* K, const uint
     return attn_tc::launch(Q, K, V, Kq, Vq, st, n_heads, scale, O, LSE,
                            reinterpret_cast<int*>(base) + kStatusWordTimeout,
                            reinterpret_cast<float*>(base + kWsHeaderBytes), stream, 0, idx);
+}
+
+// Log-sum-exps only, of a d_head 128 attention whose keys are one segment per stream (bit-identical to launch_attn's).
+pafu_status launch_attn_stats(const uint16_t* Q, const uint16_t* K, const StreamTable& st, int32_t n_heads, float scale,
+                              float* LSE, void* ws, cudaStream_t stream) {
+    uint8_t* base = static_cast<uint8_t*>(ws);
+    return attn_tc::launch_stats(Q, K, st, n_heads, scale, LSE, reinterpret_cast<int*>(base) + kStatusWordTimeout,
+                                 reinterpret_cast<float*>(base + kWsHeaderBytes), stream);
 }
 
 bool attn_indexed_supported(const StreamTable& st, int32_t d_head, bool has_chunk) {

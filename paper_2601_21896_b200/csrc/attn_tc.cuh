@@ -270,6 +270,41 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return r;
 }
 
+// The pieces of a tile's softmax that attn_stats_kernel shares, so that both form the same bits.
+// Row sum of 2^(s * scale log2 e + mb) over 64 logits; `pk` (32 words), if given, receives the
+// probabilities as bf16 pairs.
+__device__ __forceinline__ float tile_sum(const uint32_t (&sr)[64], uint64_t sl2_2, float mb, uint32_t* pk = nullptr) {
+    const uint64_t mb_2 = pack2(__float_as_uint(mb), __float_as_uint(mb));
+    uint64_t rs2[2] = {0ull, 0ull};
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        float e0, e1;
+        unpack2(ffma2(pack2(sr[2 * c], sr[2 * c + 1]), sl2_2, mb_2), e0, e1);
+        const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
+        rs2[c & 1] = fadd2(rs2[c & 1], pack2(__float_as_uint(p0), __float_as_uint(p1)));
+        if (pk != nullptr) pk[c] = pack_bf16(p0, p1);
+    }
+    float r0, r1, r2, r3;
+    unpack2(rs2[0], r0, r1);
+    unpack2(rs2[1], r2, r3);
+    return (r0 + r1) + (r2 + r3);
+}
+__device__ __forceinline__ float tile_max(const uint32_t (&sr)[64]) {
+    float mx4[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float m = fmaxf(__uint_as_float(sr[16 * q]), __uint_as_float(sr[16 * q + 1]));
+#pragma unroll
+        for (int c = 2; c < 16; c += 2)
+            m = fmax3(m, __uint_as_float(sr[16 * q + c]), __uint_as_float(sr[16 * q + c + 1]));
+        mx4[q] = m;
+    }
+    return fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+}
+__device__ __forceinline__ float final_lse(float m, float scale, float l) {
+    return l > 0.f ? __fadd_rn(__fmul_rn(m, scale), logf(l)) : -INFINITY;
+}
+
 // GATHER = false: the retained keys/values are the rows of a compacted cache (mKc, mVc are tiled
 // maps of it).  GATHER = true: they are rows idx[.] of the uncompacted cache, fetched by the
 // loader warp with 16-byte asynchronous copies (mKc, mVc unused); everything downstream of the
@@ -671,16 +706,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 }
                 if (full_pass) {
                     if ((tid & 31) == 0) atomicAdd(p.status + ((i == 0 || left < kBN) ? kStatusWordFullFirst : kStatusWordFullSum), 1);
-                    float mx4[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float m = fmaxf(__uint_as_float(sr[16 * q]), __uint_as_float(sr[16 * q + 1]));
-#pragma unroll
-                        for (int c = 2; c < 16; c += 2)
-                            m = fmax3(m, __uint_as_float(sr[16 * q + c]), __uint_as_float(sr[16 * q + c + 1]));
-                        mx4[q] = m;
-                    }
-                    const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+                    const float mx = tile_max(sr);
                     if (i == 0) {
                         m_used = mx;
                     } else if (__any_sync(0xffffffffu, (mx - m_used) * sl2 > kRescaleThresholdLog2)) {
@@ -695,7 +721,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                         if ((tid & 31) == 0) atomicAdd(p.status + kStatusWordRescale, 1);
                         const float m_new = fmaxf(m_used, mx);
                         const float alpha = fast_exp2((m_used - m_new) * sl2);
-                        l_sum *= alpha;
+                        l_sum = __fmul_rn(l_sum, alpha);
                         m_used = m_new;
 #pragma unroll
                         for (int c = 0; c < kD / 32; ++c) {
@@ -707,23 +733,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                             PAFU_TMEM_ST_X32(tO + c * 32, orr);
                         }
                     }
-                    const float mb = -m_used * sl2;
-                    const uint64_t mb_2 = pack2(__float_as_uint(mb), __float_as_uint(mb));
-                    uint64_t rs2[2] = {0ull, 0ull};
                     uint32_t pk[32];
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        float e0, e1;
-                        unpack2(ffma2(pack2(sr[2 * c], sr[2 * c + 1]), sl2_2, mb_2), e0, e1);
-                        const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
-                        rs2[c & 1] = fadd2(rs2[c & 1], pack2(__float_as_uint(p0), __float_as_uint(p1)));
-                        pk[c] = pack_bf16(p0, p1);
-                    }
+                    l_sum += tile_sum(sr, sl2_2, -m_used * sl2, pk);
                     PAFU_TMEM_ST_X32(tS, pk);
-                    float r0, r1, r2, r3;
-                    unpack2(rs2[0], r0, r1);
-                    unpack2(rs2[1], r2, r3);
-                    l_sum += (r0 + r1) + (r2 + r3);
                 }   // full_pass
                 if (i + 1 < n && __all_sync(0xffffffffu, mbar_test_wait(s_full(slot, buf ^ 1), ((tc + i + 1) >> 1) & 1u))) {
                     // S(i+1) is already complete: request it now, so that its trip from tensor
@@ -771,7 +783,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 }
                 if (p.LSE != nullptr && row < g.Lq)
                     p.LSE[(int64_t)g.head * p.total_Lq + p.st.cu_Lq[g.stream] + row] =
-                        (l_sum > 0.f) ? m_used * p.scale + logf(l_sum) : -INFINITY;
+                        final_lse(m_used, p.scale, l_sum);
             } else {
                 // part of an item: unnormalised fp32 partial for the merge kernel
                 float* piece = p.pieces + ((size_t)blockIdx.x * 2 + g.piece) * kPieceFloats;
@@ -818,7 +830,8 @@ struct MergeTable {
     int16_t cta[2 * kMaxGrid];
 };
 
-template <int D>
+// OUT = false: only the log-sum-exps are merged (attn_stats_kernel's pieces hold nothing else).
+template <int D, bool OUT>
 __global__ void __launch_bounds__(kMergeThreads)
 attn_tc_merge_kernel(const __grid_constant__ MergeTable tb, const float* __restrict__ pieces, float scale,
                      int n_heads, int64_t total_Lq, uint16_t* __restrict__ O, float* __restrict__ LSE) {
@@ -851,12 +864,12 @@ attn_tc_merge_kernel(const __grid_constant__ MergeTable tb, const float* __restr
             const int r = slot * kBM + r0 + q;
             w[q] = piece[2 * kBM * kD + r];
             l[q] = piece[2 * kBM * kD + 2 * kBM + r];
-            v[q] = lane < kD / 4 ? reinterpret_cast<const float4*>(piece + (size_t)r * kD)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[q] = OUT && lane < kD / 4 ? reinterpret_cast<const float4*>(piece + (size_t)r * kD)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int q = 0; q < kMergeRows; ++q) {
             const float ww = fast_exp2((w[q] - M[q]) * sl2);
-            L[q] += ww * l[q];
+            L[q] = __fmaf_rn(ww, l[q], L[q]);
             acc[q].x += ww * v[q].x; acc[q].y += ww * v[q].y; acc[q].z += ww * v[q].z; acc[q].w += ww * v[q].w;
         }
     }
@@ -869,9 +882,9 @@ attn_tc_merge_kernel(const __grid_constant__ MergeTable tb, const float* __restr
         uint2 o;
         o.x = pack_bf16(acc[q].x * inv, acc[q].y * inv);
         o.y = pack_bf16(acc[q].z * inv, acc[q].w * inv);
-        if (lane < kD / 4) *reinterpret_cast<uint2*>(dst) = o;
+        if (OUT && lane < kD / 4) *reinterpret_cast<uint2*>(dst) = o;
         if (LSE != nullptr && lane == 0)
-            LSE[(int64_t)it.head * total_Lq + it.o_row + row] = (L[q] > 0.f) ? M[q] * scale + logf(L[q]) : -INFINITY;
+            LSE[(int64_t)it.head * total_Lq + it.o_row + row] = final_lse(M[q], scale, L[q]);
     }
 }
 
@@ -911,6 +924,16 @@ inline int sm_count() { return device_sm_count(); }
 inline int grid_for(int64_t cost) {
     const int sms = sm_count();
     return (int)(cost < sms ? cost : sms);
+}
+
+template <int D, bool OUT>
+inline pafu_status launch_merge(const Params& p, int grid, int32_t n_heads, cudaStream_t stream) {
+    if (grid <= 1) return PAFU_OK;
+    MergeTable tb;
+    build_merge_table(p, grid, tb);
+    if (tb.n_items == 0) return PAFU_OK;
+    return cuda_ok(launch_dependent(attn_tc_merge_kernel<D, OUT>, dim3(tb.n_items * kMergeBlocksPerItem), dim3(kMergeThreads), 0, stream, 1,
+                                    tb, (const float*)p.pieces, p.scale, (int)n_heads, p.total_Lq, p.O, p.LSE));
 }
 
 // True when every stream with queries has at least one key (the cost line has no entry for a
@@ -975,15 +998,7 @@ inline pafu_status launch_d(const uint16_t* Q, const uint16_t* Kc, const uint16_
         le = launch_dependent(attn_tc_kernel<false, D>, dim3(grid), dim3(kThreads), kSmem, stream, 1, mQ, mKc, mVc, mKq, mVq, p);
     }
     if (le != cudaSuccess) return PAFU_ERR_CUDA;
-    if (grid > 1) {
-        MergeTable tb;
-        build_merge_table(p, grid, tb);
-        if (tb.n_items > 0 &&
-            launch_dependent(attn_tc_merge_kernel<D>, dim3(tb.n_items * kMergeBlocksPerItem), dim3(kMergeThreads), 0, stream, 1,
-                             tb, (const float*)pieces, scale, (int)n_heads, nQ, O, LSE) != cudaSuccess)
-            return PAFU_ERR_CUDA;
-    }
-    return PAFU_OK;
+    return launch_merge<D, true>(p, grid, n_heads, stream);
 }
 
 inline pafu_status launch(const uint16_t* Q, const uint16_t* Kc, const uint16_t* Vc,

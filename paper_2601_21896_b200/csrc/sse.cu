@@ -11,10 +11,10 @@ using namespace pafu;
 
 inline size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
-// Workspace: [status header][attention scratch][LSE N x L][O L x N x D bf16][queries' extra features][maxima].
-// The attention scratch, LSE and O parts are only used when the caller passes no LSE.
+// Workspace: [status header][attention scratch][LSE N x L][queries' extra features][maxima].
+// The attention scratch and the LSE are only used when the caller passes no LSE.
 struct SsePlan {
-    size_t attn, lse, o, neglse, maxima, total;
+    size_t attn, lse, neglse, maxima, total;
 };
 SsePlan plan(int64_t L, int32_t n_heads, int32_t d_head, int64_t LB) {
     const sse_tc::Params p = sse_tc::make_params(L, LB, n_heads, 1.0f);
@@ -25,7 +25,6 @@ SsePlan plan(int64_t L, int32_t n_heads, int32_t d_head, int64_t LB) {
     size_t off = kWsHeaderBytes;
     pl.attn = off; off = up256(off + attn_workspace_bytes(st, n_heads, d_head));
     pl.lse = off; off = up256(off + (size_t)n_heads * L * 4);
-    pl.o = off; off = up256(off + (size_t)L * n_heads * d_head * 2);
     pl.neglse = off; off = up256(off + sse_tc::aug_bytes(p));
     pl.maxima = off; off = up256(off + sse_tc::maxima_bytes(p));
     pl.total = off;
@@ -57,16 +56,13 @@ extern "C" pafu_status pafu_sse(const uint16_t* Q, const uint16_t* K, const floa
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     const float* lse = LSE;
     if (lse == nullptr) {
-        // row statistics from the attention kernel: keys = the whole sequence, values = the keys
-        // (the output is discarded; only the log-sum-exp is kept)
+        // row statistics: the attention over the whole sequence without its output
         StreamTable st;
         memset(&st, 0, sizeof st);
         st.n_streams = 1;
         st.cu_B[1] = L; st.cu_Lq[1] = L;
         float* lse_out = reinterpret_cast<float*>(base + pl.lse);
-        pafu_status e = launch_attn(Q, K, K, nullptr, nullptr, st, n_heads, d_head, scale,
-                                    reinterpret_cast<uint16_t*>(base + pl.o), lse_out, base,
-                                    pl.attn + attn_workspace_bytes(st, n_heads, d_head), cs);
+        pafu_status e = launch_attn_stats(Q, K, st, n_heads, scale, lse_out, base, cs);
         if (e != PAFU_OK) return e;
         lse = lse_out;
     }
@@ -99,9 +95,7 @@ extern "C" pafu_status pafu_sse_mean_first(const uint16_t* Q, const uint16_t* K,
         st.n_streams = 1;
         st.cu_B[1] = L; st.cu_Lq[1] = L;
         float* lse_out = reinterpret_cast<float*>(base + pl.lse);
-        pafu_status e = launch_attn(Q, K, K, nullptr, nullptr, st, n_heads, d_head, scale,
-                                    reinterpret_cast<uint16_t*>(base + pl.o), lse_out, base,
-                                    pl.attn + attn_workspace_bytes(st, n_heads, d_head), cs);
+        pafu_status e = launch_attn_stats(Q, K, st, n_heads, scale, lse_out, base, cs);
         if (e != PAFU_OK) return e;
         lse = lse_out;
     }

@@ -591,6 +591,27 @@ def test_sse_matches_oracle(L, N, LB):
     assert torch.equal(s, s2)
 
 
+@pytest.mark.parametrize("rise", [0.0, 4.0, -4.0, 20.0])
+@pytest.mark.parametrize("L", [1, 64, 65, 128, 129, 256, 257, 640, 1100])
+def test_sse_row_statistics(L, rise):
+    """The pass that computes the row log-sum-exps (LSE = NULL): sequence lengths around its 128-token tiles,
+    pairs of query tiles and two S buffers, and logits that rise or fall by `rise` nats per 64 keys, so that the
+    running maximum starts far too small, is re-based in every tile, or never."""
+    N, D, LB = 2, 128, max(1, L // 3)
+    rng = np.random.default_rng(L)
+    Q = rng.standard_normal((L, N, D), dtype=np.float32) + 1.0
+    K = rng.standard_normal((L, N, D), dtype=np.float32) + (rise / np.sqrt(D) * np.arange(L, dtype=np.float32) / 64)[:, None, None]
+    Q, K = wl.f32_to_bf16_bits(Q), wl.f32_to_bf16_bits(K.astype(np.float32))
+    want, _ = oracle.sse(Q, K, LB)
+    s = torch.empty(L, dtype=torch.float32, device="cuda")
+    ws = torch.zeros(pafu.pafu_sse_workspace_bytes(L, N, D, LB), dtype=torch.uint8, device="cuda")
+    pafu.pafu_sse(to_device_bf16(Q), to_device_bf16(K), None, LB, 0.0, s, None, ws)
+    assert pafu.pafu_workspace_status(ws) == 0
+    # s = exp(z - lse): 32-bit logits and sums of magnitude up to max|z| lose a few units of 2^-24 max|z|
+    zmax = 1.0 + np.abs(wl.bf16_bits_to_f32(Q).reshape(L, -1)).sum(1).max() * np.abs(wl.bf16_bits_to_f32(K)).max() / np.sqrt(D)
+    np.testing.assert_allclose(s.cpu().numpy(), want, rtol=8 * 2.0 ** -24 * zmax + 1e-6, atol=1e-30)
+
+
 @pytest.mark.parametrize("L,N,LB", [
     (700, 3, 200),      # four blocks, the last one half length; blocks and 64-token tiles do not line up
     (1024, 2, 256),     # blocks that are whole tiles
