@@ -650,8 +650,11 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
 
     // 1. the chunk does not fit: keep the sink prefix and the Top-k of SL, in every layer
+    const int from = c->cur;
+    int64_t keep = 0;
+    int select_ctas = 0;
     if (c->T + chunk > c->capacity) {
-        const int64_t keep = c->capacity - chunk;
+        keep = c->capacity - chunk;
         if (keep > 0) {
             StreamTable st;
             memset(&st, 0, sizeof st);
@@ -664,38 +667,23 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
             pol.n_sink = c->n_sink; pol.n_recent = 0; pol.budget = keep;
             e = fill_policy(&sh, &pol, &st);
             if (e != PAFU_OK) return e;
-            e = launch_select(c->SL[c->cur], st, c->idx, cs);
+            e = launch_select(c->SL[from], st, c->idx, cs, 1);
             if (e != PAFU_OK) return e;
-            const int o = c->cur ^ 1;
-            e = launch_compact_layers(c->K[c->cur], c->V[c->cur], c->n_layers, c->SL[c->cur], c->idx, st, (int32_t)dm,
-                                      c->K[o], c->V[o], c->SL[o], cs);
-            if (e != PAFU_OK) return e;
+            select_ctas = select_cta_count(st);
         }
         c->cur ^= 1;
         c->T = keep;
         if (pruned != nullptr) *pruned = 1;
     }
-    // 2. the chunk's salience scores go straight to the tail of SL
-    const uint16_t* parts[3] = {Qs, Ks, Vs};
-    e = launch_score(*head, parts, 3, chunk, dm, c->SL[c->cur] + c->T, ws, ws_bytes, cs);
+    // 2. every layer's new rows go to the tail of its K and V, the kept ones to the front of the other set
+    const int to = c->cur;
+    e = launch_cache_rows(Knew, Vnew, chunk, c->K[from], c->V[from], c->SL[from], c->idx, keep, c->T, c->K[to], c->V[to],
+                          c->SL[to], c->n_layers, (int32_t)dm, select_ctas, cs);
     if (e != PAFU_OK) return e;
-    // 3. every layer's new rows go to the tail of its K and V
-    {
-        StreamTable st;
-        memset(&st, 0, sizeof st);
-        st.n_streams = 1;
-        st.cu_T[1] = chunk;
-        st.cu_B[1] = chunk;
-        const uint16_t* kd[PAFU_MAX_LAYERS]; const uint16_t* vd[PAFU_MAX_LAYERS];
-        uint16_t* ko[PAFU_MAX_LAYERS]; uint16_t* vo[PAFU_MAX_LAYERS];
-        for (int l = 0; l < c->n_layers; ++l) {
-            kd[l] = Knew[l]; vd[l] = Vnew[l];
-            ko[l] = c->K[c->cur][l] + c->T * dm;
-            vo[l] = c->V[c->cur][l] + c->T * dm;
-        }
-        e = launch_compact_layers(kd, vd, c->n_layers, nullptr, nullptr, st, (int32_t)dm, ko, vo, nullptr, cs);
-        if (e != PAFU_OK) return e;
-    }
+    // 3. the chunk's salience scores go straight to the tail of SL, computed beside the copies
+    const uint16_t* parts[3] = {Qs, Ks, Vs};
+    e = launch_score(*head, parts, 3, chunk, dm, c->SL[to] + c->T, ws, ws_bytes, cs, 1);
+    if (e != PAFU_OK) return e;
     c->T += chunk;
     return PAFU_OK;
 }

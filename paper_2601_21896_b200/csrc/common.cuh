@@ -74,8 +74,8 @@ inline bool once_per_device(bool (&done)[kMaxDevices], Set set) {
 // may be scheduled, and run their local set-up, as soon as the preceding kernel's CTAs have
 // left the SMs, without waiting for that kernel's completion to be processed first.  In return
 // each kernel executes grid_dep_wait() before its first access to global memory; that wait
-// returns only when the preceding kernel has completed and its writes are visible.  No kernel
-// signals its dependents early: CTAs of a following kernel that sat on the SMs while a
+// returns only when the preceding kernel has completed and its writes are visible.  Only the
+// selection and the rolling cache's row copies let their dependents start early (see there): CTAs of a following kernel that sat on the SMs while a
 // bandwidth-bound kernel was still in its last wave cost more than the earlier start gained.
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -107,10 +107,14 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 }
 
 // Launchers (each enqueues on `stream` and returns the launch status).
+// beside_predecessor = 1: the kernel runs beside the one launched before it, which must be
+// launch_cache_rows (that kernel lets it start only once everything before it is complete), and ends after it.
 pafu_status launch_score(const pafu_head& head, const uint16_t* const* X, int n_parts, int64_t n_tokens, int64_t ldx,
-                         float* scores, void* ws, size_t ws_bytes, cudaStream_t stream);
+                         float* scores, void* ws, size_t ws_bytes, cudaStream_t stream, int beside_predecessor = 0);
+// trigger_late = 1: the kernel behind it may start early, but not before everything ahead of the
+// selection is complete
 pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx,
-                          cudaStream_t stream);
+                          cudaStream_t stream, int trigger_late = 0);
 int select_cta_count(const StreamTable& st);      // CTAs launch_select's kernels occupy for this geometry
 // work != nullptr (three zeroed words of the workspace header): the rows that are kept whatever
 // the scores say are copied before the kernel waits for its predecessor (only valid when that
@@ -122,6 +126,14 @@ pafu_status launch_compact(const uint16_t* K, const uint16_t* V, const float* SL
 pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* const* V, int32_t n_layers,
                                   const float* SL, const int32_t* idx, const StreamTable& st, int32_t d_model,
                                   uint16_t* const* Kc, uint16_t* const* Vc, float* SLc, cudaStream_t stream);
+// The row copies of a rolling-cache update, all layers in one launch: n_new rows of Knew/Vnew to row `dst0` on of
+// Kd/Vd, and rows idx[0 .. keep) of Ks/Vs (and SL) to the front of Kd/Vd (and SLd).
+// select_ctas > 0: launched directly behind launch_select(.., trigger_late = 1), which occupies that many
+// CTAs; 0: after what is ahead (keep must be 0).
+pafu_status launch_cache_rows(const uint16_t* const* Knew, const uint16_t* const* Vnew, int64_t n_new,
+                              const uint16_t* const* Ks, const uint16_t* const* Vs, const float* SL, const int32_t* idx,
+                              int64_t keep, int64_t dst0, uint16_t* const* Kd, uint16_t* const* Vd, float* SLd, int32_t n_layers,
+                              int32_t d_model, int select_ctas, cudaStream_t stream);
 pafu_status launch_attn(const uint16_t* Q, const uint16_t* Kc, const uint16_t* Vc,
                         const uint16_t* Kq, const uint16_t* Vq, const StreamTable& st,
                         int32_t n_heads, int32_t d_head, float scale, uint16_t* O, float* LSE,

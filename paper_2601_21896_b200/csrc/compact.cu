@@ -179,27 +179,20 @@ compact_layers_kernel(const __grid_constant__ LayerPtrs lp, int32_t n_layers,
         const int64_t r = w - (int64_t)layer * n_rows;
         int s = 0;
         while (s + 1 < st.n_streams && r >= st.cu_B[s + 1]) ++s;
-        // idx == nullptr: the rows in order (a plain copy of every layer's rows)
-        const int64_t src_row = st.cu_T[s] + (idx != nullptr ? (int64_t)__ldg(idx + r) : r - st.cu_B[s]);
-        const uint4* ks = lp.K[layer] + src_row * chunks_per_row;
-        const uint4* vs = lp.V[layer] + src_row * chunks_per_row;
-        uint4* kd = lp.Kc[layer] + r * chunks_per_row;
-        uint4* vd = lp.Vc[layer] + r * chunks_per_row;
-        for (int c0 = 0; c0 < chunks_per_row; c0 += 32 * kCompactUnroll) {
-            uint4 kb[kCompactUnroll], vb[kCompactUnroll];
-#pragma unroll
-            for (int u = 0; u < kCompactUnroll; ++u) {
-                const int c = c0 + u * 32 + lane;
-                if (c < chunks_per_row) { kb[u] = ld_nc_v4(ks + c); vb[u] = ld_nc_v4(vs + c); }
-            }
-#pragma unroll
-            for (int u = 0; u < kCompactUnroll; ++u) {
-                const int c = c0 + u * 32 + lane;
-                if (c < chunks_per_row) { kd[c] = kb[u]; vd[c] = vb[u]; }
-            }
-        }
-        if (layer == 0 && SLc != nullptr && lane == 0) SLc[r] = __ldg(SL + src_row);
+        const int64_t src_row = st.cu_T[s] + (int64_t)__ldg(idx + r);
+        copy_kv_row(lp.K[layer], lp.V[layer], SL, src_row, r, chunks_per_row, lp.Kc[layer], lp.Vc[layer],
+                    layer == 0 ? SLc : nullptr, lane);
     }
+}
+
+static LayerPtrs layer_ptrs(const uint16_t* const* K, const uint16_t* const* V, uint16_t* const* Kc, uint16_t* const* Vc, int32_t n_layers) {
+    LayerPtrs lp;
+    for (int l = 0; l < PAFU_MAX_LAYERS; ++l) {
+        const int i = l < n_layers ? l : 0;
+        lp.K[l] = reinterpret_cast<const uint4*>(K[i]); lp.V[l] = reinterpret_cast<const uint4*>(V[i]);
+        lp.Kc[l] = reinterpret_cast<uint4*>(Kc[i]); lp.Vc[l] = reinterpret_cast<uint4*>(Vc[i]);
+    }
+    return lp;
 }
 
 pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* const* V, int32_t n_layers,
@@ -207,17 +200,53 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
                                   uint16_t* const* Kc, uint16_t* const* Vc, float* SLc, cudaStream_t stream) {
     const int64_t n_rows = st.cu_B[st.n_streams];
     if (n_rows == 0 || n_layers == 0) return PAFU_OK;
-    LayerPtrs lp;
-    for (int l = 0; l < PAFU_MAX_LAYERS; ++l) {
-        const int i = l < n_layers ? l : 0;
-        lp.K[l] = reinterpret_cast<const uint4*>(K[i]); lp.V[l] = reinterpret_cast<const uint4*>(V[i]);
-        lp.Kc[l] = reinterpret_cast<uint4*>(Kc[i]); lp.Vc[l] = reinterpret_cast<uint4*>(Vc[i]);
-    }
     int64_t blocks = (n_rows * n_layers + kCompactWarpsPerBlock - 1) / kCompactWarpsPerBlock;
     const int64_t max_blocks = 148 * 8 * 4;
     if (blocks > max_blocks) blocks = max_blocks;
     return cuda_ok(launch_dependent(compact_layers_kernel, dim3((unsigned)blocks), dim3(kCompactWarpsPerBlock * 32), 0, stream, 1,
-                                    lp, n_layers, SL, idx, st, d_model / 8, SLc, n_rows));
+                                    layer_ptrs(K, V, Kc, Vc, n_layers), n_layers, SL, idx, st, d_model / 8, SLc, n_rows));
+}
+
+// A rolling-cache update's copies: the chunk's new rows of every layer, then the kept rows through the
+// index list.  The new rows need nothing that the selection ahead produces, so they are copied while
+// it runs; and the kernel lets the one behind it start at once: that is the salience head of the chunk,
+// tensor-bound work on one CTA an SM, which this kernel leaves registers for (one block of 256 threads
+// an SM: 86 registers each beside the head's 384 x 95 to 100).  30 layers, 4680 kept and 4680 new rows: 607 us as
+// select, gather, head and append one after the other, 586 us like this; ten or twelve warps in 78 or
+// 64 registers 590 and 662; only the append here and the gather behind the head 647.  (Row counts
+// times layers stay far below 2^32: each is at least 32 bytes of three buffers.)
+__global__ void __launch_bounds__(kCompactWarpsPerBlock * 32)
+cache_rows_kernel(const __grid_constant__ LayerPtrs add, const __grid_constant__ LayerPtrs keep, int32_t n_layers,
+                  int32_t n_new, int64_t dst0, const float* __restrict__ SL, const int32_t* __restrict__ idx, int32_t n_keep,
+                  int32_t chunks_per_row, float* __restrict__ SLd, int behind_select) {
+    if (!behind_select) grid_dep_wait();
+    grid_dep_launch_dependents();     // everything ahead of the selection (or of this kernel) is complete here
+    const int lane = threadIdx.x & 31;
+    const uint32_t warp0 = blockIdx.x * kCompactWarpsPerBlock + (threadIdx.x >> 5);
+    const uint32_t n_warps = gridDim.x * kCompactWarpsPerBlock;
+    for (uint32_t w = warp0; w < (uint32_t)n_new * n_layers; w += n_warps) {
+        const uint32_t layer = w / n_new, r = w - layer * n_new;
+        copy_kv_row(add.K[layer], add.V[layer], nullptr, r, dst0 + r, chunks_per_row, add.Kc[layer], add.Vc[layer], nullptr, lane);
+    }
+    if (behind_select) grid_dep_wait();
+    for (uint32_t w = warp0; w < (uint32_t)n_keep * n_layers; w += n_warps) {
+        const uint32_t layer = w / n_keep, r = w - layer * n_keep;
+        copy_kv_row(keep.K[layer], keep.V[layer], SL, (int64_t)__ldg(idx + r), r, chunks_per_row, keep.Kc[layer], keep.Vc[layer],
+                    layer == 0 ? SLd : nullptr, lane);
+    }
+}
+
+pafu_status launch_cache_rows(const uint16_t* const* Knew, const uint16_t* const* Vnew, int64_t n_new,
+                              const uint16_t* const* Ks, const uint16_t* const* Vs, const float* SL, const int32_t* idx,
+                              int64_t keep, int64_t dst0, uint16_t* const* Kd, uint16_t* const* Vd, float* SLd, int32_t n_layers,
+                              int32_t d_model, int select_ctas, cudaStream_t stream) {
+    int64_t blocks = ((n_new + keep) * n_layers + kCompactWarpsPerBlock - 1) / kCompactWarpsPerBlock;
+    // one block an SM, in fixed shares; the selection's SMs are left out
+    const int64_t most = device_sm_count() > select_ctas ? device_sm_count() - select_ctas : 1;
+    if (blocks > most) blocks = most;
+    return cuda_ok(launch_dependent(cache_rows_kernel, dim3((unsigned)blocks), dim3(kCompactWarpsPerBlock * 32), 0, stream, 1,
+                                    layer_ptrs(Knew, Vnew, Kd, Vd, n_layers), layer_ptrs(Ks, Vs, Kd, Vd, n_layers), n_layers,
+                                    (int32_t)n_new, dst0, SL, idx, (int32_t)keep, d_model / 8, SLd, select_ctas > 0 ? 1 : 0));
 }
 
 // `work`: three zeroed 32-bit words of device memory (the step's workspace header) - then the

@@ -46,6 +46,7 @@ struct Params {
     int64_t n_tokens;
     int d_in, d_hidden, d_out, act, final;
     int k_per_part;      // reduction slices (of kBK features) taken from each input matrix
+    int beside;          // 1: run beside the preceding kernel (see launch_score), finish after it
     int split;           // 1: one (tile, chunk) per CTA, clusters of n_chunks CTAs
     int tail_tiles;      // > 0: the last tail_tiles tiles are each split between the two CTAs of a cluster,
     int tail_width;      //      tail_width hidden units per CTA (d_hidden / 2)
@@ -141,7 +142,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap mX, const __grid_constant__ 
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_sh;
-    grid_dep_wait();          // set-up above is local; everything below reads or writes global memory
+    if (!p.beside) grid_dep_wait();   // set-up above is local; everything below reads or writes global memory
     // Folded second layer and first-layer bias, fp32 in shared memory: the read-out warps' business
     // (they meet at a barrier of their own below), so the loader and the first MMAs do not wait
     // for these global reads.
@@ -310,12 +311,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap mX, const __grid_constant__ 
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, 512);
+    if (p.beside) grid_dep_wait();    // what waits for this kernel relies on the one before it as well
 }
 
 // X[0..n_parts) are the matrices whose rows, side by side, form a token's d_in features
 // (n_parts = 1: a plain [n_tokens, d_in] matrix; 3: query, key and value rows of d_in / 3 each).
 inline pafu_status launch(const pafu_head& head, const uint16_t* const* X, int n_parts, int64_t n_tokens, int64_t ldx,
-                          float* scores, int* status, int sm_count, cudaStream_t stream) {
+                          float* scores, int* status, int sm_count, cudaStream_t stream, int beside) {
     CUtensorMap mX[3], mW;
     const int d_part = head.d_in / n_parts;
     for (int i = 0; i < 3; ++i)
@@ -326,7 +328,7 @@ inline pafu_status launch(const pafu_head& head, const uint16_t* const* X, int n
     Params p;
     p.n_tokens = n_tokens; p.d_in = head.d_in; p.d_hidden = head.d_hidden; p.d_out = head.d_out;
     p.act = head.act; p.final = head.final; p.w2 = head.w2; p.b1 = head.b1; p.b2 = head.b2;
-    p.scores = scores; p.status = status;
+    p.scores = scores; p.status = status; p.beside = beside;
     p.k_per_part = d_part / kBK;
     const int64_t n_tiles = (n_tokens + kBM - 1) / kBM;
     const int n_chunks = (head.d_hidden + kNMax - 1) / kNMax;

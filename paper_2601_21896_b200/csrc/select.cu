@@ -132,11 +132,12 @@ __device__ __forceinline__ void radix_pass(cg::cluster_group& cluster, SelShared
 
 __global__ void __launch_bounds__(kSelThreads, 1)
 select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ StreamTable st, int32_t keys_bytes,
-                      int32_t* __restrict__ idx) {
+                      int32_t* __restrict__ idx, int trigger_late) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     __shared__ SelShared sh;
-    grid_dep_launch_dependents();
+    if (!trigger_late) grid_dep_launch_dependents();
     grid_dep_wait();
+    if (trigger_late) grid_dep_launch_dependents();
     cg::cluster_group cluster = cg::this_cluster();
     const int nc = (int)cluster.num_blocks();                // 1, 2, 4 or 8: the host's choice for this launch
     const int s = blockIdx.x / nc;
@@ -306,9 +307,10 @@ select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ 
 // Streams with more candidates than a cluster's shared memory holds: keys are re-read from L2 in every pass
 // (4 passes of 8 bits), and each thread emits a contiguous token range.
 __global__ void __launch_bounds__(kSelThreads)
-select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* __restrict__ idx) {
-    grid_dep_launch_dependents();
+select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* __restrict__ idx, int trigger_late) {
+    if (!trigger_late) grid_dep_launch_dependents();
     grid_dep_wait();
+    if (trigger_late) grid_dep_launch_dependents();
     {
         const int64_t T = st.cu_T[blockIdx.x + 1] - st.cu_T[blockIdx.x], B = st.cu_B[blockIdx.x + 1] - st.cu_B[blockIdx.x];
         if (B >= T || T - st.n_sink[blockIdx.x] - st.n_recent[blockIdx.x] <= kSelCapCluster) return;   // the other kernel owns this stream
@@ -450,7 +452,7 @@ int select_cta_count(const StreamTable& st) {
     return (pl.any_cluster ? st.n_streams * pl.nc : 0) + (pl.any_stream ? st.n_streams : 0);
 }
 
-pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx, cudaStream_t stream) {
+pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx, cudaStream_t stream, int trigger_late) {
     if (st.n_streams == 0 || st.cu_B[st.n_streams] == 0) return PAFU_OK;
     const SelLaunch pl = plan_select(st);
     if (pl.any_cluster) {
@@ -462,12 +464,12 @@ pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* i
         const int32_t keys_bytes = (int32_t)(pl.per_cta * 4);
         const size_t smem = (size_t)keys_bytes + kSelListCap * 4 + kSelHistBins * 4 * 2;
         if (launch_dependent(select_cluster_kernel, dim3((unsigned)(st.n_streams * pl.nc)), dim3(kSelThreads), smem, stream,
-                             (unsigned)pl.nc, scores, st, keys_bytes, idx) != cudaSuccess)
+                             (unsigned)pl.nc, scores, st, keys_bytes, idx, trigger_late) != cudaSuccess)
             return PAFU_ERR_CUDA;
     }
     if (pl.any_stream &&
         launch_dependent(select_stream_kernel, dim3((unsigned)st.n_streams), dim3(kSelThreads), 0, stream, 1, scores, st,
-                         idx) != cudaSuccess)
+                         idx, trigger_late) != cudaSuccess)
         return PAFU_ERR_CUDA;
     return PAFU_OK;
 }
