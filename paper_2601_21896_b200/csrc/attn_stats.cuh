@@ -216,8 +216,9 @@ inline pafu_status launch_stats(const uint16_t* Q, const uint16_t* K, const Stre
             return cudaFuncSetAttribute(attn_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStatsSmemBytes) == cudaSuccess;
         }))
         return PAFU_ERR_CUDA;
-    const int grid = grid_for(cost);
-    plan_shares(p, grid, cost);
+    bool whole;
+    const int grid = grid_for(st, n_heads, 0, cost, 0, whole);
+    plan_shares(p, grid, cost, whole);
     if (launch_dependent(attn_stats_kernel, dim3(grid), dim3(kThreads), kStatsSmemBytes, stream, 1, mQ, mK, p) != cudaSuccess)
         return PAFU_ERR_CUDA;
     return launch_merge<kD, false>(p, grid, n_heads, stream);

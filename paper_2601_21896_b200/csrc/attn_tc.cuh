@@ -66,7 +66,7 @@ constexpr int kRegsLaunch = 168, kRegsLow = 80, kRegsHigh = 208;
 static_assert((kRegsLaunch - kRegsLow) * 128 >= (kRegsHigh - kRegsLaunch) * 256,
               "setmaxnreg.inc would wait forever");
 constexpr int kMaxGrid = kMaxPersistentGrid;
-// one partial: O [256][128] fp32, then m [256], then l [256]
+// one partial: O [128][256] fp32 (column-major: a column's 256 rows together), then m [256], then l [256]
 constexpr int kPieceFloats = 2 * kBM * kD + 2 * 2 * kBM;
 constexpr size_t kPieceBytes = (size_t)kPieceFloats * 4;
 
@@ -202,7 +202,13 @@ struct SegIter {
 // the cost line, 148 different heads are read at once, far more than L2 holds: 40 heads x 4 streams
 // of the 14B-class layer 6.24 -> 5.09 ms a launch, 12 heads x 18 720 keys 559 -> 530 us.)  What is left
 // of the line is cut so that all CTAs end with the same total.
-inline void plan_shares(Params& p, int grid, int64_t total) {
+inline void plan_shares(Params& p, int grid, int64_t total, bool whole) {
+    if (whole) {                                     // one round of whole items and nothing left
+        p.n_waves = 1;
+        p.rest0 = total;
+        for (int b = 0; b <= grid; ++b) p.share[b] = 0;
+        return;
+    }
     const int64_t even = total / grid;
     int64_t done[kMaxGrid] = {}, next[kMaxGrid];
     p.n_waves = 0;
@@ -318,7 +324,7 @@ struct HeadDims {
     static constexpr int kHalfBytes = kBN * 64 * 2;              // one [64 rows x 64 cols] swizzled block of a K or V tile
     static constexpr int kTileBytes = kBN * D * 2;
     static constexpr int kSmemBytes = 2 * kQBytes + kStages * kTileBytes + 1024 /*align*/ + 512 /*barriers*/;
-    static constexpr int kPieceFloats = 2 * kBM * D + 2 * 2 * kBM;   // one partial: O [256][D], m [256], l [256]
+    static constexpr int kPieceFloats = 2 * kBM * D + 2 * 2 * kBM;   // one partial: O [D][256], m [256], l [256]
 };
 
 template <bool GATHER, int D>
@@ -788,16 +794,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 // part of an item: unnormalised fp32 partial for the merge kernel
                 float* piece = p.pieces + ((size_t)blockIdx.x * 2 + g.piece) * kPieceFloats;
                 const int prow = slot * kBM + row_in_slot;
-                float4* dst = reinterpret_cast<float4*>(piece + (size_t)prow * kD);
+                // column by column, so that a warp's 32 rows are 128 contiguous bytes (row by row the
+                // two partials of a CTA took 10 us to write)
+                float* dst = piece + prow;
 #pragma unroll
                 for (int c = 0; c < kD / 32; ++c) {
                     uint32_t orr[32];
                     PAFU_TMEM_LD_X32(tO + c * 32, orr);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        dst[c * 8 + q] = make_float4(__uint_as_float(orr[4 * q]), __uint_as_float(orr[4 * q + 1]),
-                                                     __uint_as_float(orr[4 * q + 2]), __uint_as_float(orr[4 * q + 3]));
+                    for (int q = 0; q < 32; ++q) dst[(c * 32 + q) * (2 * kBM)] = __uint_as_float(orr[q]);
                 }
                 piece[2 * kBM * kD + prow] = m_used;
                 piece[2 * kBM * kD + 2 * kBM + prow] = l_sum;
@@ -812,12 +818,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
 // Merges the partials of every item that was split across CTAs.  The host walks the CTAs'
 // shares once per launch and passes the work as a table: item i was begun by CTA cta[first]
 // (its last run, stored as that CTA's piece 1) and continued by the following entries (each
-// CTA's first run, piece 0), in key order, which keeps the result deterministic.  Eight blocks
-// of 256 threads per item (two slots x four groups of 32 rows); a warp handles four rows, so
-// all loads of a block are in flight together.
-constexpr int kMergeRows = 4;
+// CTA's first run, piece 0), in key order.  A warp takes eight rows and every `lanes`-th piece of
+// them; `lanes` (2, 4 or 8: the host's choice by the longest list) warps share the rows and
+// their sums are added in warp order, which keeps the result deterministic.  The pieces come from
+// L2, a trip of about a microsecond, so they are fetched side by side: with a warp walking all
+// pieces of its rows one after the other an item of 37 pieces took 67 us.
+constexpr int kMergeRows = 8;
 constexpr int kMergeThreads = 256;
-constexpr int kMergeBlocksPerItem = 2 * (kBM / (kMergeThreads / 32 * kMergeRows));   // 8
+constexpr int kMergeWarps = kMergeThreads / 32;
 struct MergeItem {
     int32_t o_row;        // row of O (and LSE column) of the item's first query
     int32_t rows;         // valid query rows of the item (<= 256)
@@ -826,6 +834,7 @@ struct MergeItem {
 };
 struct MergeTable {
     int32_t n_items;
+    int32_t lanes;             // warps that share a group of rows
     MergeItem item[kMaxGrid];
     int16_t cta[2 * kMaxGrid];
 };
@@ -837,61 +846,98 @@ attn_tc_merge_kernel(const __grid_constant__ MergeTable tb, const float* __restr
                      int n_heads, int64_t total_Lq, uint16_t* __restrict__ O, float* __restrict__ LSE) {
     constexpr int kD = D;
     constexpr int kPieceFloats = HeadDims<D>::kPieceFloats;
+    constexpr int kVec = kD / 4;                                       // float4 per row of the output
+    constexpr int kPitch = OUT ? kD + 4 : 4;                           // floats: 16-byte rows, four of them half the banks apart
+    __shared__ __align__(16) float part[kMergeWarps][kMergeRows][kPitch];
+    __shared__ float part_l[kMergeWarps][kMergeRows];
     grid_dep_wait();
-    const MergeItem& it = tb.item[blockIdx.x / kMergeBlocksPerItem];
-    const int slot = (blockIdx.x / (kMergeBlocksPerItem / 2)) & 1;
-    const int group = blockIdx.x % (kMergeBlocksPerItem / 2);
-    if (slot >= it.n_slots) return;                                    // block-uniform
+    const int lanes = tb.lanes, blocks_per_item = 4 * lanes;
+    const MergeItem& it = tb.item[blockIdx.x / blocks_per_item];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int group = warp / lanes, pl = warp % lanes;
+    const int rows_per_block = kMergeRows * kMergeWarps / lanes;
+    const int b0 = (blockIdx.x % blocks_per_item) * rows_per_block;    // rows of the item (slot * 128 + row of the slot)
+    if (b0 >= it.rows) return;                                         // block-uniform
+    const int r0 = b0 + group * kMergeRows;
     const int n_pieces = it.n_pieces;
     const float sl2 = scale * 1.4426950408889634f;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;        // 32 float4 per row
-    const int r0 = group * (kMergeThreads / 32 * kMergeRows) + warp * kMergeRows;
-    float M[kMergeRows], L[kMergeRows];
-    float4 acc[kMergeRows];
-#pragma unroll
-    for (int q = 0; q < kMergeRows; ++q) { M[q] = -INFINITY; L[q] = 0.f; acc[q] = make_float4(0.f, 0.f, 0.f, 0.f); }
-    for (int i = 0; i < n_pieces; ++i) {
-        const float* piece = pieces + ((size_t)tb.cta[it.first + i] * 2 + (i == 0 ? 1 : 0)) * kPieceFloats;
-#pragma unroll
-        for (int q = 0; q < kMergeRows; ++q) M[q] = fmaxf(M[q], piece[2 * kBM * kD + slot * kBM + r0 + q]);
+    const int rs = (lane & 1) * 4, d0 = lane >> 1;                     // this lane's four rows, and its columns d0 + 16 k
+    auto piece_at = [&](int i) { return pieces + ((size_t)tb.cta[it.first + i] * 2 + (i == 0 ? 1 : 0)) * kPieceFloats; };
+    auto f4 = [](const float* p) { return *reinterpret_cast<const float4*>(p); };
+    // the rows' maxima over all pieces (every warp for itself, a lane pair per piece)
+    float4 M = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    for (int i = d0; i < n_pieces; i += 16) {
+        const float4 m = f4(piece_at(i) + 2 * kBM * kD + r0 + rs);
+        M.x = fmaxf(M.x, m.x); M.y = fmaxf(M.y, m.y); M.z = fmaxf(M.z, m.z); M.w = fmaxf(M.w, m.w);
     }
-    for (int i = 0; i < n_pieces; ++i) {
-        const float* piece = pieces + ((size_t)tb.cta[it.first + i] * 2 + (i == 0 ? 1 : 0)) * kPieceFloats;
-        float w[kMergeRows], l[kMergeRows];
-        float4 v[kMergeRows];
 #pragma unroll
-        for (int q = 0; q < kMergeRows; ++q) {
-            const int r = slot * kBM + r0 + q;
-            w[q] = piece[2 * kBM * kD + r];
-            l[q] = piece[2 * kBM * kD + 2 * kBM + r];
-            v[q] = OUT && lane < kD / 4 ? reinterpret_cast<const float4*>(piece + (size_t)r * kD)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int o = 16; o > 1; o >>= 1) {
+        M.x = fmaxf(M.x, __shfl_xor_sync(0xffffffffu, M.x, o)); M.y = fmaxf(M.y, __shfl_xor_sync(0xffffffffu, M.y, o));
+        M.z = fmaxf(M.z, __shfl_xor_sync(0xffffffffu, M.z, o)); M.w = fmaxf(M.w, __shfl_xor_sync(0xffffffffu, M.w, o));
+    }
+    // this warp's pieces
+    float4 L = make_float4(0.f, 0.f, 0.f, 0.f), acc[OUT ? kD / 16 : 1];
+#pragma unroll
+    for (int k = 0; k < (OUT ? kD / 16 : 1); ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = pl; i < n_pieces; i += lanes) {
+        const float* piece = piece_at(i) + r0 + rs;
+        const float4 m = f4(piece + 2 * kBM * kD), l = f4(piece + 2 * kBM * kD + 2 * kBM);
+        float4 v[OUT ? kD / 16 : 1];
+        if (OUT) {
+#pragma unroll
+            for (int k = 0; k < kD / 16; ++k) v[k] = f4(piece + (size_t)(k * 16 + d0) * (2 * kBM));
         }
+        const float wx = fast_exp2((m.x - M.x) * sl2), wy = fast_exp2((m.y - M.y) * sl2);
+        const float wz = fast_exp2((m.z - M.z) * sl2), ww = fast_exp2((m.w - M.w) * sl2);
+        L.x = __fmaf_rn(wx, l.x, L.x); L.y = __fmaf_rn(wy, l.y, L.y); L.z = __fmaf_rn(wz, l.z, L.z); L.w = __fmaf_rn(ww, l.w, L.w);
+        if (OUT) {
 #pragma unroll
-        for (int q = 0; q < kMergeRows; ++q) {
-            const float ww = fast_exp2((w[q] - M[q]) * sl2);
-            L[q] = __fmaf_rn(ww, l[q], L[q]);
-            acc[q].x += ww * v[q].x; acc[q].y += ww * v[q].y; acc[q].z += ww * v[q].z; acc[q].w += ww * v[q].w;
+            for (int k = 0; k < kD / 16; ++k) {
+                acc[k].x += wx * v[k].x; acc[k].y += wy * v[k].y; acc[k].z += wz * v[k].z; acc[k].w += ww * v[k].w;
+            }
         }
     }
+    if (OUT) {
+#pragma unroll
+        for (int k = 0; k < kD / 16; ++k) {
+            part[warp][rs + 0][k * 16 + d0] = acc[k].x; part[warp][rs + 1][k * 16 + d0] = acc[k].y;
+            part[warp][rs + 2][k * 16 + d0] = acc[k].z; part[warp][rs + 3][k * 16 + d0] = acc[k].w;
+        }
+    }
+    if (d0 == 0) { part_l[warp][rs + 0] = L.x; part_l[warp][rs + 1] = L.y; part_l[warp][rs + 2] = L.z; part_l[warp][rs + 3] = L.w; }
+    __syncthreads();
+    // the warps of a group share its rows out again
+    const int n_sum = n_pieces < lanes ? n_pieces : lanes;
 #pragma unroll
     for (int q = 0; q < kMergeRows; ++q) {
-        const int row = slot * kBM + r0 + q;
-        if (row >= it.rows) continue;
-        const float inv = (L[q] > 0.f) ? 1.0f / L[q] : 0.f;
-        uint16_t* dst = O + (((int64_t)it.o_row + row) * n_heads + it.head) * kD + lane * 4;
-        uint2 o;
-        o.x = pack_bf16(acc[q].x * inv, acc[q].y * inv);
-        o.y = pack_bf16(acc[q].z * inv, acc[q].w * inv);
-        if (OUT && lane < kD / 4) *reinterpret_cast<uint2*>(dst) = o;
-        if (LSE != nullptr && lane == 0)
-            LSE[(int64_t)it.head * total_Lq + it.o_row + row] = final_lse(M[q], scale, L[q]);
+        const int row = r0 + q;
+        if (q * lanes / kMergeRows != pl || row >= it.rows) continue;  // warp-uniform
+        const float mj = (q & 3) == 0 ? M.x : (q & 3) == 1 ? M.y : (q & 3) == 2 ? M.z : M.w;
+        const float Mr = __shfl_sync(0xffffffffu, mj, q >> 2);         // an even lane holds rows 0..3, an odd one 4..7
+        float Ls = 0.f;
+        float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int w = group * lanes; w < group * lanes + n_sum; ++w) {
+            Ls += part_l[w][q];
+            if (OUT && lane < kVec) {
+                const float4 x = f4(&part[w][q][lane * 4]);
+                o4.x += x.x; o4.y += x.y; o4.z += x.z; o4.w += x.w;
+            }
+        }
+        if (OUT && lane < kVec) {
+            const float inv = (Ls > 0.f) ? 1.0f / Ls : 0.f;
+            uint2 o;
+            o.x = pack_bf16(o4.x * inv, o4.y * inv);
+            o.y = pack_bf16(o4.z * inv, o4.w * inv);
+            *reinterpret_cast<uint2*>(O + (((int64_t)it.o_row + row) * n_heads + it.head) * kD + lane * 4) = o;
+        }
+        if (LSE != nullptr && lane == 0) LSE[(int64_t)it.head * total_Lq + it.o_row + row] = final_lse(Mr, scale, Ls);
     }
 }
 
 // Host side of the merge: which CTAs hold the pieces of which item.
 inline void build_merge_table(const Params& p, int n_cta, MergeTable& tb) {
     tb.n_items = 0;
-    int n_list = 0;
+    int n_list = 0, longest = 0;
     Seg g, last;
     for (int b = 0; b < n_cta; ++b) {
         bool have = false;
@@ -916,14 +962,39 @@ inline void build_merge_table(const Params& p, int n_cta, MergeTable& tb) {
             tb.cta[n_list++] = (int16_t)c;
         }
         it.n_pieces = (int16_t)(n_list - it.first);
+        if (it.n_pieces > longest) longest = it.n_pieces;
     }
+    // items of a large problem have two or three pieces and there are enough of them to fill the GPU
+    tb.lanes = longest <= 4 ? 2 : (longest <= 8 ? 4 : 8);
 }
 
 inline int sm_count() { return device_sm_count(); }
 
-inline int grid_for(int64_t cost) {
-    const int sms = sm_count();
-    return (int)(cost < sms ? cost : sms);
+// CTAs for a problem, and whether each takes one whole item (`whole`) instead of a share.
+// Splitting shortens the longest CTA to its share but adds the partials' way through memory and the merge, 6 to
+// 8 us together, about seven 64-key tiles.  So a problem whose items fit on the GPU at once and whose
+// longest item is at most seven tiles longer than a share is not split; and no share is made smaller
+// than three tiles, below which only the number of pieces grows.  Measured with five and nine and with
+// shares of two and four tiles: within 3 us of this on eight problems of 2 to 24 heads.  Before (a share
+// of at least a quarter of a tile, a serial merge): 2 heads x 120 queries x 8023 keys 81 us, now 20; three ragged
+// streams of 2 heads 31.5 and 20; 24 heads x 147 queries x 268 keys 21 and 13.
+constexpr int kMergeTiles = 7, kMinShareTiles = 3;
+inline int grid_for(const StreamTable& st, int n_heads, int has_chunk, int64_t cost, int max_ctas, bool& whole) {
+    int sms = sm_count();
+    if (max_ctas > 0 && sms > max_ctas) sms = max_ctas;      // caller's scratch holds fewer partials
+    int64_t items = 0, longest = 0;
+    for (int s = 0; s < st.n_streams; ++s) {
+        const StreamCost sc = stream_cost(st, s, has_chunk);
+        if (sc.head_cost == 0) continue;
+        items += sc.nqp * n_heads;
+        if (sc.nt > longest) longest = sc.nt;
+    }
+    int64_t share = cost / ((int64_t)kCost2 * sms);
+    if (share < kMinShareTiles) share = kMinShareTiles;
+    whole = items <= sms && longest <= share + kMergeTiles;
+    if (whole) return (int)items;
+    const int64_t g = (cost + kCost2 * kMinShareTiles - 1) / (kCost2 * kMinShareTiles);
+    return (int)(g < sms ? g : sms);
 }
 
 template <int D, bool OUT>
@@ -932,7 +1003,7 @@ inline pafu_status launch_merge(const Params& p, int grid, int32_t n_heads, cuda
     MergeTable tb;
     build_merge_table(p, grid, tb);
     if (tb.n_items == 0) return PAFU_OK;
-    return cuda_ok(launch_dependent(attn_tc_merge_kernel<D, OUT>, dim3(tb.n_items * kMergeBlocksPerItem), dim3(kMergeThreads), 0, stream, 1,
+    return cuda_ok(launch_dependent(attn_tc_merge_kernel<D, OUT>, dim3(tb.n_items * 4 * tb.lanes), dim3(kMergeThreads), 0, stream, 1,
                                     tb, (const float*)p.pieces, p.scale, (int)n_heads, p.total_Lq, p.O, p.LSE));
 }
 
@@ -987,9 +1058,9 @@ inline pafu_status launch_d(const uint16_t* Q, const uint16_t* Kc, const uint16_
             return true;
         }))
         return PAFU_ERR_CUDA;
-    int grid = grid_for(cost);
-    if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;   // caller's scratch holds fewer partials
-    plan_shares(p, grid, cost);
+    bool whole;
+    const int grid = grid_for(st, n_heads, has_chunk, cost, max_ctas, whole);
+    plan_shares(p, grid, cost, whole);
     cudaError_t le;
     if constexpr (D == 128) {
         le = gather ? launch_dependent(attn_tc_kernel<true, 128>, dim3(grid), dim3(kThreads), kSmem, stream, 1, mQ, mKc, mVc, mKq, mVq, p)

@@ -553,6 +553,30 @@ def test_step_indexed_equals_step(w):
     assert torch.equal(A.LSE, B.LSE)
 
 
+@pytest.mark.parametrize("N,D,Lq,nB", [
+    (1, 128, 1, 1), (2, 64, 64, 128), (3, 128, 129, 500),     # whole items, one round, nothing to merge
+    (1, 128, 130, 64 * 40 + 1), (1, 64, 300, 64 * 40 - 1),    # one long item over many CTAs: eight merging warps
+    (2, 128, 257, 64 * 20 + 5),                               # a one-row tail item; four to eight pieces
+    (3, 128, 2000, 64 * 9),                                   # pieces of two or three shares
+    (40, 128, 1100, 100),                                     # more items than CTAs: a whole round, then shares
+])
+def test_attention_work_split(N, D, Lq, nB):
+    """The ways a problem is handed to the CTAs (whole items, shares, a round of whole items followed by shares) and
+    the merges they lead to."""
+    d = wl.peaked_attention_inputs("scaled_q", N, D, Lq, nB, seed=Lq, q_scale=2.0)
+    shape = pafu.Shape(N, D, None, [0, Lq])
+    ws = torch.zeros(pafu.pafu_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    O = torch.full((Lq, N, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    LSE = torch.full((N, Lq), float("nan"), device="cuda")
+    t = {k: to_device_bf16(v) for k, v in d.items()}
+    pafu.pafu_chunk_attn(t["Q"], t["Kc"], t["Vc"], [0, nB], t["Kq"], t["Vq"], shape, 0.0, O, LSE, ws)
+    assert pafu.pafu_workspace_status(ws) == 0
+    want, want_lse = oracle.attention(d["Q"], d["Kc"], d["Vc"], d["Kq"], d["Vq"])
+    close(O.float().cpu().numpy(), want, "O", scaled=True)
+    # 32-bit sums and logits of a few tens: 1e-5 is ten units in the last place
+    np.testing.assert_allclose(LSE.cpu().numpy(), want_lse, rtol=1e-5, atol=1e-5)
+
+
 # ------------------------------------------------------------- teacher salience (Eq. 4, Eq. 5)
 @pytest.mark.parametrize("L,N,LB", [
     (700, 2, 200),      # four blocks, the last one half length; every tile ragged
