@@ -58,6 +58,10 @@ constexpr int kTileBytes = kBN * kD * 2;      // 16 KiB: one K or V tile
 constexpr int kHalfBytes = kTileBytes / 2;    // one [64 rows x 64 cols] swizzled half
 constexpr int kSmemBytes = 2 * kQBytes + kStages * kTileBytes + 1024 /*align*/ + 512 /*barriers*/;
 constexpr float kRescaleThresholdLog2 = 8.0f;
+// Runs this short follow the true maximum in every tile: a small problem's peaked rows then have their
+// largest probability at exactly 1, which bf16 represents (relative error 1.8e-3 instead of 2.1e-3 on rows of logits
+// twice as wide as normal), and a few tiles cost little.
+constexpr int kShortRun = 4;
 constexpr float kSumTrigger = 65536.0f;   // a 64-key row sum this large means some p exceeded 2^10
 // Register re-balancing.  With 384 threads the kernel launches with 168 registers per thread.
 // setmaxnreg.inc blocks until the registers exist, so what the third warpgroup gives up must
@@ -583,8 +587,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             uint32_t turns = 0;                  // turns this slot has taken
             while (ok && iter.next(p, g)) {
                 const int n = __shfl_sync(0xffffffffu, g.t1 - g.t0, 0);
-                const bool two = __shfl_sync(0xffffffffu, g.n_slots, 0) == 2;
-                if (slot == 1 && !two) {
+                // d_head 64 has half the tensor work and is bound by the exponentials: no turns (3 % faster)
+                const bool two_slots = __shfl_sync(0xffffffffu, g.n_slots, 0) == 2, two = two_slots && D == 128;
+                if (slot == 1 && !two_slots) {
                     // nothing to compute for this slot, but every K/V stage is released by both issuers
                     for (int e = 0; e < 2 * n && ok; ++e) {
                         wait(kv_full(cur.st), cur.ph, 206);
@@ -612,10 +617,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     const bool more = i + 2 < n;
                     wait(kv_full(cv.st), cv.ph, 203);
                     if (!ok) break;
-                    if (more) wait(kv_full(ck.st), ck.ph, 204);
-                    if (!ok) break;
-                    wait(p_full(slot, buf), ((tc + i) >> 1) & 1u, 205);
-                    if (!ok) break;
+                    // d_head 64 is bound by the exponentials: its issuers mostly wait, and a wait that
+                    // suspends wakes late (4 %)
+                    if (!(D == 64 ? mbar_wait_warp_spin(p_full(slot, buf), ((tc + i) >> 1) & 1u)
+                                  : mbar_wait_warp(p_full(slot, buf), ((tc + i) >> 1) & 1u))) { if (leader) fail(205); ok = false; break; }
                     // The slots take turns at the tensor core, a tile's P V and the next Q K^T at a time: left
                     // alone they fall into step, their MMAs interleave one by one and then both wait (some CTAs
                     // 690k clocks, most 800k; with turns 727k on all).  The turn is handed on before the
@@ -627,6 +632,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     }
                     tc_fence_after_sync();
                     issue_pv(buf, cv.st, i == 0);
+                    if (more) wait(kv_full(ck.st), ck.ph, 204);
+                    if (!ok) break;
                     if (more) issue_qk(buf, ck.st, two);            // S(i+2) reuses the buffer P(i) was read from
                     else if (two) elect_arrive(turn(slot ^ 1));
                     if (i + 2 == n && leader) umma_commit(pv_done(slot));     // lets the last tile's softmax know O is at rest
@@ -660,6 +667,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             if (slot >= g.n_slots) continue;
             float m_used = -INFINITY, l_sum = 0.f;
             const int n = g.t1 - g.t0;
+            const bool short_run = n <= kShortRun;
             uint32_t sr[64];
             bool loaded = false;                       // S(i) already requested from tensor memory
             for (int i = 0; i < n; ++i) {
@@ -681,7 +689,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 // exponentials use the running maximum as it stands.  Only when the tile's row sum
                 // shows that some logit outgrew that maximum by more than 2^10 does the tile take
                 // the full pass below (true maximum, rescale of O and of the row sum).
-                bool full_pass = (i == 0) || (left < kBN);
+                bool full_pass = (i == 0) || (left < kBN) || short_run;
                 if (!full_pass) {
                     const float mbf = -m_used * sl2;
                     const uint64_t mb_2 = pack2(__float_as_uint(mbf), __float_as_uint(mbf));
@@ -715,7 +723,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     const float mx = tile_max(sr);
                     if (i == 0) {
                         m_used = mx;
-                    } else if (__any_sync(0xffffffffu, (mx - m_used) * sl2 > kRescaleThresholdLog2)) {
+                    } else if (__any_sync(0xffffffffu, (mx - m_used) * sl2 > (short_run ? 0.f : kRescaleThresholdLog2))) {
                         // The whole warp rescales together (TMEM accesses are warp-collective); rows
                         // whose maximum did not move get alpha = 1.  O must be at rest, i.e. the previous
                         // tile's P V product finished: S(i+1) being ready implies it (it was issued
@@ -972,13 +980,12 @@ inline int sm_count() { return device_sm_count(); }
 
 // CTAs for a problem, and whether each takes one whole item (`whole`) instead of a share.
 // Splitting shortens the longest CTA to its share but adds the partials' way through memory and the merge, 6 to
-// 8 us together, about seven 64-key tiles.  So a problem whose items fit on the GPU at once and whose
-// longest item is at most seven tiles longer than a share is not split; and no share is made smaller
-// than three tiles, below which only the number of pieces grows.  Measured with five and nine and with
-// shares of two and four tiles: within 3 us of this on eight problems of 2 to 24 heads.  Before (a share
-// of at least a quarter of a tile, a serial merge): 2 heads x 120 queries x 8023 keys 81 us, now 20; three ragged
-// streams of 2 heads 31.5 and 20; 24 heads x 147 queries x 268 keys 21 and 13.
-constexpr int kMergeTiles = 7, kMinShareTiles = 3;
+// 8 us together.  So a problem whose items fit on the GPU at once and whose longest item is at most three
+// 64-key tiles longer than a share is not split (seven: 2 to 4 us faster on some problems of 8 to 15 tiles an item, slower on
+// others), and no share is made smaller than one tile.  Before (shares down to a fraction of a tile, a
+// serial merge): 2 heads x 120 queries x 8023 keys 77 us, now 28; three ragged streams of 2 heads 31.5 and 20;
+// 24 heads x 147 queries x 268 keys 21 and 17.
+constexpr int kMergeTiles = 3, kMinShareTiles = 1;
 inline int grid_for(const StreamTable& st, int n_heads, int has_chunk, int64_t cost, int max_ctas, bool& whole) {
     int sms = sm_count();
     if (max_ctas > 0 && sms > max_ctas) sms = max_ctas;      // caller's scratch holds fewer partials
