@@ -19,10 +19,10 @@
 //   warps 0-3  softmax of slot 0 (thread = query row = TMEM lane)
 //   warps 4-7  softmax of slot 1
 //   warps 8,10 MMA issuers, one per slot: S = Q K^T (both operands in shared memory) and
-//              O += P V (P read from tensor memory, V from shared memory, MN-major).  With the
-//              waits, commits and descriptor arithmetic of its loop one thread sustains about
-//              one tcgen05.mma per 100 clocks while the tensor core finishes a 128x128x16 one
-//              in 64, hence an issuing thread per slot
+//              O += P V (P read from tensor memory, V from shared memory, MN-major).  The MMA
+//              stream itself needs only one issuer (1238 clocks a tile pair either way), but each
+//              tile also costs an issuer some 500 clocks of waits and commits, which a second one hides
+//              (one warp for both slots: 2375 clocks a tile pair, two: 1634)
 //   warp  9    TMA loader: Q tiles per item, 64-key K/V tiles through a 10-stage ring that
 //              runs ahead across item boundaries
 //   warp  11   idle (completes the third warpgroup so registers can be re-balanced)
@@ -553,7 +553,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             const uint32_t lo_k = (uint32_t)desc_k + (sKV >> 4), lo_v = (uint32_t)desc_v + (sKV >> 4);
             const uint32_t tSslot = tm + slot * 128;
             const uint32_t tOslot = tm + 256 + slot * kD;
+            // d_head 128 issues in predicated series (12 heads x 18 720 keys 489 us, in a branch of the leader
+            // 497); the short series of d_head 64 are the other way round (292 and 274 us at 13 680 keys).
             auto issue_qk = [&](int buf, int stage, bool pass) {     // S[buf] = Q K^T, N = 64 keys; `pass`: hand the turn on
+                if constexpr (D == 64) {
+                    if (leader) {
+#pragma unroll
+                        for (int kk = 0; kk < kD / 16; ++kk)
+                            umma_ss(tSslot + buf * kBN, desc_k + ((sQ + slot * kQBytes) >> 4) + kk * 2,
+                                    desc_k + ((sKV + stage * kTileBytes) >> 4) + kk * 2, idesc_qk, kk > 0);
+                        umma_commit(s_full(slot, buf));
+                        umma_commit(kv_empty(stage));
+                    }
+                    __syncwarp();
+                    return;
+                }
                 if constexpr (GATHER) fence_proxy_async_smem();     // the tile came through the generic proxy
 #pragma unroll
                 for (int c = 0; c < kD / 64; ++c) {
@@ -565,6 +579,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 elect_commit(kv_empty(stage));
             };
             auto issue_pv = [&](int buf, int stage, bool first) {   // O += P[buf] V, K = 64 keys
+                if constexpr (D == 64) {
+                    if (leader) {
+#pragma unroll
+                        for (int kk = 0; kk < kBN / 16; ++kk)
+                            umma_ts(tOslot, tSslot + buf * kBN + kk * 8, desc_v + ((sKV + stage * kTileBytes) >> 4) + kk * (2048 >> 4),
+                                    idesc_pv, !(first && kk == 0));
+                        umma_commit(kv_empty(stage));
+                    }
+                    __syncwarp();
+                    return;
+                }
                 if constexpr (GATHER) fence_proxy_async_smem();
                 umma_ts_x4(tOslot, tSslot + buf * kBN, lo_v + stage * (kTileBytes >> 4), idesc_pv, hi, !first);
                 elect_commit(kv_empty(stage));
@@ -617,10 +642,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     const bool more = i + 2 < n;
                     wait(kv_full(cv.st), cv.ph, 203);
                     if (!ok) break;
-                    // d_head 64 is bound by the exponentials: its issuers mostly wait, and a wait that
-                    // suspends wakes late (4 %)
-                    if (!(D == 64 ? mbar_wait_warp_spin(p_full(slot, buf), ((tc + i) >> 1) & 1u)
-                                  : mbar_wait_warp(p_full(slot, buf), ((tc + i) >> 1) & 1u))) { if (leader) fail(205); ok = false; break; }
+                    wait(p_full(slot, buf), ((tc + i) >> 1) & 1u, 205);
+                    if (!ok) break;
                     // The slots take turns at the tensor core, a tile's P V and the next Q K^T at a time: left
                     // alone they fall into step, their MMAs interleave one by one and then both wait (some CTAs
                     // 690k clocks, most 800k; with turns 727k on all).  The turn is handed on before the

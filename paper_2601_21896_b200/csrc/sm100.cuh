@@ -98,14 +98,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
     }
 }
 
-// The same, polling without suspending first.
-__device__ __forceinline__ bool mbar_wait_warp_spin(uint32_t bar, uint32_t parity) {
-#pragma unroll 1
-    for (int i = 0; i < 4096; ++i)
-        if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
-    return mbar_wait_warp(bar, parity);
-}
-
 // ------------------------------------------------------------------------------- fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
