@@ -653,6 +653,7 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
     const int from = c->cur;
     int64_t keep = 0;
     int select_ctas = 0;
+    bool prune = false;
     if (c->T + chunk > c->capacity) {
         keep = c->capacity - chunk;
         if (keep > 0) {
@@ -671,18 +672,21 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
             if (e != PAFU_OK) return e;
             select_ctas = select_cta_count(st);
         }
-        c->cur ^= 1;
-        c->T = keep;
-        if (pruned != nullptr) *pruned = 1;
+        prune = true;
     }
     // 2. every layer's new rows go to the tail of its K and V, the kept ones to the front of the other set
-    const int to = c->cur;
-    e = launch_cache_rows(Knew, Vnew, chunk, c->K[from], c->V[from], c->SL[from], c->idx, keep, c->T, c->K[to], c->V[to],
+    const int to = prune ? from ^ 1 : from;
+    const int64_t dst0 = prune ? keep : c->T;
+    e = launch_cache_rows(Knew, Vnew, chunk, c->K[from], c->V[from], c->SL[from], c->idx, keep, dst0, c->K[to], c->V[to],
                           c->SL[to], c->n_layers, (int32_t)dm, select_ctas, cs);
     if (e != PAFU_OK) return e;
+    // the host fields follow what is enqueued: a launch that failed leaves them as they were
+    c->cur = to;
+    c->T = dst0;
+    if (pruned != nullptr && prune) *pruned = 1;
     // 3. the chunk's salience scores go straight to the tail of SL, computed beside the copies
     const uint16_t* parts[3] = {Qs, Ks, Vs};
-    e = launch_score(*head, parts, 3, chunk, dm, c->SL[to] + c->T, ws, ws_bytes, cs, 1);
+    e = launch_score(*head, parts, 3, chunk, dm, c->SL[to] + dst0, ws, ws_bytes, cs, 1);
     if (e != PAFU_OK) return e;
     c->T += chunk;
     return PAFU_OK;

@@ -6,6 +6,7 @@ import re
 
 import numpy as np
 import pytest
+import torch
 
 import paper_2601_21896_b200 as pafu
 from paper_2601_21896_b200 import binding as B
@@ -215,6 +216,27 @@ def test_cache_update_rejects_bad_arguments_on_host(L):
     c65, _ = make(); c65.n_layers = 65
     assert call(c65)[0] == 3
     assert (c.T, c.cur) == (300, 0)
+
+
+@pytest.mark.skipif(torch.cuda.is_available(), reason="the launches must fail: fake device addresses")
+@pytest.mark.parametrize("T,chunk", [(300, 1024), (1024, 256), (300, 256)])
+def test_cache_update_leaves_the_cache_as_it_was_when_a_launch_fails(L, T, chunk):
+    """Without a device the first launch fails: the update reports it and the host fields still describe the
+    buffers, whether the chunk replaces the whole cache (nothing to select), prunes it or fits."""
+    fake, n_layers, N, D, cap, MB = 0x7f0000000000, 2, 2, 64, 1024, 1 << 20
+    ptrs = lambda base: (ctypes.c_void_p * n_layers)(*[base + l * MB for l in range(n_layers)])
+    arrs = [ptrs(fake + 16 * MB * i) for i in range(1, 5)]
+    c = B.CCache()
+    c.n_layers, c.n_heads, c.d_head, c.cur, c.capacity, c.n_sink, c.T = n_layers, N, D, 1, cap, 16, T
+    c.K[0], c.K[1], c.V[0], c.V[1] = [ctypes.cast(a, ctypes.c_void_p) for a in arrs]
+    c.SL[0], c.SL[1], c.idx = fake + 96 * MB, fake + 97 * MB, fake + 98 * MB
+    head = B.CHead(3 * N * D, 64, 12, 1, 0, fake + 100 * MB, None, fake + 101 * MB, None)
+    new = ptrs(fake + 110 * MB)
+    pr = ctypes.c_int32(7)
+    rc = L.pafu_cache_update(ctypes.byref(c), ctypes.byref(head), fake, fake, fake, new, new, chunk, ctypes.byref(pr),
+                             fake + 120 * MB, 1 << 20, None)
+    assert rc == 6                                              # PAFU_ERR_CUDA
+    assert (c.T, c.cur, pr.value) == (T, 1, 0)
 
 
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
