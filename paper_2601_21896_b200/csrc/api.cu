@@ -677,17 +677,32 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
     // 2. every layer's new rows go to the tail of its K and V, the kept ones to the front of the other set
     const int to = prune ? from ^ 1 : from;
     const int64_t dst0 = prune ? keep : c->T;
-    e = launch_cache_rows(Knew, Vnew, chunk, c->K[from], c->V[from], c->SL[from], c->idx, keep, dst0, c->K[to], c->V[to],
-                          c->SL[to], c->n_layers, (int32_t)dm, select_ctas, cs);
+    const uint16_t* parts[3] = {Qs, Ks, Vs};
+    // The S-MLP runs beside the copies unless its inputs lie where they write: rows that the append
+    // overwrites have to be read first, and rows that the gather fills have to be filled first.
+    const int64_t first = prune ? 0 : dst0;
+    bool apart = false;
+    for (int l = 0; l < c->n_layers; ++l)
+        for (const uint16_t* x : parts)
+            apart = apart || ranges_overlap(x, (size_t)chunk * dm * 2, c->K[to][l] + first * dm, (size_t)(dst0 + chunk - first) * dm * 2) ||
+                    ranges_overlap(x, (size_t)chunk * dm * 2, c->V[to][l] + first * dm, (size_t)(dst0 + chunk - first) * dm * 2);
+    auto copy_rows = [&](int64_t n_new, int64_t n_keep, int sel) {
+        return launch_cache_rows(Knew, Vnew, n_new, c->K[from], c->V[from], c->SL[from], c->idx, n_keep, dst0, c->K[to], c->V[to],
+                                 c->SL[to], c->n_layers, (int32_t)dm, sel, cs);
+    };
+    e = apart && keep == 0 ? PAFU_OK : copy_rows(apart ? 0 : chunk, keep, select_ctas);
     if (e != PAFU_OK) return e;
     // the host fields follow what is enqueued: a launch that failed leaves them as they were
     c->cur = to;
     c->T = dst0;
     if (pruned != nullptr && prune) *pruned = 1;
-    // 3. the chunk's salience scores go straight to the tail of SL, computed beside the copies
-    const uint16_t* parts[3] = {Qs, Ks, Vs};
-    e = launch_score(*head, parts, 3, chunk, dm, c->SL[to] + dst0, ws, ws_bytes, cs, 1);
+    // 3. the chunk's salience scores go straight to the tail of SL
+    e = launch_score(*head, parts, 3, chunk, dm, c->SL[to] + dst0, ws, ws_bytes, cs, apart ? 0 : 1);
     if (e != PAFU_OK) return e;
+    if (apart) {
+        e = copy_rows(chunk, 0, 0);
+        if (e != PAFU_OK) return e;
+    }
     c->T += chunk;
     return PAFU_OK;
 }

@@ -129,7 +129,7 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
 // The row copies of a rolling-cache update, all layers in one launch: n_new rows of Knew/Vnew to row `dst0` on of
 // Kd/Vd, and rows idx[0 .. keep) of Ks/Vs (and SL) to the front of Kd/Vd (and SLd).
 // select_ctas > 0: launched directly behind launch_select(.., trigger_late = 1), which occupies that many
-// CTAs; 0: after what is ahead (keep must be 0).
+// CTAs; 0: after what is ahead (keep must be 0).  n_new or keep may be 0, not both.
 pafu_status launch_cache_rows(const uint16_t* const* Knew, const uint16_t* const* Vnew, int64_t n_new,
                               const uint16_t* const* Ks, const uint16_t* const* Vs, const float* SL, const int32_t* idx,
                               int64_t keep, int64_t dst0, uint16_t* const* Kd, uint16_t* const* Vd, float* SLd, int32_t n_layers,

@@ -493,6 +493,47 @@ def test_cache_update_entry_point_over_chunks(chunk, cap, n_sink):
     assert n_pruned >= 3
 
 
+@pytest.mark.parametrize("T,where", [(300, "append"), (128, "append"), (300, "kept"), (256, "append")])
+def test_cache_update_head_inputs_in_the_idle_buffers(T, where):
+    """The head's input rows may lie in buffers that the update writes: in rows that the append overwrites (they are
+    read before), or in rows that the gather fills (they are read after).  Pruning (T = 300, 256), nothing kept (a chunk of the
+    whole capacity at T = 256) and not pruning (T = 128)."""
+    N, D, n_layers, cap = 2, 128, 3, 300
+    chunk = cap if T == 256 else 150
+    rng = np.random.default_rng(T)
+    rows = lambda n: to_device_bf16(wl.f32_to_bf16_bits(rng.standard_normal((n, N, D)).astype(np.float32)))
+    w1, w2 = rng.standard_normal((64, 3 * N * D)) / 30, rng.standard_normal((12, 64)) / 8
+    head = pafu.Head(*[to_device_bf16(wl.f32_to_bf16_bits(w.astype(np.float32))) for w in (w1, w1[:, 0], w2, w2[:, 0])],
+                     wl.ACT_SILU, wl.FINAL_NONE)
+    ws = torch.zeros(pafu.pafu_workspace_bytes(pafu.Shape(N, D, [0, cap], [0, chunk]), None, head), dtype=torch.uint8, device="cuda")
+    old = [[rows(cap) for _ in range(n_layers)] for _ in range(2)]
+    new = [[rows(chunk) for _ in range(n_layers)] for _ in range(2)]
+    SL, q = torch.randn(cap, generator=torch.Generator().manual_seed(T)), rows(chunk)
+    res = []
+    for inside in (False, True):
+        cache = pafu.Cache(n_layers, N, D, cap, 16)
+        for l in range(n_layers):
+            cache.Kb[0][l].copy_(old[0][l]); cache.Vb[0][l].copy_(old[1][l])
+        cache.SLb[0].copy_(SL)
+        cache.c.T = T
+        prune = T + chunk > cap
+        to, dst = (1, cap - chunk) if prune else (0, T)
+        Qs, Ks, Vs = q, new[0][-1], new[1][-1]
+        if where == "kept":                               # the first `chunk` rows that the pruning keeps in layer 1
+            kept = np.sort(np.concatenate([np.arange(16), 16 + np.argsort(-SL.numpy()[16:T], kind="stable")[: cap - chunk - 16]]))
+            Qs = old[0][1][torch.from_numpy(kept).cuda()]
+            if inside:
+                Qs = cache.Kb[to][1][:chunk]
+        elif inside:
+            cache.Kb[to][0][dst:dst + chunk].copy_(q); Qs = cache.Kb[to][0][dst:dst + chunk]
+            cache.Vb[to][2][dst:dst + chunk].copy_(Vs); Vs = cache.Vb[to][2][dst:dst + chunk]
+        assert pafu.pafu_cache_update(cache, head, Qs, Ks, Vs, new[0], new[1], ws) == prune
+        assert pafu.pafu_workspace_status(ws) == 0
+        res.append([t.clone() for t in [cache.SL] + cache.K + cache.V])
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
+
+
 # --------------------------------------------------------------- attention through indices
 def test_indexed_attention_matches_oracle_and_compacted_path():
     """Select(KV; ids) applied inside the attention loader (Eq. 7's index set) instead of as a
