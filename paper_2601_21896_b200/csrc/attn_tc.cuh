@@ -452,9 +452,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     o0 = o1 = 0;
                     if (j < g.t1 && j < g.nt1) {
                         int64_t pos = (int64_t)j * kBN + lane;
-                        o0 = (uint32_t)(row_base + __ldg(sidx + (pos < g.nB ? pos : g.nB - 1))) * row16;
+                        o0 = (uint32_t)(row_base + ld_index(sidx + (pos < g.nB ? pos : g.nB - 1))) * row16;
                         pos += 32;
-                        o1 = (uint32_t)(row_base + __ldg(sidx + (pos < g.nB ? pos : g.nB - 1))) * row16;
+                        o1 = (uint32_t)(row_base + ld_index(sidx + (pos < g.nB ? pos : g.nB - 1))) * row16;
                     }
                 };
                 uint32_t o0, o1, n0, n1;

@@ -82,6 +82,14 @@ __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.w
 // Lets the kernel launched behind this one (as a programmatic dependent) start now; that kernel
 // still sees this one's results only after its own grid_dep_wait().
 __device__ __forceinline__ void grid_dep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// An index written by the kernel ahead while this one may already be running: read after
+// grid_dep_wait(), and not through the read-only path (__ldg, const __restrict__), which may be used - and moved
+// above the wait - only for what nothing writes during the kernel's whole lifetime.
+__device__ __forceinline__ int32_t ld_index(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 #endif
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,

@@ -69,7 +69,7 @@ __device__ __forceinline__ int64_t claim_get(int pending) { return __shfl_sync(0
 
 __global__ void __launch_bounds__(kCompactWarpsPerBlock * 32)
 compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
-                    const float* __restrict__ SL, const int32_t* __restrict__ idx,
+                    const float* __restrict__ SL, const int32_t* idx,
                     const __grid_constant__ StreamTable st, int32_t chunks_per_row,
                     uint4* __restrict__ Kc, uint4* __restrict__ Vc, float* __restrict__ SLc,
                     int64_t n_rows, int* __restrict__ work, int early_static) {
@@ -81,7 +81,7 @@ compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
         for (int64_t r = warp0; r < n_rows; r += n_warps) {
             int s = 0;
             while (s + 1 < st.n_streams && r >= st.cu_B[s + 1]) ++s;
-            copy_kv_row(K, V, SL, st.cu_T[s] + (int64_t)__ldg(idx + r), r, chunks_per_row, Kc, Vc, SLc, lane);
+            copy_kv_row(K, V, SL, st.cu_T[s] + (int64_t)ld_index(idx + r), r, chunks_per_row, Kc, Vc, SLc, lane);
         }
         return;
     }
@@ -111,7 +111,7 @@ compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
         int64_t p = q;
         for (; p >= st.k[s]; ++s) p -= st.k[s];
         const int64_t r = st.cu_B[s] + st.n_sink[s] + p;
-        copy_kv_row(K, V, SL, st.cu_T[s] + (int64_t)__ldg(idx + r), r, chunks_per_row, Kc, Vc, SLc, lane);
+        copy_kv_row(K, V, SL, st.cu_T[s] + (int64_t)ld_index(idx + r), r, chunks_per_row, Kc, Vc, SLc, lane);
     };
     int64_t n_top = 0;
     for (int s = 0; s < st.n_streams; ++s) n_top += st.k[s];
@@ -121,7 +121,7 @@ compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
             int s = 0;
             while (s + 1 < st.n_streams && a >= st.cu_B[s + 1]) ++s;
             const int64_t ns = st.n_sink[s], k = st.k[s], p = a - st.cu_B[s];
-            if (k == 0 || p < ns || p >= ns + k) SLc[a] = __ldg(SL + st.cu_T[s] + __ldg(idx + a));
+            if (k == 0 || p < ns || p >= ns + k) SLc[a] = __ldg(SL + st.cu_T[s] + ld_index(idx + a));
         }
     };
     if (early_static) {
@@ -167,7 +167,7 @@ struct LayerPtrs {
 
 __global__ void __launch_bounds__(kCompactWarpsPerBlock * 32)
 compact_layers_kernel(const __grid_constant__ LayerPtrs lp, int32_t n_layers,
-                      const float* __restrict__ SL, const int32_t* __restrict__ idx,
+                      const float* __restrict__ SL, const int32_t* idx,
                       const __grid_constant__ StreamTable st, int32_t chunks_per_row,
                       float* __restrict__ SLc, int64_t n_rows) {
     grid_dep_wait();
@@ -179,7 +179,7 @@ compact_layers_kernel(const __grid_constant__ LayerPtrs lp, int32_t n_layers,
         const int64_t r = w - (int64_t)layer * n_rows;
         int s = 0;
         while (s + 1 < st.n_streams && r >= st.cu_B[s + 1]) ++s;
-        const int64_t src_row = st.cu_T[s] + (int64_t)__ldg(idx + r);
+        const int64_t src_row = st.cu_T[s] + (int64_t)ld_index(idx + r);
         copy_kv_row(lp.K[layer], lp.V[layer], SL, src_row, r, chunks_per_row, lp.Kc[layer], lp.Vc[layer],
                     layer == 0 ? SLc : nullptr, lane);
     }
@@ -217,7 +217,7 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
 // times layers stay far below 2^32: each is at least 32 bytes of three buffers.)
 __global__ void __launch_bounds__(kCompactWarpsPerBlock * 32)
 cache_rows_kernel(const __grid_constant__ LayerPtrs add, const __grid_constant__ LayerPtrs keep, int32_t n_layers,
-                  int32_t n_new, int64_t dst0, const float* __restrict__ SL, const int32_t* __restrict__ idx, int32_t n_keep,
+                  int32_t n_new, int64_t dst0, const float* __restrict__ SL, const int32_t* idx, int32_t n_keep,
                   int32_t chunks_per_row, float* __restrict__ SLd, int behind_select) {
     if (!behind_select) grid_dep_wait();
     grid_dep_launch_dependents();     // everything ahead of the selection (or of this kernel) is complete here
@@ -231,7 +231,7 @@ cache_rows_kernel(const __grid_constant__ LayerPtrs add, const __grid_constant__
     if (behind_select) grid_dep_wait();
     for (uint32_t w = warp0; w < (uint32_t)n_keep * n_layers; w += n_warps) {
         const uint32_t layer = w / n_keep, r = w - layer * n_keep;
-        copy_kv_row(keep.K[layer], keep.V[layer], SL, (int64_t)__ldg(idx + r), r, chunks_per_row, keep.Kc[layer], keep.Vc[layer],
+        copy_kv_row(keep.K[layer], keep.V[layer], SL, (int64_t)ld_index(idx + r), r, chunks_per_row, keep.Kc[layer], keep.Vc[layer],
                     layer == 0 ? SLd : nullptr, lane);
     }
 }

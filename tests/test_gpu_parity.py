@@ -493,6 +493,46 @@ def test_cache_update_entry_point_over_chunks(chunk, cap, n_sink):
     assert n_pruned >= 3
 
 
+@pytest.mark.parametrize("cap,chunk", [
+    (1000, 200),                # one selecting CTA
+    (24576 + 16 + 129, 129),    # one candidate more than it takes: two
+    (60001, 700),               # four
+    (363001, 800),              # more candidates than a cluster holds: the streaming selection
+])
+def test_cache_updates_without_a_synchronisation_between_them(cap, chunk):
+    """Three updates of a full cache enqueued back to back: each one's selection, copies and head overlap, and the
+    next one starts behind them.  Against the oracle's selection on the scores the head gives for the same rows."""
+    N, D, n_layers, n_sink = 1, 64, 2, 16
+    g = torch.Generator(device="cuda").manual_seed(cap)
+    rows = lambda n: torch.randn(n, N, D, generator=g, device="cuda").to(torch.bfloat16)
+    w = [torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16) / 8 for s in ((64, 3 * N * D), (64,), (12, 64), (12,))]
+    head = pafu.Head(*w, wl.ACT_SILU, wl.FINAL_NONE)
+    ws = torch.zeros(pafu.pafu_workspace_bytes(pafu.Shape(N, D, [0, cap], [0, chunk]), None, head), dtype=torch.uint8, device="cuda")
+    cache = pafu.Cache(n_layers, N, D, cap, n_sink)
+    K, V = [rows(cap) for _ in range(n_layers)], [rows(cap) for _ in range(n_layers)]
+    for l in range(n_layers):
+        cache.Kb[0][l].copy_(K[l]); cache.Vb[0][l].copy_(V[l])
+    SL = torch.randn(cap, generator=g, device="cuda")
+    cache.SLb[0].copy_(SL)
+    cache.c.T = cap
+    chunks = [(rows(chunk), [rows(chunk) for _ in range(n_layers)], [rows(chunk) for _ in range(n_layers)]) for _ in range(3)]
+    torch.cuda.synchronize()
+    for q, kn, vn in chunks:
+        assert pafu.pafu_cache_update(cache, head, q, kn[-1], vn[-1], kn, vn, ws)
+    assert pafu.pafu_workspace_status(ws) == 0
+    for q, kn, vn in chunks:
+        ids = oracle.select(SL.cpu().numpy(), n_sink, 0, cap - chunk)
+        i = torch.from_numpy(ids.astype(np.int64)).cuda()
+        s = torch.empty(chunk, device="cuda")
+        pafu.pafu_score_qkv(head, q, kn[-1], vn[-1], s, ws, ld=N * D)
+        K = [torch.cat([a[i], b]) for a, b in zip(K, kn)]; V = [torch.cat([a[i], b]) for a, b in zip(V, vn)]
+        SL = torch.cat([SL[i], s])
+    assert np.array_equal(cache.idx[: cap - chunk].cpu().numpy(), ids)
+    assert torch.equal(cache.SL, SL)
+    for l in range(n_layers):
+        assert torch.equal(cache.K[l], K[l]) and torch.equal(cache.V[l], V[l])
+
+
 @pytest.mark.parametrize("T,where", [(300, "append"), (128, "append"), (300, "kept"), (256, "append")])
 def test_cache_update_head_inputs_in_the_idle_buffers(T, where):
     """The head's input rows may lie in buffers that the update writes: in rows that the append overwrites (they are
