@@ -210,43 +210,86 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
 // A rolling-cache update's copies: the chunk's new rows of every layer, then the kept rows through the
 // index list.  The new rows need nothing that the selection ahead produces, so they are copied while
 // it runs; and the kernel lets the one behind it start at once: that is the salience head of the chunk,
-// tensor-bound work on one CTA an SM, which this kernel leaves registers for (one block of 256 threads
-// an SM: 86 registers each beside the head's 384 x 95 to 100).  30 layers, 4680 kept and 4680 new rows: 607 us as
-// select, gather, head and append one after the other, 586 us like this; ten or twelve warps in 78 or
-// 64 registers 590 and 662; only the append here and the gather behind the head 647.  (Row counts
-// times layers stay far below 2^32: each is at least 32 bytes of three buffers.)
+// tensor-bound work on one CTA an SM, which this kernel leaves registers for (one block of 256 threads an SM).
+//
+// Bound by memory.  What one block an SM reaches is set by its bytes in flight, so a warp's batch is a stretch of
+// kCompactUnroll x 32 sixteen-byte units of a layer's rows laid end to end, whatever the row width, and the
+// batch's indices are fetched one batch ahead.  (With a row at a time a warp had only that row in flight: 30
+// layers, 4680 kept and 4680 new rows of 256, 512, 1536, 3072 and 4096 bytes took 219, 243, 375, 590 and 828 us, now 71,
+// 117, 305, 588 and 781; as select, gather, head and append one after the other, many blocks an SM, 140, 164, 324,
+// 612 and 807.  With the indices fetched before the batch's loads instead of behind them 618 at 3072 bytes.)
+constexpr int kCacheSeg = kCompactUnroll * 32;     // units of a warp's batch
+
+// One batch: unit dst + 32 i comes from src[i]; `between` runs while its loads are under way.
+template <typename Between>
+__device__ __forceinline__ void copy_units(const uint4* K, const uint4* V, const uint32_t (&src)[kCompactUnroll], uint4* Kd, uint4* Vd,
+                                           uint32_t dst, uint32_t end, Between between) {
+    uint4 kb[kCompactUnroll], vb[kCompactUnroll];
+#pragma unroll
+    for (int i = 0; i < kCompactUnroll; ++i)
+        if (dst + i * 32 < end) { kb[i] = ld_nc_v4(K + src[i]); vb[i] = ld_nc_v4(V + src[i]); }
+    between();
+#pragma unroll
+    for (int i = 0; i < kCompactUnroll; ++i)
+        if (dst + i * 32 < end) { Kd[dst + i * 32] = kb[i]; Vd[dst + i * 32] = vb[i]; }
+}
+
+// (A layer's buffer holds less than 2^32 units: 64 GiB.)
 __global__ void __launch_bounds__(kCompactWarpsPerBlock * 32)
-cache_rows_kernel(const __grid_constant__ LayerPtrs add, const __grid_constant__ LayerPtrs keep, int32_t n_layers,
-                  int32_t n_new, int64_t dst0, const float* __restrict__ SL, const int32_t* idx, int32_t n_keep,
-                  int32_t chunks_per_row, float* __restrict__ SLd, int behind_select) {
+cache_rows_kernel(const __grid_constant__ LayerPtrs add, const __grid_constant__ LayerPtrs keep, uint32_t n_layers,
+                  uint32_t n_new, int64_t dst0, const float* __restrict__ SL, const int32_t* idx, uint32_t n_keep,
+                  uint32_t chunks_per_row, float* __restrict__ SLd, int behind_select) {
     if (!behind_select) grid_dep_wait();
     grid_dep_launch_dependents();     // everything ahead of the selection (or of this kernel) is complete here
     const int lane = threadIdx.x & 31;
     const uint32_t warp0 = blockIdx.x * kCompactWarpsPerBlock + (threadIdx.x >> 5);
     const uint32_t n_warps = gridDim.x * kCompactWarpsPerBlock;
-    for (uint32_t w = warp0; w < (uint32_t)n_new * n_layers; w += n_warps) {
-        const uint32_t layer = w / n_new, r = w - layer * n_new;
-        copy_kv_row(add.K[layer], add.V[layer], nullptr, r, dst0 + r, chunks_per_row, add.Kc[layer], add.Vc[layer], nullptr, lane);
+    const uint32_t new_units = n_new * chunks_per_row, new_segs = (new_units + kCacheSeg - 1) / kCacheSeg;
+    for (uint32_t w = warp0; w < new_segs * n_layers; w += n_warps) {
+        const uint32_t layer = w / new_segs, u = (w - layer * new_segs) * kCacheSeg + lane;
+        uint32_t src[kCompactUnroll];
+#pragma unroll
+        for (int i = 0; i < kCompactUnroll; ++i) src[i] = u + i * 32;
+        copy_units(add.K[layer], add.V[layer], src, add.Kc[layer] + dst0 * chunks_per_row, add.Vc[layer] + dst0 * chunks_per_row, u, new_units,
+                   [] {});
     }
     if (behind_select) grid_dep_wait();
-    for (uint32_t w = warp0; w < (uint32_t)n_keep * n_layers; w += n_warps) {
-        const uint32_t layer = w / n_keep, r = w - layer * n_keep;
-        copy_kv_row(keep.K[layer], keep.V[layer], SL, (int64_t)ld_index(idx + r), r, chunks_per_row, keep.Kc[layer], keep.Vc[layer],
-                    layer == 0 ? SLd : nullptr, lane);
+    const uint32_t keep_units = n_keep * chunks_per_row, keep_segs = (keep_units + kCacheSeg - 1) / kCacheSeg;
+    const uint32_t total = keep_segs * n_layers;
+    auto fetch = [&](uint32_t w, uint32_t (&src)[kCompactUnroll]) {      // where batch w's units come from
+        const uint32_t u = (w - w / keep_segs * keep_segs) * kCacheSeg + lane;
+#pragma unroll
+        for (int i = 0; i < kCompactUnroll; ++i) {
+            const uint32_t row = (u + i * 32) / chunks_per_row;
+            src[i] = 0;
+            if (u + i * 32 < keep_units) src[i] = (uint32_t)ld_index(idx + row) * chunks_per_row + (u + i * 32 - row * chunks_per_row);
+        }
+    };
+    uint32_t src[kCompactUnroll], ahead[kCompactUnroll];
+    if (warp0 < total) fetch(warp0, src);
+    for (uint32_t w = warp0; w < total; w += n_warps) {
+        const uint32_t layer = w / keep_segs;
+        copy_units(keep.K[layer], keep.V[layer], src, keep.Kc[layer], keep.Vc[layer], (w - layer * keep_segs) * kCacheSeg + lane,
+                   keep_units, [&] { if (w + n_warps < total) fetch(w + n_warps, ahead); });
+#pragma unroll
+        for (int i = 0; i < kCompactUnroll; ++i) src[i] = ahead[i];
     }
+    for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n_keep; r += gridDim.x * blockDim.x) SLd[r] = __ldg(SL + ld_index(idx + r));
 }
 
 pafu_status launch_cache_rows(const uint16_t* const* Knew, const uint16_t* const* Vnew, int64_t n_new,
                               const uint16_t* const* Ks, const uint16_t* const* Vs, const float* SL, const int32_t* idx,
                               int64_t keep, int64_t dst0, uint16_t* const* Kd, uint16_t* const* Vd, float* SLd, int32_t n_layers,
                               int32_t d_model, int select_ctas, cudaStream_t stream) {
-    int64_t blocks = ((n_new + keep) * n_layers + kCompactWarpsPerBlock - 1) / kCompactWarpsPerBlock;
+    const int64_t cpr = d_model / 8;
+    const int64_t segs = ((n_new * cpr + kCacheSeg - 1) / kCacheSeg + (keep * cpr + kCacheSeg - 1) / kCacheSeg) * n_layers;
+    int64_t blocks = (segs + kCompactWarpsPerBlock - 1) / kCompactWarpsPerBlock;
     // one block an SM, in fixed shares; the selection's SMs are left out
     const int64_t most = device_sm_count() > select_ctas ? device_sm_count() - select_ctas : 1;
     if (blocks > most) blocks = most;
     return cuda_ok(launch_dependent(cache_rows_kernel, dim3((unsigned)blocks), dim3(kCompactWarpsPerBlock * 32), 0, stream, 1,
-                                    layer_ptrs(Knew, Vnew, Kd, Vd, n_layers), layer_ptrs(Ks, Vs, Kd, Vd, n_layers), n_layers,
-                                    (int32_t)n_new, dst0, SL, idx, (int32_t)keep, d_model / 8, SLd, select_ctas > 0 ? 1 : 0));
+                                    layer_ptrs(Knew, Vnew, Kd, Vd, n_layers), layer_ptrs(Ks, Vs, Kd, Vd, n_layers), (uint32_t)n_layers,
+                                    (uint32_t)n_new, dst0, SL, idx, (uint32_t)keep, (uint32_t)cpr, SLd, select_ctas > 0 ? 1 : 0));
 }
 
 // `work`: three zeroed 32-bit words of device memory (the step's workspace header) - then the

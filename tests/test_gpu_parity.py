@@ -493,16 +493,19 @@ def test_cache_update_entry_point_over_chunks(chunk, cap, n_sink):
     assert n_pruned >= 3
 
 
-@pytest.mark.parametrize("cap,chunk", [
-    (1000, 200),                # one selecting CTA
-    (24576 + 16 + 129, 129),    # one candidate more than it takes: two
-    (60001, 700),               # four
-    (363001, 800),              # more candidates than a cluster holds: the streaming selection
+@pytest.mark.parametrize("cap,chunk,N", [
+    (1000, 200, 1),                # one selecting CTA
+    (24576 + 16 + 129, 129, 1),    # one candidate more than it takes: two
+    (60001, 700, 1),               # four
+    (363001, 800, 1),              # more candidates than a cluster holds: the streaming selection
+    # rows of 8, 24, 56 and 200 sixteen-byte units: the 192-unit batches of the row copies hold whole rows, end inside
+    # one, or are shorter than one; one row kept or new
+    (97, 96, 1), (131, 1, 3), (700, 333, 7), (777, 100, 25), (24, 23, 25), (1500, 1, 7),
 ])
-def test_cache_updates_without_a_synchronisation_between_them(cap, chunk):
+def test_cache_updates_without_a_synchronisation_between_them(cap, chunk, N):
     """Three updates of a full cache enqueued back to back: each one's selection, copies and head overlap, and the
     next one starts behind them.  Against the oracle's selection on the scores the head gives for the same rows."""
-    N, D, n_layers, n_sink = 1, 64, 2, 16
+    D, n_layers, n_sink = 64, 2, 16
     g = torch.Generator(device="cuda").manual_seed(cap)
     rows = lambda n: torch.randn(n, N, D, generator=g, device="cuda").to(torch.bfloat16)
     w = [torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16) / 8 for s in ((64, 3 * N * D), (64,), (12, 64), (12,))]
