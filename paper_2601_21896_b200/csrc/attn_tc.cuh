@@ -311,8 +311,8 @@ __device__ __forceinline__ float tile_max(const uint32_t (&sr)[64]) {
     }
     return fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
 }
-__device__ __forceinline__ float final_lse(float m, float scale, float l) {
-    return l > 0.f ? __fadd_rn(__fmul_rn(m, scale), logf(l)) : -INFINITY;
+__device__ __forceinline__ float final_lse(float m, float scale, float l) {      // one rounding, the same bits wherever it is inlined
+    return l > 0.f ? __fmaf_rn(m, scale, logf(l)) : -INFINITY;
 }
 
 // GATHER = false: the retained keys/values are the rows of a compacted cache (mKc, mVc are tiled

@@ -661,6 +661,31 @@ def test_attention_work_split(N, D, Lq, nB):
     np.testing.assert_allclose(LSE.cpu().numpy(), want_lse, rtol=1e-5, atol=1e-5)
 
 
+@pytest.mark.parametrize("nB", [2, 64 * 300])                  # one CTA; merged from the pieces of many
+@pytest.mark.parametrize("D", [64, 128])
+def test_lse_is_rounded_once(D, nB):
+    """LSE = m scale + log l is one fused operation: nB equal keys and integer logits give exact maxima and sums, so the
+    result is off by its own rounding (half a unit) and logf's (at most one unit of log l), and not by a rounding of m scale as
+    well.  The scale is one whose product with log2 e is exactly 1/8, so that every probability is 1."""
+    Lq, N = 300, 2
+    log2e = np.float32(1.4426950408889634)
+    s0 = np.float32(0.125 / 1.4426950408889634)
+    scale = next(s for s in (s0, np.nextafter(s0, np.float32(1)), np.nextafter(s0, np.float32(0))) if s * log2e == np.float32(0.125))
+    rng = np.random.default_rng(D + nB)
+    q = rng.integers(0, 200, (Lq, N, D)).astype(np.float32)     # at most 8 bits: exact in bf16, dot products exact in 32 bits
+    Q = to_device_bf16(wl.f32_to_bf16_bits(q))
+    K = torch.ones((nB, N, D), dtype=torch.bfloat16, device="cuda")
+    shape = pafu.Shape(N, D, None, [0, Lq])
+    ws = torch.zeros(pafu.pafu_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    O, LSE = torch.empty_like(Q), torch.empty((N, Lq), device="cuda")
+    pafu.pafu_chunk_attn(Q, K, K, [0, nB], None, None, shape, float(scale), O, LSE, ws)
+    assert pafu.pafu_workspace_status(ws) == 0
+    want = q.sum(2).T.astype(np.float64) * float(scale) + np.log(float(nB))
+    bound = 0.5 * np.spacing(want.astype(np.float32)).astype(np.float64) * 1.0001 + np.spacing(np.float32(np.log(nB)))
+    err = np.abs(LSE.cpu().numpy().astype(np.float64) - want)
+    assert np.all(err <= bound), (err / bound).max()
+
+
 # ------------------------------------------------------------- teacher salience (Eq. 4, Eq. 5)
 @pytest.mark.parametrize("L,N,LB", [
     (700, 2, 200),      # four blocks, the last one half length; every tile ragged
