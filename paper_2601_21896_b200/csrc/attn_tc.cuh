@@ -849,12 +849,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
 // Merges the partials of every item that was split across CTAs.  The host walks the CTAs'
 // shares once per launch and passes the work as a table: item i was begun by CTA cta[first]
 // (its last run, stored as that CTA's piece 1) and continued by the following entries (each
-// CTA's first run, piece 0), in key order.  A warp takes eight rows and every `lanes`-th piece of
-// them; `lanes` (2, 4 or 8: the host's choice by the longest list) warps share the rows and
-// their sums are added in warp order, which keeps the result deterministic.  The pieces come from
-// L2, a trip of about a microsecond, so they are fetched side by side: with a warp walking all
-// pieces of its rows one after the other an item of 37 pieces took 67 us.
-constexpr int kMergeRows = 8;
+// CTA's first run, piece 0), in key order.  Sums are formed in a fixed order, which keeps the result
+// deterministic.  Bound by the pieces' way through L2: two kernels, by how many pieces the longest item has.
 constexpr int kMergeThreads = 256;
 constexpr int kMergeWarps = kMergeThreads / 32;
 struct MergeItem {
@@ -865,110 +861,184 @@ struct MergeItem {
 };
 struct MergeTable {
     int32_t n_items;
-    int32_t lanes;             // warps that share a group of rows
+    int32_t longest;           // most pieces of an item
     MergeItem item[kMaxGrid];
     int16_t cta[2 * kMaxGrid];
 };
+__device__ __forceinline__ const float* merge_piece(const MergeTable& tb, const MergeItem& it, const float* pieces, int i, int piece_floats) {
+    return pieces + ((size_t)tb.cta[it.first + i] * 2 + (i == 0 ? 1 : 0)) * piece_floats;
+}
+__device__ __forceinline__ float4 ld_f4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 fmax4(float4 a, float4 b) {
+    return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), fmaxf(a.w, b.w));
+}
+__device__ __forceinline__ float4 merge_weights(float4 m, float4 M, float sl2) {
+    return make_float4(fast_exp2((m.x - M.x) * sl2), fast_exp2((m.y - M.y) * sl2), fast_exp2((m.z - M.z) * sl2), fast_exp2((m.w - M.w) * sl2));
+}
+__device__ __forceinline__ void fma4(float4& acc, float4 w, float4 v) {
+    acc.x = __fmaf_rn(w.x, v.x, acc.x); acc.y = __fmaf_rn(w.y, v.y, acc.y); acc.z = __fmaf_rn(w.z, v.z, acc.z); acc.w = __fmaf_rn(w.w, v.w, acc.w);
+}
 
+// Few pieces: such a problem has so many items that their rows alone fill the GPU.  A block takes 32 rows, a warp an eighth of
+// the columns, a lane four rows of every fourth of those, so that a column's rows are read as whole 128-byte
+// lines; the pieces follow one another.  (Groups of eight rows, 32 bytes of a line at a time, pieces shared out between two
+// warps: 12 heads x 1764 queries x 2595 keys, 84 items of two or three pieces,
+// 15.6 us, now 8.6; 4 streams x 40 heads of the 14B-class layer 19.8 and 10.5.  With up to 20 pieces here 12 heads x 4680 keys x
+// 256 queries, 12 pieces an item, take 13.0 us instead of 7.2.)
 // OUT = false: only the log-sum-exps are merged (attn_stats_kernel's pieces hold nothing else).
+constexpr int kFewPieces = 8;
+constexpr int kFewRows = 32;
 template <int D, bool OUT>
 __global__ void __launch_bounds__(kMergeThreads)
-attn_tc_merge_kernel(const __grid_constant__ MergeTable tb, const float* __restrict__ pieces, float scale,
-                     int n_heads, int64_t total_Lq, uint16_t* __restrict__ O, float* __restrict__ LSE) {
-    constexpr int kD = D;
+attn_tc_merge_few_kernel(const __grid_constant__ MergeTable tb, const float* pieces, float scale,
+                         int n_heads, int64_t total_Lq, uint16_t* O, float* LSE) {
     constexpr int kPieceFloats = HeadDims<D>::kPieceFloats;
-    constexpr int kVec = kD / 4;                                       // float4 per row of the output
-    constexpr int kPitch = OUT ? kD + 4 : 4;                           // floats: 16-byte rows, four of them half the banks apart
+    constexpr int kCols = D / kMergeWarps / 4;                         // columns of a lane
+    __shared__ float part[OUT ? kFewRows : 1][OUT ? D + 1 : 1];        // odd pitch: the lanes' four rows and columns hit 32 banks
+    grid_dep_wait();
+    constexpr int kBlocks = 2 * kBM / kFewRows;
+    const MergeItem& it = tb.item[blockIdx.x / kBlocks];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b0 = (blockIdx.x % kBlocks) * kFewRows;                  // rows of the item (slot * 128 + row of the slot)
+    if (b0 >= it.rows) return;                                         // block-uniform
+    const int n_pieces = it.n_pieces;
+    const float sl2 = scale * 1.4426950408889634f;
+    const int rs = (lane & 7) * 4, col = warp * (D / kMergeWarps) + (lane >> 3);
+    float4 M = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+#pragma unroll 4
+    for (int i = 0; i < n_pieces; ++i) M = fmax4(M, ld_f4(merge_piece(tb, it, pieces, i, kPieceFloats) + 2 * kBM * D + b0 + rs));
+    float4 L = make_float4(0.f, 0.f, 0.f, 0.f), acc[OUT ? kCols : 1];
+#pragma unroll
+    for (int k = 0; k < (OUT ? kCols : 1); ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int i = 0; i < n_pieces; ++i) {
+        const float* piece = merge_piece(tb, it, pieces, i, kPieceFloats) + b0 + rs;
+        float4 v[OUT ? kCols : 1];
+        if (OUT) {
+#pragma unroll
+            for (int k = 0; k < kCols; ++k) v[k] = ld_f4(piece + (size_t)(col + 4 * k) * (2 * kBM));
+        }
+        const float4 w = merge_weights(ld_f4(piece + 2 * kBM * D), M, sl2);
+        fma4(L, w, ld_f4(piece + 2 * kBM * D + 2 * kBM));
+        if (OUT) {
+#pragma unroll
+            for (int k = 0; k < kCols; ++k) fma4(acc[k], w, v[k]);
+        }
+    }
+    const float Mr[4] = {M.x, M.y, M.z, M.w}, Lr[4] = {L.x, L.y, L.z, L.w};
+    if (OUT) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float inv = (Lr[q] > 0.f) ? 1.0f / Lr[q] : 0.f;
+#pragma unroll
+            for (int k = 0; k < kCols; ++k)
+                part[rs + q][col + 4 * k] = (q == 0 ? acc[k].x : q == 1 ? acc[k].y : q == 2 ? acc[k].z : acc[k].w) * inv;
+        }
+    }
+    if (LSE != nullptr && warp == 0 && lane < 8) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (b0 + rs + q < it.rows) LSE[(int64_t)it.head * total_Lq + it.o_row + b0 + rs + q] = final_lse(Mr[q], scale, Lr[q]);
+    }
+    if (OUT) {
+        __syncthreads();
+        for (int r = warp; r < kFewRows && b0 + r < it.rows; r += kMergeWarps) {
+            uint32_t* dst = reinterpret_cast<uint32_t*>(O + (((int64_t)it.o_row + b0 + r) * n_heads + it.head) * D);
+#pragma unroll
+            for (int h = 0; h < D / 64; ++h) dst[h * 32 + lane] = pack_bf16(part[r][h * 64 + 2 * lane], part[r][h * 64 + 2 * lane + 1]);
+        }
+    }
+}
+
+// Many pieces: a few items cut up over dozens of CTAs.  A block takes eight rows, each of its eight warps every eighth
+// piece of them, and the warps' sums are added in warp order: the pieces come from L2, a trip of about a microsecond, so
+// they are fetched side by side (with a warp walking all pieces of its rows one after the other an item of 37 pieces took
+// 67 us).  Four blocks an SM fit with d_head 64 without spills (7.4 -> 6.2 us at 11 pieces); with 128 they cost one (7.2 -> 8.4).
+constexpr int kMergeRows = 8;
+static_assert(kMergeRows == kMergeWarps, "each warp finishes one row");
+template <int D, bool OUT>
+__global__ void __launch_bounds__(kMergeThreads, D == 64 ? 4 : 3)
+attn_tc_merge_kernel(const __grid_constant__ MergeTable tb, const float* pieces, float scale,
+                     int n_heads, int64_t total_Lq, uint16_t* O, float* LSE) {
+    constexpr int kPieceFloats = HeadDims<D>::kPieceFloats;
+    constexpr int kVec = D / 4;                                        // float4 per row of the output
+    constexpr int kPitch = OUT ? D + 4 : 4;                            // floats: 16-byte rows, four of them half the banks apart
     __shared__ __align__(16) float part[kMergeWarps][kMergeRows][kPitch];
     __shared__ float part_l[kMergeWarps][kMergeRows];
     grid_dep_wait();
-    const int lanes = tb.lanes, blocks_per_item = 4 * lanes;
-    const MergeItem& it = tb.item[blockIdx.x / blocks_per_item];
+    constexpr int kBlocks = 2 * kBM / kMergeRows;
+    const MergeItem& it = tb.item[blockIdx.x / kBlocks];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int group = warp / lanes, pl = warp % lanes;
-    const int rows_per_block = kMergeRows * kMergeWarps / lanes;
-    const int b0 = (blockIdx.x % blocks_per_item) * rows_per_block;    // rows of the item (slot * 128 + row of the slot)
+    const int b0 = (blockIdx.x % kBlocks) * kMergeRows;                // rows of the item (slot * 128 + row of the slot)
     if (b0 >= it.rows) return;                                         // block-uniform
-    const int r0 = b0 + group * kMergeRows;
     const int n_pieces = it.n_pieces;
     const float sl2 = scale * 1.4426950408889634f;
     const int rs = (lane & 1) * 4, d0 = lane >> 1;                     // this lane's four rows, and its columns d0 + 16 k
-    auto piece_at = [&](int i) { return pieces + ((size_t)tb.cta[it.first + i] * 2 + (i == 0 ? 1 : 0)) * kPieceFloats; };
-    auto f4 = [](const float* p) { return *reinterpret_cast<const float4*>(p); };
     // the rows' maxima over all pieces (every warp for itself, a lane pair per piece)
     float4 M = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-    for (int i = d0; i < n_pieces; i += 16) {
-        const float4 m = f4(piece_at(i) + 2 * kBM * kD + r0 + rs);
-        M.x = fmaxf(M.x, m.x); M.y = fmaxf(M.y, m.y); M.z = fmaxf(M.z, m.z); M.w = fmaxf(M.w, m.w);
-    }
+    for (int i = d0; i < n_pieces; i += 16) M = fmax4(M, ld_f4(merge_piece(tb, it, pieces, i, kPieceFloats) + 2 * kBM * D + b0 + rs));
 #pragma unroll
-    for (int o = 16; o > 1; o >>= 1) {
-        M.x = fmaxf(M.x, __shfl_xor_sync(0xffffffffu, M.x, o)); M.y = fmaxf(M.y, __shfl_xor_sync(0xffffffffu, M.y, o));
-        M.z = fmaxf(M.z, __shfl_xor_sync(0xffffffffu, M.z, o)); M.w = fmaxf(M.w, __shfl_xor_sync(0xffffffffu, M.w, o));
-    }
+    for (int o = 16; o > 1; o >>= 1)
+        M = fmax4(M, make_float4(__shfl_xor_sync(0xffffffffu, M.x, o), __shfl_xor_sync(0xffffffffu, M.y, o),
+                                 __shfl_xor_sync(0xffffffffu, M.z, o), __shfl_xor_sync(0xffffffffu, M.w, o)));
     // this warp's pieces
-    float4 L = make_float4(0.f, 0.f, 0.f, 0.f), acc[OUT ? kD / 16 : 1];
+    float4 L = make_float4(0.f, 0.f, 0.f, 0.f), acc[OUT ? D / 16 : 1];
 #pragma unroll
-    for (int k = 0; k < (OUT ? kD / 16 : 1); ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = pl; i < n_pieces; i += lanes) {
-        const float* piece = piece_at(i) + r0 + rs;
-        const float4 m = f4(piece + 2 * kBM * kD), l = f4(piece + 2 * kBM * kD + 2 * kBM);
-        float4 v[OUT ? kD / 16 : 1];
+    for (int k = 0; k < (OUT ? D / 16 : 1); ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = warp; i < n_pieces; i += kMergeWarps) {
+        const float* piece = merge_piece(tb, it, pieces, i, kPieceFloats) + b0 + rs;
+        const float4 m = ld_f4(piece + 2 * kBM * D), l = ld_f4(piece + 2 * kBM * D + 2 * kBM);
+        float4 v[OUT ? D / 16 : 1];
         if (OUT) {
 #pragma unroll
-            for (int k = 0; k < kD / 16; ++k) v[k] = f4(piece + (size_t)(k * 16 + d0) * (2 * kBM));
+            for (int k = 0; k < D / 16; ++k) v[k] = ld_f4(piece + (size_t)(k * 16 + d0) * (2 * kBM));
         }
-        const float wx = fast_exp2((m.x - M.x) * sl2), wy = fast_exp2((m.y - M.y) * sl2);
-        const float wz = fast_exp2((m.z - M.z) * sl2), ww = fast_exp2((m.w - M.w) * sl2);
-        L.x = __fmaf_rn(wx, l.x, L.x); L.y = __fmaf_rn(wy, l.y, L.y); L.z = __fmaf_rn(wz, l.z, L.z); L.w = __fmaf_rn(ww, l.w, L.w);
+        const float4 w = merge_weights(m, M, sl2);
+        fma4(L, w, l);
         if (OUT) {
 #pragma unroll
-            for (int k = 0; k < kD / 16; ++k) {
-                acc[k].x += wx * v[k].x; acc[k].y += wy * v[k].y; acc[k].z += wz * v[k].z; acc[k].w += ww * v[k].w;
-            }
+            for (int k = 0; k < D / 16; ++k) fma4(acc[k], w, v[k]);
         }
     }
     if (OUT) {
 #pragma unroll
-        for (int k = 0; k < kD / 16; ++k) {
+        for (int k = 0; k < D / 16; ++k) {
             part[warp][rs + 0][k * 16 + d0] = acc[k].x; part[warp][rs + 1][k * 16 + d0] = acc[k].y;
             part[warp][rs + 2][k * 16 + d0] = acc[k].z; part[warp][rs + 3][k * 16 + d0] = acc[k].w;
         }
     }
     if (d0 == 0) { part_l[warp][rs + 0] = L.x; part_l[warp][rs + 1] = L.y; part_l[warp][rs + 2] = L.z; part_l[warp][rs + 3] = L.w; }
     __syncthreads();
-    // the warps of a group share its rows out again
-    const int n_sum = n_pieces < lanes ? n_pieces : lanes;
-#pragma unroll
-    for (int q = 0; q < kMergeRows; ++q) {
-        const int row = r0 + q;
-        if (q * lanes / kMergeRows != pl || row >= it.rows) continue;  // warp-uniform
-        const float mj = (q & 3) == 0 ? M.x : (q & 3) == 1 ? M.y : (q & 3) == 2 ? M.z : M.w;
-        const float Mr = __shfl_sync(0xffffffffu, mj, q >> 2);         // an even lane holds rows 0..3, an odd one 4..7
-        float Ls = 0.f;
-        float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int w = group * lanes; w < group * lanes + n_sum; ++w) {
-            Ls += part_l[w][q];
-            if (OUT && lane < kVec) {
-                const float4 x = f4(&part[w][q][lane * 4]);
-                o4.x += x.x; o4.y += x.y; o4.z += x.z; o4.w += x.w;
-            }
-        }
+    // each warp finishes one row
+    const int row = b0 + warp;
+    if (row >= it.rows) return;
+    const int q = warp & 3;
+    const float Mr = __shfl_sync(0xffffffffu, q == 0 ? M.x : q == 1 ? M.y : q == 2 ? M.z : M.w, warp >> 2);   // lane 0 holds rows 0..3, lane 1 4..7
+    const int n_sum = n_pieces < kMergeWarps ? n_pieces : kMergeWarps;
+    float Ls = 0.f;
+    float4 o4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int w = 0; w < n_sum; ++w) {
+        Ls += part_l[w][warp];
         if (OUT && lane < kVec) {
-            const float inv = (Ls > 0.f) ? 1.0f / Ls : 0.f;
-            uint2 o;
-            o.x = pack_bf16(o4.x * inv, o4.y * inv);
-            o.y = pack_bf16(o4.z * inv, o4.w * inv);
-            *reinterpret_cast<uint2*>(O + (((int64_t)it.o_row + row) * n_heads + it.head) * kD + lane * 4) = o;
+            const float4 x = ld_f4(&part[w][warp][lane * 4]);
+            o4.x += x.x; o4.y += x.y; o4.z += x.z; o4.w += x.w;
         }
-        if (LSE != nullptr && lane == 0) LSE[(int64_t)it.head * total_Lq + it.o_row + row] = final_lse(Mr, scale, Ls);
     }
+    if (OUT && lane < kVec) {
+        const float inv = (Ls > 0.f) ? 1.0f / Ls : 0.f;
+        uint2 o;
+        o.x = pack_bf16(o4.x * inv, o4.y * inv);
+        o.y = pack_bf16(o4.z * inv, o4.w * inv);
+        *reinterpret_cast<uint2*>(O + (((int64_t)it.o_row + row) * n_heads + it.head) * D + lane * 4) = o;
+    }
+    if (LSE != nullptr && lane == 0) LSE[(int64_t)it.head * total_Lq + it.o_row + row] = final_lse(Mr, scale, Ls);
 }
 
 // Host side of the merge: which CTAs hold the pieces of which item.
 inline void build_merge_table(const Params& p, int n_cta, MergeTable& tb) {
     tb.n_items = 0;
-    int n_list = 0, longest = 0;
+    tb.longest = 0;
+    int n_list = 0;
     Seg g, last;
     for (int b = 0; b < n_cta; ++b) {
         bool have = false;
@@ -993,10 +1063,8 @@ inline void build_merge_table(const Params& p, int n_cta, MergeTable& tb) {
             tb.cta[n_list++] = (int16_t)c;
         }
         it.n_pieces = (int16_t)(n_list - it.first);
-        if (it.n_pieces > longest) longest = it.n_pieces;
+        if (it.n_pieces > tb.longest) tb.longest = it.n_pieces;
     }
-    // items of a large problem have two or three pieces and there are enough of them to fill the GPU
-    tb.lanes = longest <= 4 ? 2 : (longest <= 8 ? 4 : 8);
 }
 
 inline int sm_count() { return device_sm_count(); }
@@ -1033,7 +1101,9 @@ inline pafu_status launch_merge(const Params& p, int grid, int32_t n_heads, cuda
     MergeTable tb;
     build_merge_table(p, grid, tb);
     if (tb.n_items == 0) return PAFU_OK;
-    return cuda_ok(launch_dependent(attn_tc_merge_kernel<D, OUT>, dim3(tb.n_items * 4 * tb.lanes), dim3(kMergeThreads), 0, stream, 1,
+    const bool few = tb.longest <= kFewPieces;
+    return cuda_ok(launch_dependent(few ? attn_tc_merge_few_kernel<D, OUT> : attn_tc_merge_kernel<D, OUT>,
+                                    dim3(tb.n_items * (2 * kBM / (few ? kFewRows : kMergeRows))), dim3(kMergeThreads), 0, stream, 1,
                                     tb, (const float*)p.pieces, p.scale, (int)n_heads, p.total_Lq, p.O, p.LSE));
 }
 

@@ -638,11 +638,13 @@ def test_step_indexed_equals_step(w):
 
 
 @pytest.mark.parametrize("N,D,Lq,nB", [
-    (1, 128, 1, 1), (2, 64, 64, 128), (3, 128, 129, 500),     # whole items, one round, nothing to merge
-    (1, 128, 130, 64 * 40 + 1), (1, 64, 300, 64 * 40 - 1),    # one long item over many CTAs: eight merging warps
-    (2, 128, 257, 64 * 20 + 5),                               # a one-row tail item; four to eight pieces
-    (3, 128, 2000, 64 * 9),                                   # pieces of two or three shares
+    (1, 128, 1, 1), (2, 64, 64, 128),                         # whole items, one round, nothing to merge
+    (3, 128, 129, 500),                                       # 11 tiles an item, one tile a CTA: 11 pieces
+    (1, 128, 130, 64 * 40 + 1), (1, 64, 300, 64 * 40 - 1),    # one or two items over many CTAs: about 40 pieces
+    (2, 128, 257, 64 * 20 + 5),                               # a one-row tail item; over 20 pieces
+    (3, 128, 2000, 64 * 9),                                   # seven pieces: the merge for few pieces
     (40, 128, 1100, 100),                                     # more items than CTAs: a whole round, then shares
+    (6, 64, 1900, 700), (30, 64, 515, 900),                   # d_head 64: two to four pieces, a three-row tail item
 ])
 def test_attention_work_split(N, D, Lq, nB):
     """The ways a problem is handed to the CTAs (whole items, shares, a round of whole items followed by shares) and
