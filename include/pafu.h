@@ -128,7 +128,7 @@ pafu_status pafu_workspace_status(const void* ws, void* stream);
  * (32-row group, 64-key tile):
  *   counts[0]  tiles that took the exact pass because they open a run or end a key segment raggedly
  *   counts[1]  tiles that took the exact pass because a row sum showed a logit far above the
- *              running maximum, or because their run has at most four tiles
+ *              running maximum
  *   counts[2]  tiles at which the output accumulator and the row sums were rescaled
  * counts is a HOST array of 3 entries.  Tests use it to show that an input reaches those paths.
  *

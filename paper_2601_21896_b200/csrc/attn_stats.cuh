@@ -145,7 +145,6 @@ attn_stats_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant_
             if (slot >= g.n_slots) continue;
             float m_used = -INFINITY, l_sum = 0.f;
             const int n = g.t1 - g.t0;
-            const bool short_run = n <= kShortRun;
             const int rag = (g.nB % kBN) != 0 ? g.nt - 1 - g.t0 : -1, lim = (int)(g.nB % kBN);   // the segment's ragged last tile
 #pragma unroll 1
             for (int i = 0; i < n; ++i, ++tc) {
@@ -161,7 +160,7 @@ attn_stats_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant_
                 __syncwarp();
                 if (lane == 0) mbar_arrive(s_empty(slot, buf));
                 const int left = i == rag ? lim : kBN;
-                bool full_pass = (i == 0) || (left < kBN) || short_run;
+                bool full_pass = (i == 0) || (left < kBN);
                 if (!full_pass) {
                     const float rs = tile_sum(sr, sl2_2, -m_used * sl2);
                     full_pass = __any_sync(0xffffffffu, !(rs < kSumTrigger));    // also true for inf / NaN
@@ -175,7 +174,7 @@ attn_stats_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant_
                     const float mx = tile_max(sr);
                     if (i == 0) {
                         m_used = mx;
-                    } else if (__any_sync(0xffffffffu, (mx - m_used) * sl2 > (short_run ? 0.f : kRescaleThresholdLog2))) {
+                    } else if (__any_sync(0xffffffffu, (mx - m_used) * sl2 > kRescaleThresholdLog2)) {
                         const float m_new = fmaxf(m_used, mx);
                         l_sum = __fmul_rn(l_sum, fast_exp2((m_used - m_new) * sl2));
                         m_used = m_new;

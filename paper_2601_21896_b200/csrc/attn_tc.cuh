@@ -34,11 +34,14 @@
 //
 // Online softmax with lazy rescaling: the running maximum only moves when the new tile
 // exceeds it by more than 2^8 in the exponent, so the O accumulator is rarely rescaled; when
-// it is, the slot's own softmax warps do it after waiting for the previous P V product.
+// it is, the slot's own softmax warps do it after waiting for the previous P V product.  Small problems
+// hand the tensor core P's rounding error as well (round_mode()).
 //
 // Every mbarrier wait is bounded.  A wait that runs out sets the status word, raises a CTA-wide
 // abort flag, and all roles fall through to the common exit where TMEM is released.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -58,10 +61,6 @@ constexpr int kTileBytes = kBN * kD * 2;      // 16 KiB: one K or V tile
 constexpr int kHalfBytes = kTileBytes / 2;    // one [64 rows x 64 cols] swizzled half
 constexpr int kSmemBytes = 2 * kQBytes + kStages * kTileBytes + 1024 /*align*/ + 512 /*barriers*/;
 constexpr float kRescaleThresholdLog2 = 8.0f;
-// Runs this short follow the true maximum in every tile: a small problem's peaked rows then have their
-// largest probability at exactly 1, which bf16 represents (relative error 1.8e-3 instead of 2.1e-3 on rows of logits
-// twice as wide as normal), and a few tiles cost little.
-constexpr int kShortRun = 4;
 constexpr float kSumTrigger = 65536.0f;   // a 64-key row sum this large means some p exceeded 2^10
 // Register re-balancing.  With 384 threads the kernel launches with 168 registers per thread.
 // setmaxnreg.inc blocks until the registers exist, so what the third warpgroup gives up must
@@ -279,11 +278,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
+// what rounding (lo, hi) to the bf16 pair `rounded` left over, as a bf16 pair
+__device__ __forceinline__ uint32_t pack_rest(float lo, float hi, uint32_t rounded) {
+    return pack_bf16(lo - __uint_as_float(rounded << 16), hi - __uint_as_float(rounded & 0xffff0000u));
+}
 
 // The pieces of a tile's softmax that attn_stats_kernel shares, so that both form the same bits.
 // Row sum of 2^(s * scale log2 e + mb) over 64 logits; `pk` (32 words), if given, receives the
-// probabilities as bf16 pairs.
-__device__ __forceinline__ float tile_sum(const uint32_t (&sr)[64], uint64_t sl2_2, float mb, uint32_t* pk = nullptr) {
+// probabilities as bf16 pairs, and `lo` what that rounding leaves over.
+__device__ __forceinline__ float tile_sum(const uint32_t (&sr)[64], uint64_t sl2_2, float mb, uint32_t* pk = nullptr, uint32_t* lo = nullptr) {
     const uint64_t mb_2 = pack2(__float_as_uint(mb), __float_as_uint(mb));
     uint64_t rs2[2] = {0ull, 0ull};
 #pragma unroll
@@ -293,6 +296,7 @@ __device__ __forceinline__ float tile_sum(const uint32_t (&sr)[64], uint64_t sl2
         const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
         rs2[c & 1] = fadd2(rs2[c & 1], pack2(__float_as_uint(p0), __float_as_uint(p1)));
         if (pk != nullptr) pk[c] = pack_bf16(p0, p1);
+        if (lo != nullptr) lo[c] = pack_rest(p0, p1, pk[c]);
     }
     float r0, r1, r2, r3;
     unpack2(rs2[0], r0, r1);
@@ -331,7 +335,15 @@ struct HeadDims {
     static constexpr int kPieceFloats = 2 * kBM * D + 2 * 2 * kBM;   // one partial: O [D][256], m [256], l [256]
 };
 
-template <bool GATHER, int D>
+// ROUND: how P's rounding is kept small where that matters (round_mode() decides).
+//   kRoundPlain    P as one bf16 operand, relative to the lazy running maximum
+//   kRoundSplit    P as two, its rounded value and what rounding left over (the second half of the S buffer, whose
+//                  logits are in registers by then)
+//   kRoundOpening  as two in the tiles that open a run
+constexpr int kRoundPlain = 0, kRoundSplit = 1, kRoundOpening = 2;
+constexpr int kOpeningTiles = 2;
+
+template <bool GATHER, int D, int ROUND>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mKc,
                const __grid_constant__ CUtensorMap mVc, const __grid_constant__ CUtensorMap mKq,
@@ -578,13 +590,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 elect_commit(s_full(slot, buf));
                 elect_commit(kv_empty(stage));
             };
-            auto issue_pv = [&](int buf, int stage, bool first) {   // O += P[buf] V, K = 64 keys
+            auto issue_pv = [&](int buf, int stage, bool first, auto split) {   // O += P[buf] V, K = 64 keys
                 if constexpr (D == 64) {
                     if (leader) {
 #pragma unroll
                         for (int kk = 0; kk < kBN / 16; ++kk)
                             umma_ts(tOslot, tSslot + buf * kBN + kk * 8, desc_v + ((sKV + stage * kTileBytes) >> 4) + kk * (2048 >> 4),
                                     idesc_pv, !(first && kk == 0));
+                        if constexpr (decltype(split)::value) {
+#pragma unroll
+                            for (int kk = 0; kk < kBN / 16; ++kk)
+                                umma_ts(tOslot, tSslot + buf * kBN + 32 + kk * 8, desc_v + ((sKV + stage * kTileBytes) >> 4) + kk * (2048 >> 4),
+                                        idesc_pv, true);
+                        }
                         umma_commit(kv_empty(stage));
                     }
                     __syncwarp();
@@ -592,6 +610,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 }
                 if constexpr (GATHER) fence_proxy_async_smem();
                 umma_ts_x4(tOslot, tSslot + buf * kBN, lo_v + stage * (kTileBytes >> 4), idesc_pv, hi, !first);
+                if constexpr (decltype(split)::value) umma_ts_x4(tOslot, tSslot + buf * kBN + 32, lo_v + stage * (kTileBytes >> 4), idesc_pv, hi, 1);
                 elect_commit(kv_empty(stage));
             };
             bool ok = true;
@@ -636,34 +655,43 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     ck.step(2);
                 }
                 if (n == 1) ck.step(2);                              // keep ck two tiles ahead of cv
+                // tiles [i0, i1) of the run; split: P is carried in two operands
+                auto tiles = [&](int i0, int i1, auto split) {
 #pragma unroll 1
-                for (int i = 0; i < n && ok; ++i) {
-                    const int buf = (tc + i) & 1;
-                    const bool more = i + 2 < n;
-                    wait(kv_full(cv.st), cv.ph, 203);
-                    if (!ok) break;
-                    wait(p_full(slot, buf), ((tc + i) >> 1) & 1u, 205);
-                    if (!ok) break;
-                    // The slots take turns at the tensor core, a tile's P V and the next Q K^T at a time: left
-                    // alone they fall into step, their MMAs interleave one by one and then both wait (some CTAs
-                    // 690k clocks, most 800k; with turns 727k on all).  The turn is handed on before the
-                    // last block of Q K^T so that the other slot's MMAs queue up behind it without a gap.
-                    if (two) {
-                        wait(turn(slot), (turns & 1u) ^ (slot == 0 ? 1u : 0u), 207);
+                    for (int i = i0; i < i1 && ok; ++i) {
+                        const int buf = (tc + i) & 1;
+                        const bool more = i + 2 < n;
+                        wait(kv_full(cv.st), cv.ph, 203);
                         if (!ok) break;
-                        ++turns;
+                        wait(p_full(slot, buf), ((tc + i) >> 1) & 1u, 205);
+                        if (!ok) break;
+                        // The slots take turns at the tensor core, a tile's P V and the next Q K^T at a time: left
+                        // alone they fall into step, their MMAs interleave one by one and then both wait (some CTAs
+                        // 690k clocks, most 800k; with turns 727k on all).  The turn is handed on before the
+                        // last block of Q K^T so that the other slot's MMAs queue up behind it without a gap.
+                        if (two) {
+                            wait(turn(slot), (turns & 1u) ^ (slot == 0 ? 1u : 0u), 207);
+                            if (!ok) break;
+                            ++turns;
+                        }
+                        tc_fence_after_sync();
+                        issue_pv(buf, cv.st, i == 0, split);
+                        if (more) wait(kv_full(ck.st), ck.ph, 204);
+                        if (!ok) break;
+                        if (more) issue_qk(buf, ck.st, two);            // S(i+2) reuses the buffer P(i) was read from
+                        else if (two) elect_arrive(turn(slot ^ 1));
+                        if (i + 2 == n && leader) umma_commit(pv_done(slot));     // lets the last tile's softmax know O is at rest
+                        if (i == n - 1 && leader) { umma_commit(o_done(slot)); umma_commit(q_empty(slot)); }
+                        __syncwarp();
+                        cv.step(2);
+                        ck.step(2);
                     }
-                    tc_fence_after_sync();
-                    issue_pv(buf, cv.st, i == 0);
-                    if (more) wait(kv_full(ck.st), ck.ph, 204);
-                    if (!ok) break;
-                    if (more) issue_qk(buf, ck.st, two);            // S(i+2) reuses the buffer P(i) was read from
-                    else if (two) elect_arrive(turn(slot ^ 1));
-                    if (i + 2 == n && leader) umma_commit(pv_done(slot));     // lets the last tile's softmax know O is at rest
-                    if (i == n - 1 && leader) { umma_commit(o_done(slot)); umma_commit(q_empty(slot)); }
-                    __syncwarp();
-                    cv.step(2);
-                    ck.step(2);
+                };
+                if constexpr (ROUND == kRoundOpening) {      // two loops: a branch in the long one costs every tile
+                    tiles(0, n < kOpeningTiles ? n : kOpeningTiles, std::true_type{});
+                    tiles(kOpeningTiles, n, std::false_type{});
+                } else {
+                    tiles(0, n, std::integral_constant<bool, ROUND == kRoundSplit>{});
                 }
                 tc += (uint32_t)n;
                 cur.step((2u * (uint32_t)n) % kStages);
@@ -690,7 +718,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
             if (slot >= g.n_slots) continue;
             float m_used = -INFINITY, l_sum = 0.f;
             const int n = g.t1 - g.t0;
-            const bool short_run = n <= kShortRun;
             uint32_t sr[64];
             bool loaded = false;                       // S(i) already requested from tensor memory
             for (int i = 0; i < n; ++i) {
@@ -712,14 +739,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 // exponentials use the running maximum as it stands.  Only when the tile's row sum
                 // shows that some logit outgrew that maximum by more than 2^10 does the tile take
                 // the full pass below (true maximum, rescale of O and of the row sum).
-                bool full_pass = (i == 0) || (left < kBN) || short_run;
+                const bool opening = i < (ROUND == kRoundOpening ? kOpeningTiles : 1);
+                bool full_pass = opening || (left < kBN);
                 if (!full_pass) {
                     const float mbf = -m_used * sl2;
                     const uint64_t mb_2 = pack2(__float_as_uint(mbf), __float_as_uint(mbf));
                     uint64_t rs2[2] = {0ull, 0ull};
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
-                        uint32_t pk[16];
+                        uint32_t pk[16], lo[ROUND == kRoundSplit ? 16 : 1];
 #pragma unroll
                         for (int q = 0; q < 16; ++q) {
                             float e0, e1;
@@ -727,8 +755,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                             const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
                             rs2[q & 1] = fadd2(rs2[q & 1], pack2(__float_as_uint(p0), __float_as_uint(p1)));
                             pk[q] = pack_bf16(p0, p1);
+                            if constexpr (ROUND == kRoundSplit) lo[q] = pack_rest(p0, p1, pk[q]);
                         }
                         PAFU_TMEM_ST_X16(tS + 16 * c, pk);
+                        if constexpr (ROUND == kRoundSplit) PAFU_TMEM_ST_X16(tS + 32 + 16 * c, lo);
                     }
                     float r0, r1, r2, r3;
                     unpack2(rs2[0], r0, r1);
@@ -742,11 +772,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                         if (c >= left) sr[c] = 0xff800000u;   // -inf
                 }
                 if (full_pass) {
-                    if ((tid & 31) == 0) atomicAdd(p.status + ((i == 0 || left < kBN) ? kStatusWordFullFirst : kStatusWordFullSum), 1);
+                    if ((tid & 31) == 0) atomicAdd(p.status + ((opening || left < kBN) ? kStatusWordFullFirst : kStatusWordFullSum), 1);
                     const float mx = tile_max(sr);
                     if (i == 0) {
                         m_used = mx;
-                    } else if (__any_sync(0xffffffffu, (mx - m_used) * sl2 > (short_run ? 0.f : kRescaleThresholdLog2))) {
+                    } else if (__any_sync(0xffffffffu, (mx - m_used) * sl2 > kRescaleThresholdLog2)) {
                         // The whole warp rescales together (TMEM accesses are warp-collective); rows
                         // whose maximum did not move get alpha = 1.  O must be at rest, i.e. the previous
                         // tile's P V product finished: S(i+1) being ready implies it (it was issued
@@ -770,9 +800,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                             PAFU_TMEM_ST_X32(tO + c * 32, orr);
                         }
                     }
-                    uint32_t pk[32];
-                    l_sum += tile_sum(sr, sl2_2, -m_used * sl2, pk);
+                    uint32_t pk[32], lo[ROUND != kRoundPlain ? 32 : 1];
+                    l_sum += tile_sum(sr, sl2_2, -m_used * sl2, pk, ROUND != kRoundPlain ? lo : nullptr);
                     PAFU_TMEM_ST_X32(tS, pk);
+                    if constexpr (ROUND != kRoundPlain) PAFU_TMEM_ST_X32(tS + 32, lo);      // read only where issue_pv is told to
                 }   // full_pass
                 if (i + 1 < n && __all_sync(0xffffffffu, mbar_test_wait(s_full(slot, buf ^ 1), ((tc + i + 1) >> 1) & 1u))) {
                     // S(i+1) is already complete: request it now, so that its trip from tensor
@@ -1077,22 +1108,48 @@ inline int sm_count() { return device_sm_count(); }
 // serial merge): 2 heads x 120 queries x 8023 keys 77 us, now 28; three ragged streams of 2 heads 31.5 and 20;
 // 24 heads x 147 queries x 268 keys 21 and 17.
 constexpr int kMergeTiles = 3, kMinShareTiles = 1;
-inline int grid_for(const StreamTable& st, int n_heads, int has_chunk, int64_t cost, int max_ctas, bool& whole) {
-    int sms = sm_count();
-    if (max_ctas > 0 && sms > max_ctas) sms = max_ctas;      // caller's scratch holds fewer partials
-    int64_t items = 0, longest = 0;
+inline int cta_limit(int max_ctas) {                         // max_ctas > 0: the caller's scratch holds fewer partials
+    const int sms = sm_count();
+    return max_ctas > 0 && sms > max_ctas ? max_ctas : sms;
+}
+inline int longest_item(const StreamTable& st, int has_chunk) {
+    int64_t longest = 0;
     for (int s = 0; s < st.n_streams; ++s) {
         const StreamCost sc = stream_cost(st, s, has_chunk);
-        if (sc.head_cost == 0) continue;
-        items += sc.nqp * n_heads;
-        if (sc.nt > longest) longest = sc.nt;
+        if (sc.head_cost > 0 && sc.nt > longest) longest = sc.nt;
+    }
+    return (int)longest;
+}
+inline int grid_for(const StreamTable& st, int n_heads, int has_chunk, int64_t cost, int max_ctas, bool& whole) {
+    const int sms = cta_limit(max_ctas);
+    int64_t items = 0;
+    for (int s = 0; s < st.n_streams; ++s) {
+        const StreamCost sc = stream_cost(st, s, has_chunk);
+        if (sc.head_cost > 0) items += sc.nqp * n_heads;
     }
     int64_t share = cost / ((int64_t)kCost2 * sms);
     if (share < kMinShareTiles) share = kMinShareTiles;
-    whole = items <= sms && longest <= share + kMergeTiles;
+    whole = items <= sms && longest_item(st, has_chunk) <= share + kMergeTiles;
     if (whole) return (int)items;
     const int64_t g = (cost + kCost2 * kMinShareTiles - 1) / (kCost2 * kMinShareTiles);
     return (int)(g < sms ? g : sms);
+}
+
+// How P is rounded.  Relative to its run's running maximum a probability is rounded to bf16, a relative error of 2^-9; only
+// the maximum itself is exact (1).  A problem cut into single tiles has an exact one in each, which shows on peaked
+// rows (logits twice as wide as normal: error 1.76e-3 in single tiles, 2.2e-3 and more in long runs; 1.66e-3 is the output's own
+// rounding).  So that leaving items whole, and shares a little longer, costs no precision, P's rounding error is carried along
+//   - in every tile below kSplitShare tiles a share: 2 heads x 600 queries x 2000 keys 1.97e-3 in pieces of a tile or two, 1.66e-3;
+//     18.7 us, 18.9 without it;
+//   - in the two tiles that open a run below kOpeningShare, and in whole items of up to kOpeningItem tiles, where carrying it
+//     everywhere would cost up to a quarter: 140 heads x 256 queries x 704 keys 2.25e-3 in pieces, 2.30e-3 whole, 2.24e-3 like this;
+//     19.8 us, 18.9 without it, 40.8 in pieces.
+// Longer runs show no difference: a piece more or less is a few exact probabilities among hundreds.
+constexpr int kSplitShare = 5, kOpeningShare = 8, kOpeningItem = 64;
+inline int round_mode(const StreamTable& st, int has_chunk, int64_t cost, int max_ctas, bool whole) {
+    const int64_t tile = (int64_t)kCost2 * cta_limit(max_ctas);     // cost of a share of one tile
+    if (cost < kSplitShare * tile) return kRoundSplit;
+    return cost < kOpeningShare * tile || (whole && longest_item(st, has_chunk) <= kOpeningItem) ? kRoundOpening : kRoundPlain;
 }
 
 template <int D, bool OUT>
@@ -1152,22 +1209,27 @@ inline pafu_status launch_d(const uint16_t* Q, const uint16_t* Kc, const uint16_
     p.O = O; p.LSE = LSE; p.status = status; p.pieces = pieces; p.idx = idx; p.Kraw = gather ? Kc : nullptr; p.Vraw = gather ? Vc : nullptr; p.total_Lq = nQ;
     static bool attr_set[kMaxDevices] = {};
     if (!once_per_device(attr_set, [] {
-            if (cudaFuncSetAttribute(attn_tc_kernel<false, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return false;
+            auto opt_in = [](auto* kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) == cudaSuccess; };
+            if (!opt_in(attn_tc_kernel<false, D, kRoundPlain>) || !opt_in(attn_tc_kernel<false, D, kRoundSplit>) ||
+                !opt_in(attn_tc_kernel<false, D, kRoundOpening>)) return false;
             if constexpr (D == 128)
-                return cudaFuncSetAttribute(attn_tc_kernel<true, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) == cudaSuccess;
+                return opt_in(attn_tc_kernel<true, 128, kRoundPlain>) && opt_in(attn_tc_kernel<true, 128, kRoundSplit>) &&
+                       opt_in(attn_tc_kernel<true, 128, kRoundOpening>);
             return true;
         }))
         return PAFU_ERR_CUDA;
     bool whole;
     const int grid = grid_for(st, n_heads, has_chunk, cost, max_ctas, whole);
     plan_shares(p, grid, cost, whole);
-    cudaError_t le;
+    const int mode = round_mode(st, has_chunk, cost, max_ctas, whole);
+    auto go = [&](auto* kernel) { return launch_dependent(kernel, dim3(grid), dim3(kThreads), kSmem, stream, 1, mQ, mKc, mVc, mKq, mVq, p); };
+    cudaError_t le = cudaSuccess;
     if constexpr (D == 128) {
-        le = gather ? launch_dependent(attn_tc_kernel<true, 128>, dim3(grid), dim3(kThreads), kSmem, stream, 1, mQ, mKc, mVc, mKq, mVq, p)
-                    : launch_dependent(attn_tc_kernel<false, 128>, dim3(grid), dim3(kThreads), kSmem, stream, 1, mQ, mKc, mVc, mKq, mVq, p);
-    } else {
-        le = launch_dependent(attn_tc_kernel<false, D>, dim3(grid), dim3(kThreads), kSmem, stream, 1, mQ, mKc, mVc, mKq, mVq, p);
+        if (gather) le = mode == kRoundPlain ? go(attn_tc_kernel<true, 128, kRoundPlain>) : mode == kRoundSplit ? go(attn_tc_kernel<true, 128, kRoundSplit>)
+                                                                                                             : go(attn_tc_kernel<true, 128, kRoundOpening>);
     }
+    if (!gather) le = mode == kRoundPlain ? go(attn_tc_kernel<false, D, kRoundPlain>) : mode == kRoundSplit ? go(attn_tc_kernel<false, D, kRoundSplit>)
+                                                                                                        : go(attn_tc_kernel<false, D, kRoundOpening>);
     if (le != cudaSuccess) return PAFU_ERR_CUDA;
     return launch_merge<D, true>(p, grid, n_heads, stream);
 }

@@ -357,6 +357,64 @@ def test_attention_run_opening_on_tiny_logits(size):
     assert c[1] > 0 and c[2] > 0
 
 
+@pytest.mark.parametrize("size", ["short", "long"])
+def test_path_counters_stay_at_zero_on_ordinary_logits(size):
+    """The control for the tests above: on N(0, 1) logits no row sum outgrows the running maximum (2^16 would take a logit
+    11 nats above the opening tile's maximum) and nothing is rescaled, however short the runs are."""
+    N, Lq, nB = PEAKED_SIZES[size]
+    c = _attention_all_entry_points(wl.peaked_attention_inputs("scaled_q", N, 128, Lq, nB, seed=9, q_scale=1.0), N, 128, Lq, nB, "control")
+    assert c[0] > 0 and c[1] == 0 and c[2] == 0, c.tolist()
+
+
+@pytest.mark.parametrize("N,D,Lq,nB,run", [
+    (2, 64, 64, 128, 1), (2, 128, 100, 300, 1),                  # one or two tiles a CTA at the finest: whole, or single tiles
+    (4, 128, 600, 2000, 3), (4, 64, 600, 2000, 3),               # shares of three tiles
+    (120, 128, 256, 300, 5), (140, 64, 256, 448, 6), (140, 128, 256, 448, 6),   # whole items of 9 and 11 tiles
+    (8, 128, 600, 2000, 7),                                      # shares of six and a half
+])
+@pytest.mark.parametrize("q_scale", [1.0, 2.0, 4.0])
+def test_attention_error_is_no_larger_than_in_pieces(N, D, Lq, nB, run, q_scale):
+    """However a small problem is handed out, its error against 64 bits is at most that of the arithmetic in which
+    items are cut into runs of `run` tiles, P is rounded to bf16 relative to its run's running maximum (the opening
+    tile's, re-based for 32 rows together by more than 2^8 only, and looked at again only where a row sum reaches 2^16 or
+    the segment ends) and the runs are added in 64 bits."""
+    g = torch.Generator(device="cuda").manual_seed(N + nB)
+    r = lambda n, s=1.0: (torch.randn(n, N, D, generator=g, device="cuda") * s).to(torch.bfloat16)
+    Q, Kc, Vc, Kq, Vq = r(Lq, q_scale), r(nB), r(nB), r(Lq), r(Lq)
+    shape = pafu.Shape(N, D, None, [0, Lq])
+    ws = torch.zeros(pafu.pafu_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    O = torch.empty_like(Q)
+    pafu.pafu_chunk_attn(Q, Kc, Vc, [0, nB], Kq, Vq, shape, 0.0, O, None, ws)
+    assert pafu.pafu_workspace_status(ws) == 0
+    edges = list(range(0, nB, 64)) + list(range(nB, nB + Lq, 64)) + [nB + Lq]
+    some = lambda x: torch.nn.functional.pad(x, (0, -Lq % 32)).view(-1, 32).any(1).repeat_interleave(32)[:Lq, None]   # x[Lq], by groups of 32 rows
+    e_got = e_cut = 0.0
+    for n in range(N):
+        k, v = torch.cat([Kc[:, n], Kq[:, n]]).double(), torch.cat([Vc[:, n], Vq[:, n]]).double()
+        z = Q[:, n].double() @ k.T * (D ** -0.5 / np.log(2.0))
+        want = torch.softmax(z * np.log(2.0), 1) @ v
+        top, o, l = z.max(1).values[:, None], 0.0, 0.0
+        for t0 in range(0, len(edges) - 1, run):
+            m, o_run, l_run = None, 0.0, 0.0
+            for t in range(t0, min(t0 + run, len(edges) - 1)):
+                zt, vt = z[:, edges[t]:edges[t + 1]], v[edges[t]:edges[t + 1]]
+                mx = zt.max(1).values[:, None]
+                if m is None:
+                    m = mx
+                else:
+                    look = some((torch.exp2(zt - m).sum(1) >= 65536)) if zt.shape[1] == 64 else torch.ones_like(mx, dtype=torch.bool)
+                    m_new = torch.where(look & some((mx - m)[:, 0] > 8), torch.maximum(mx, m), m)
+                    o_run, l_run, m = o_run * torch.exp2(m - m_new), l_run * torch.exp2(m - m_new), m_new
+                p = torch.exp2(zt - m)
+                o_run, l_run = o_run + p.to(torch.bfloat16).double() @ vt, l_run + p.sum(1, keepdim=True)
+            o, l = o + torch.exp2(m - top) * o_run, l + torch.exp2(m - top) * l_run
+        e_got += float(((O[:, n].double() - want) ** 2).sum())
+        e_cut += float((((o / l).to(torch.bfloat16).double() - want) ** 2).sum())
+    print("error relative to the pieces': %.4f" % (e_got / e_cut) ** 0.5)
+    # both are sums over Lq N D independent roundings: their ratio scatters by about (Lq N D / row correlation)^-1/2 < 1 %
+    assert e_got <= 1.02 * e_cut
+
+
 def test_attention_bounded_wait_runs_out_and_recovers():
     """Every wait in the kernels is bounded.  With the workspace header's test hook set, the
     attention kernel's loader issues no copies: the MMA issuers' and softmax warps' waits run out,
