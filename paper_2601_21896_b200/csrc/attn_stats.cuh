@@ -87,9 +87,12 @@ attn_stats_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant_
                     tma_load_3d(sK + st * kTileBytes + kHalfBytes, &mK, k_full(st), 64, g.head, row);
                 }
             }
-            if (!ok)       // let copies already in flight land before the CTA exits
+            if (!ok) {     // let copies already in flight land before the CTA exits
                 for (uint32_t r = ring > (uint32_t)kStatsStages ? ring - kStatsStages : 0; r < ring; ++r)
                     mbar_wait(k_full(r % kStatsStages), (r / kStatsStages) & 1u);
+                if (qc0 > 0) mbar_wait(q_full(0), (qc0 - 1) & 1u);
+                if (qc1 > 0) mbar_wait(q_full(1), (qc1 - 1) & 1u);
+            }
         }
         __syncwarp();
     } else if (warp == 8 || warp == 10) {

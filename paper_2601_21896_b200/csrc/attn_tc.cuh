@@ -504,6 +504,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                     o0 = n0; o1 = n1;
                 }
             }
+            if (!ok) {
+                // let lane 0's copies already in flight land before the CTA exits
+                for (uint32_t r = ring >= (uint32_t)kStages ? ring - kStages : (uint32_t)kv; r < ring; r += 2)
+                    mbar_wait(kv_full(r % kStages), (r / kStages) & 1u);
+                if (qcnt0 > 0) mbar_wait(q_full(0), (qcnt0 - 1) & 1u);
+                if (qcnt1 > 0) mbar_wait(q_full(1), (qcnt1 - 1) & 1u);
+            }
             cp_async_wait_all();
         } else if (elect_one() && p.status[kStatusWordStallLoader] == 0) {
             prefetch_tmap(&mQ); prefetch_tmap(&mKc); prefetch_tmap(&mVc);
@@ -541,6 +548,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                 // let copies already in flight land before the CTA exits
                 for (uint32_t r = ring > (uint32_t)kStages ? ring - kStages : 0; r < ring; ++r)
                     mbar_wait(kv_full(r % kStages), (r / kStages) & 1u);
+                if (qcnt0 > 0) mbar_wait(q_full(0), (qcnt0 - 1) & 1u);
+                if (qcnt1 > 0) mbar_wait(q_full(1), (qcnt1 - 1) & 1u);
             }
         }
         __syncwarp();
