@@ -132,8 +132,8 @@ pafu_status pafu_workspace_status(const void* ws, void* stream);
  *   counts[2]  tiles at which the output accumulator and the row sums were rescaled
  * counts is a HOST array of 3 entries.  Tests use it to show that an input reaches those paths.
  *
- * The header also holds a test hook: while its 32-bit word 32 is non-zero the attention kernel's
- * loader issues no copies, every consumer's bounded wait runs out and the launch ends with
+ * The header also holds a test hook: while its 32-bit word 32 is non-zero the loaders of the attention
+ * kernel (compacted cache) and of the salience target's row statistics issue no copies, every consumer's bounded wait runs out and the launch ends with
  * PAFU_ERR_TIMEOUT in the header (outputs undefined).  It exists so that the time-out path can
  * be exercised without faulting the device; zero the header to return to normal operation. */
 pafu_status pafu_workspace_counters(const void* ws, int64_t* counts, void* stream);

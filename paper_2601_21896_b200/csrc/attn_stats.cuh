@@ -63,7 +63,7 @@ attn_stats_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant_
 
     if (warp == 9) {
         // ---------------------------------------------------------------------- TMA loader
-        if (elect_one()) {
+        if (elect_one() && p.status[kStatusWordStallLoader] == 0) {
             prefetch_tmap(&mQ); prefetch_tmap(&mK);
             SegIter iter(p, blockIdx.x, gridDim.x);
             Seg g;

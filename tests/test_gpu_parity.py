@@ -784,13 +784,16 @@ def test_sse_matches_oracle(L, N, LB):
     assert torch.equal(s, s2)
 
 
-@pytest.mark.parametrize("rise", [0.0, 4.0, -4.0, 20.0])
-@pytest.mark.parametrize("L", [1, 64, 65, 128, 129, 256, 257, 640, 1100])
-def test_sse_row_statistics(L, rise):
-    """The pass that computes the row log-sum-exps (LSE = NULL): sequence lengths around its 128-token tiles,
-    pairs of query tiles and two S buffers, and logits that rise or fall by `rise` nats per 64 keys, so that the
-    running maximum starts far too small, is re-based in every tile, or never."""
-    N, D, LB = 2, 128, max(1, L // 3)
+@pytest.mark.parametrize("rise", [0.0, 4.0, -4.0, 20.0, -20.0])
+@pytest.mark.parametrize("L,N", [(1, 2), (64, 2), (65, 2), (128, 2), (129, 2), (256, 2), (257, 2), (640, 2), (1100, 2),   # runs of one to four tiles
+                                 (4000, 2),      # runs of 13 tiles: past the nine K stages and the four S buffers
+                                 (1100, 40)])    # whole items of 18 tiles and shares of what is left
+def test_sse_row_statistics(L, N, rise):
+    """The pass that computes the row log-sum-exps (LSE = NULL): sequence lengths around its 64-token key tiles, pairs of
+    128-row query tiles and rings of buffers, and logits that rise or fall by `rise` nats per 64 keys: in a run of
+    several tiles the opening tile's maximum then goes stale, is outgrown beyond a row sum of 2^16 again and again,
+    or holds for good.  The same bits as with the log-sum-exps of the attention kernel."""
+    D, LB = 128, max(1, L // 3)
     rng = np.random.default_rng(L)
     Q = rng.standard_normal((L, N, D), dtype=np.float32) + 1.0
     K = rng.standard_normal((L, N, D), dtype=np.float32) + (rise / np.sqrt(D) * np.arange(L, dtype=np.float32) / 64)[:, None, None]
@@ -803,6 +806,35 @@ def test_sse_row_statistics(L, rise):
     # s = exp(z - lse): 32-bit logits and sums of magnitude up to max|z| lose a few units of 2^-24 max|z|
     zmax = 1.0 + np.abs(wl.bf16_bits_to_f32(Q).reshape(L, -1)).sum(1).max() * np.abs(wl.bf16_bits_to_f32(K)).max() / np.sqrt(D)
     np.testing.assert_allclose(s.cpu().numpy(), want, rtol=8 * 2.0 ** -24 * zmax + 1e-6, atol=1e-30)
+    q, k = to_device_bf16(Q), to_device_bf16(K)
+    shape = pafu.Shape(N, D, None, [0, L])
+    ws2 = torch.zeros(pafu.pafu_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    LSE, s2 = torch.empty((N, L), device="cuda"), torch.empty_like(s)
+    pafu.pafu_chunk_attn(q, k, k, [0, L], None, None, shape, 0.0, torch.empty_like(q), LSE, ws2)
+    pafu.pafu_sse(q, k, LSE, LB, 0.0, s2, None, ws)
+    assert torch.equal(s, s2)
+    if L == 4000 and rise == 20.0:
+        c = pafu.pafu_workspace_counters(ws2)
+        assert c[1] > 0 and c[2] > 0      # such an input does send tiles through the redo and the re-base
+
+
+def test_sse_row_statistics_bounded_wait_runs_out_and_recovers():
+    """The row-statistics pass with its loader stalled (the header's test hook): every role's wait runs out, the launch
+    ends, the header holds a time-out code of that pass, and after it is cleared the workspace serves a normal call."""
+    L, N, D, LB = 700, 2, 128, 200
+    rng = np.random.default_rng(4)
+    Q, K = [wl.f32_to_bf16_bits(rng.standard_normal((L, N, D), dtype=np.float32)) for _ in range(2)]
+    q, k, s = to_device_bf16(Q), to_device_bf16(K), torch.zeros(L, device="cuda")
+    ws = torch.zeros(pafu.pafu_sse_workspace_bytes(L, N, D, LB), dtype=torch.uint8, device="cuda")
+    ws.view(torch.int32)[32] = 1
+    pafu.pafu_sse(q, k, None, LB, 0.0, s, None, ws)
+    assert pafu.pafu_workspace_status(ws) == 7                   # PAFU_ERR_TIMEOUT, after about half a second
+    assert int(ws.view(torch.int32)[0].item()) in (711, 712, 721)
+    ws[:256] = 0
+    pafu.pafu_sse(q, k, None, LB, 0.0, s, None, ws)
+    assert pafu.pafu_workspace_status(ws) == 0
+    want, _ = oracle.sse(Q, K, LB)
+    np.testing.assert_allclose(s.cpu().numpy(), want, rtol=1e-4, atol=1e-30)   # logits below 100: 8 x 2^-24 x 100 < 1e-4
 
 
 @pytest.mark.parametrize("L,N,LB", [
