@@ -284,7 +284,7 @@ def _attention_all_entry_points(d, N, D, Lq, nB, what, seed=0):
 
 # (heads, chunk queries, retained keys): "short" gives every CTA a run of about two key tiles and
 # splits every item over dozens of CTAs (the merge sees many pieces); "long" gives runs of about
-# eight tiles (the in-kernel rescale has tiles before and after it).  Both have a ragged last query
+# ten tiles (the in-kernel rescale has tiles before and after it).  Both have a ragged last query
 # block, a ragged last retained tile and a ragged last chunk tile.
 PEAKED_SIZES = {"short": (2, 600, 3017), "long": (2, 770, 12013)}
 
