@@ -244,8 +244,8 @@ inline int sm_count() { return device_sm_count(); }
 // 8 us together.  So a problem whose items fit on the GPU at once and whose longest item is at most three
 // 64-key tiles longer than a share is not split (seven: 2 to 4 us faster on some problems of 8 to 15 tiles an item, slower on
 // others), and no share is made smaller than one tile.  Before (shares down to a fraction of a tile, a
-// serial merge): 2 heads x 120 queries x 8023 keys 77 us, now 28; three ragged streams of 2 heads 31.5 and 20;
-// 24 heads x 147 queries x 268 keys 21 and 17.
+// serial merge): 2 heads x 120 queries x 8023 keys 80 us, now 20; three ragged streams of 2 heads 31.7 and 16.7;
+// 2 heads x 600 queries x 2000 keys 44 and 18.
 constexpr int kMergeTiles = 3, kMinShareTiles = 1;
 inline int cta_limit(int max_ctas) {                         // max_ctas > 0: the caller's scratch holds fewer partials
     const int sms = sm_count();
