@@ -206,7 +206,8 @@ pafu_status pafu_compact_layers(const uint16_t* const* K, const uint16_t* const*
  * Per stream s, head n, query row i: o_i = sum_j softmax_j(scale * q_i . k_j) v_j where j runs
  * over the B_s retained tokens (Kc, Vc) and then the stream's own Lq_s chunk tokens (Kq, Vq).
  * No mask: the chunk is bidirectional and sees the whole retained cache.  bf16 operands,
- * fp32 accumulation and softmax; probabilities are rounded to bf16 before the P V product.
+ * fp32 accumulation and softmax; probabilities are rounded to bf16 before the P V product (where few
+ * tiles of 64 keys fall to an SM, what that rounding leaves over goes through the product as well).
  *   Q         device bf16 [cu_Lq[n_streams], n_heads, d_head]
  *   Kc, Vc    device bf16 [cu_B[n_streams], n_heads, d_head]
  *   cu_B      HOST prefix array [n_streams + 1] of retained tokens
