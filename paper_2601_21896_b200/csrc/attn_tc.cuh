@@ -514,7 +514,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ C
                         ck.step(2);
                     }
                 };
-                if constexpr (ROUND == kRoundOpening) {      // two loops: a branch in the long one costs every tile
+                if constexpr (ROUND == kRoundOpening) {      // two loops, so that issue_pv knows its form
                     tiles(0, n < kOpeningTiles ? n : kOpeningTiles, std::true_type{});
                     tiles(kOpeningTiles, n, std::false_type{});
                 } else {
