@@ -51,13 +51,15 @@ __device__ __forceinline__ void copy_kv_row(const uint4* __restrict__ K, const u
 // the top-k rows.  K and V are not written by the step's earlier kernels, and the outputs are
 // not read by them, so the early part touches nothing the predecessor produces.  (SL is the
 // score array in a step: all of its entries are copied after the wait.)
-// When the selection occupies more than two SMs, rows are handed out through two counters in the
+// When the selection occupies more than kStaticSelect SMs, rows are handed out through two counters in the
 // workspace header (`work`: early rows, late rows, finished blocks), one row per claim with the
 // next claim under way during the copy: the blocks that only get an SM when the selection's CTAs
 // leave simply find less work left, instead of starting a fixed share late (that tail cost 40 us
-// at the batch-4 size); the last block to finish puts the counters back to zero.  With a one- or
-// two-CTA selection the grid leaves those SMs out and every block takes a fixed share
-// (early_static; 5 us faster at the 28 080-token cache than claiming).
+// at the batch-4 size); the last block to finish puts the counters back to zero.  With a selection
+// of one cluster the grid leaves its SMs out and every block takes a fixed share (early_static;
+// selection and gather of the 28 080-token cache, selected by eight CTAs, 39.6 us with claiming, 31.4 with shares; of the
+// 93 600-token one 33.5 and 29.3; four streams, 32 CTAs: no difference).
+constexpr int kStaticSelect = 8;
 constexpr int kCompactClaim = 1;
 
 // A claim in two halves: lane 0 issues the add; its result is fetched (and shared with the warp)
@@ -324,7 +326,7 @@ pafu_status launch_compact(const uint16_t* K, const uint16_t* V, const float* SL
     // A few resident waves, larger inputs loop.  With the early part the grid is what the device
     // holds at once (three blocks fit on an SM): a block must not queue behind blocks that are
     // waiting for the selection.  Fixed shares: the selection's SMs are left out of the count.
-    const int early_static = work != nullptr && select_ctas <= 2;
+        const int early_static = work != nullptr && select_ctas <= kStaticSelect;
     int sms = device_sm_count() - (early_static ? select_ctas : 0);
     if (sms < 1) sms = 1;
     const int64_t max_blocks = work != nullptr ? (int64_t)sms * 3 : 148 * 8 * 4;

@@ -2,22 +2,25 @@
 // Sec. 4.1): kept = [0, n_sink) U top-k salient of the middle U [T - n_recent, T), written as
 // ascending token indices, ties to the lower index.
 //
-// The step moves a few hundred KB, so it is latency-bound.  One CTA, or a cluster of two, four or
-// eight (the host picks by the stream length), works on one stream; CTA r holds the r-th part of
-// the candidates in its shared memory.
+// The step moves a few hundred KB, so it is latency-bound: what counts is the chain of barriers, the trips through
+// distributed shared memory, and instructions that every warp executes (a scan by 32 warps costs four times the issue slots of
+// one by eight, so short shares run in blocks of 256 threads and eight warps do what is done once).  One CTA, or a
+// cluster of two, four or eight (the host picks by the stream length), works on one stream; CTA r holds the r-th part of the
+// candidates in its shared memory.  Back to back, 444 / 4000 / 7800 / 21 840 / 87 360 candidates: 4.3 / 7.6 / 8.5 / 9.4 / 16.7 us; with
+// three passes over digits of the key (11 + 11 + 10 bits, a tenth of the candidates left after the first), blocks of 1024 and one CTA
+// up to 24 576 candidates 8.4 / 10.1 / 11.8 / 19.6 / 25.4.
 //   1. fp32 scores map to order-preserving 32-bit keys (-0 folded onto +0, NaN lowest).
-//   2. MSB-first radix select (11 + 11 + 10 bits) finds the key of the k-th largest candidate and
-//      how many candidates equal to it are still needed.  Per pass every CTA builds the histogram
-//      of its own candidates, one cluster barrier later every CTA adds up all eight histograms
-//      through distributed shared memory and finds the bin by itself: all eight reach the same
-//      decision, so nothing has to be sent back (one barrier per pass; the histograms alternate
-//      between two buffers so that a CTA may start the next pass while others still read).  After
-//      the first digit a CTA's surviving candidates are few and move to a short list that the
-//      later passes read instead of the whole array.
-//   3. Ordered emission: candidate j belongs to (CTA, round, warp, lane); warp ballots count
-//      kept and tied candidates per (round, warp), the CTAs exchange their totals (one more
-//      barrier), and scans over those counts give every kept token its output slot, so the
-//      result is ascending and ties resolve to the lowest indices.
+//   2. One histogram of 1024 equal steps between the smallest and the largest of 256 sampled scores (the same sample in
+//      every CTA, so nothing is exchanged for it; values outside fall into the end bins).  One cluster barrier later
+//      every CTA adds up all histograms through distributed shared memory and finds by itself the bin that holds the k-th
+//      largest candidate.  Every CTA sends its few candidates of that bin to all others; one more barrier, and each ranks
+//      them against one another by itself.
+//   3. A bin that holds too many (ties, a far outlier in the sample) is narrowed down: the smallest and the largest of
+//      its candidates are exchanged, and if they differ another histogram divides what lies between them, first in equal
+//      steps of the score, then of the key (which ends: 2^32 keys, a factor of 1024 each time).
+//   4. Ordered emission: every warp owns a contiguous stretch of the CTA's candidates, counts what it keeps and, once the counts
+//      of the warps and CTAs before it are known, writes it in order: the result is ascending and ties resolve to
+//      the lowest indices.
 // Streams with more candidates than eight CTAs hold (360 448) use one CTA that re-reads L2 in every pass.
 // A kernel launched behind these as a programmatic dependent may start at once (the trigger at
 // their top): inside a layer step that is the row gather, which copies the rows that are kept
@@ -30,13 +33,18 @@ namespace pafu {
 
 namespace cg = cooperative_groups;
 
-constexpr int kSelThreads = 1024;
+constexpr int kSelThreads = 256;            // block of a CTA with a short share; kSelThreadsMax with a long one
+constexpr int kSelThreadsMax = 1024;
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelWarpsMax = kSelThreadsMax / 32;
 constexpr int kSelCluster = 8;              // at most this many CTAs cooperate on one stream
 constexpr int kSelCapCta = 45056;           // candidates one CTA holds (176 KiB of keys)
 constexpr int kSelCapCluster = kSelCluster * kSelCapCta;
-constexpr int kSelHistBins = 2048;
-constexpr int kSelListCap = 4096;           // candidates of a CTA the later passes can take from its short list
+constexpr int kSelBins = 1024;
+constexpr int kSelList = 1024;              // most candidates in the bin of the k-th largest one that are ranked directly
 constexpr int kSelBatch = 8;                // independent loads a thread keeps in flight
+constexpr int kSelStreamThreads = 1024;     // the streaming kernel's block
+static_assert(kSelBins == 4 * kSelThreads, "four bins a thread");
 
 __device__ __forceinline__ uint32_t score_key(float f) {
     uint32_t u = __float_as_uint(f);
@@ -45,7 +53,7 @@ __device__ __forceinline__ uint32_t score_key(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Exclusive prefix sum of one int per thread over the block; also returns the block total.
+// Exclusive prefix sum of one int per thread over a block of 1024; also returns the block total.
 __device__ __forceinline__ int sel_exclusive_scan(int v, int* warp_sums, int* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int inc = v;
@@ -73,240 +81,301 @@ __device__ __forceinline__ int sel_exclusive_scan(int v, int* warp_sums, int* to
     return warp_sums[warp] + inc - v;
 }
 
+// The score a key stands for (a NaN for key 0).
+__device__ __forceinline__ float key_score(uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); }
+
 struct SelShared {
-    int warp_sums[33];
-    uint32_t prefix;
-    int k_rem, bin_count, list_n;
-    int tot[kSelCluster][2];         // every CTA's count of candidates above / equal to the threshold
+    int sums[kSelWarps];
+    uint32_t lo[kSelWarpsMax], hi[kSelWarpsMax];
+    int bin, k_rem, bin_count;
+    uint32_t thr;
+    int need_eq, eq_total;
+    int list_n;
+    int warp_gt[kSelWarpsMax], warp_eq[kSelWarpsMax];
+    // from every CTA: its candidates in the bin and above it, and the smallest and largest of those in it
+    int in_bin[kSelCluster], above[kSelCluster];
+    uint32_t cta_lo[kSelCluster], cta_hi[kSelCluster];
 };
 
-// One radix pass: histogram of `bits` bits at `shift` over this CTA's n candidates that `get`
-// admits, into `hist` (this pass's buffer, at the same address in every CTA); then, one cluster
-// barrier later, the sum of the eight CTAs' histograms and the bin that holds the k_rem-th largest
-// admitted key.  (Spreading the lanes over several copies of the histogram, or grouping equal
-// digits with match.any before adding, did not make the adds cheaper: a shared-memory add costs
-// about 13 clocks per warp instruction whether or not its lanes collide.)
-template <typename Get>
-__device__ __forceinline__ void radix_pass(cg::cluster_group& cluster, SelShared& sh, int* hist, int n, int shift,
-                                           int bits, uint32_t& prefix, int& k_rem, int& bin_count, Get get) {
-    const int tid = threadIdx.x;
-    const int nb = 1 << bits, nc = (int)cluster.num_blocks();
-    for (int b = tid; b < nb; b += kSelThreads) hist[b] = 0;
-    __syncthreads();
-    for (int j0 = 0; j0 < n; j0 += kSelThreads * kSelBatch) {
-        uint32_t key[kSelBatch];
-        bool in[kSelBatch];
-#pragma unroll
-        for (int u = 0; u < kSelBatch; ++u) {
-            const int j = j0 + u * kSelThreads + tid;
-            key[u] = 0u;
-            in[u] = (j < n) && get(j, key[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < kSelBatch; ++u)
-            if (in[u]) atomicAdd(&hist[(key[u] >> shift) & (uint32_t)(nb - 1)], 1);
-    }
-    cluster.sync();                  // every CTA's histogram is complete (and visible to the cluster)
-    // bins from the top: thread t holds bins nb-1-2t and nb-2-2t (nb <= 2048 = 2 x block size)
-    int c[2] = {0, 0};
-    const int b_hi = nb - 1 - 2 * tid;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int b = b_hi - i;
-        if (b >= 0) {
-            int v = 0;
-            for (int r = 0; r < nc; ++r) v += *cluster.map_shared_rank(hist + b, r);
-            c[i] = v;
-        }
-    }
-    int total;
-    const int above = sel_exclusive_scan(c[0] + c[1], sh.warp_sums, &total);
-    if (above < k_rem && k_rem <= above + c[0]) {
-        sh.prefix = prefix | ((uint32_t)b_hi << shift); sh.k_rem = k_rem - above; sh.bin_count = c[0];
-    } else if (above + c[0] < k_rem && k_rem <= above + c[0] + c[1]) {
-        sh.prefix = prefix | ((uint32_t)(b_hi - 1) << shift); sh.k_rem = k_rem - above - c[0]; sh.bin_count = c[1];
-    }
-    __syncthreads();
-    prefix = sh.prefix; k_rem = sh.k_rem; bin_count = sh.bin_count;
+__device__ __forceinline__ void sel_barrier(cg::cluster_group& cluster, int nc) {
+    if (nc > 1) cluster.sync(); else __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSelThreads, 1)
+// The bin that holds the k_rem-th largest of what the CTAs' histograms `hist` (the same address in every CTA) count, to
+// sh.bin, sh.k_rem, sh.bin_count.  The barrier at the top makes every histogram complete and visible.  (Eight warps do it
+// whatever the block: a scan by 32 costs four times the issue slots.)
+__device__ __forceinline__ void find_bin(cg::cluster_group& cluster, int nc, SelShared& sh, const int* hist, int k_rem) {
+    sel_barrier(cluster, nc);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // bins from the top: thread t holds bins 1023 - 4 t .. 1020 - 4 t
+    const int b_hi = kSelBins - 1 - 4 * tid;
+    int c[4] = {0, 0, 0, 0}, own = 0, inc = 0;
+    if (warp < kSelWarps) {
+        const int* mine = hist + b_hi - 3;
+        for (int r0 = 0; r0 < nc; r0 += 4) {
+            int4 v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) v[r] = r0 + r < nc ? *reinterpret_cast<const int4*>(cluster.map_shared_rank(mine, r0 + r)) : make_int4(0, 0, 0, 0);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) { c[0] += v[r].w; c[1] += v[r].z; c[2] += v[r].y; c[3] += v[r].x; }
+        }
+        own = inc = c[0] + c[1] + c[2] + c[3];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int n = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += n;
+        }
+        if (lane == 31) sh.sums[warp] = inc;
+    }
+    __syncthreads();
+    if (warp < kSelWarps) {
+        int above = inc - own;
+#pragma unroll
+        for (int w = 0; w < kSelWarps - 1; ++w) above += w < warp ? sh.sums[w] : 0;
+        if (above < k_rem && k_rem <= above + own) {
+            int i = 0;
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+                if (i == u && above + c[u] < k_rem) { above += c[u]; ++i; }
+            sh.bin = b_hi - i; sh.k_rem = k_rem - above; sh.bin_count = i == 0 ? c[0] : i == 1 ? c[1] : i == 2 ? c[2] : c[3];
+        }
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kSelThreadsMax, 1)
 select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ StreamTable st, int32_t keys_bytes,
                       int32_t* __restrict__ idx, int trigger_late) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     __shared__ SelShared sh;
     if (!trigger_late) grid_dep_launch_dependents();
-    grid_dep_wait();
-    if (trigger_late) grid_dep_launch_dependents();
     cg::cluster_group cluster = cg::this_cluster();
     const int nc = (int)cluster.num_blocks();                // 1, 2, 4 or 8: the host's choice for this launch
     const int s = blockIdx.x / nc;
     const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = kSelThreads / 32;
-    const int64_t T64 = st.cu_T[s + 1] - st.cu_T[s], B64 = st.cu_B[s + 1] - st.cu_B[s];
-    // cluster-uniform exits (before any cluster barrier)
-    if (B64 == 0) return;
-    const int T = (int)T64, B = (int)B64;
+    const int threads = (int)blockDim.x, warps = threads >> 5;
+    uint32_t* keys = reinterpret_cast<uint32_t*>(sel_smem);
+    int* hist = reinterpret_cast<int*>(sel_smem + keys_bytes);               // two histograms
+    uint32_t* list = reinterpret_cast<uint32_t*>(hist + 2 * kSelBins);       // [kSelCluster][kSelList]: every CTA's candidates in the bin
+    uint32_t* all = list + kSelCluster * kSelList;                           // [kSelList]: the same side by side
+    if (tid < kSelThreads) *reinterpret_cast<int4*>(hist + 4 * tid) = make_int4(0, 0, 0, 0);
+    if (tid == 0) sh.list_n = 0;
+    const int T = (int)(st.cu_T[s + 1] - st.cu_T[s]), B = (int)(st.cu_B[s + 1] - st.cu_B[s]);
     // a stream that keeps everything is one long "sink"
-    const bool all = B >= T;
-    const int ns = all ? T : (int)st.n_sink[s], nr = all ? 0 : (int)st.n_recent[s], k = all ? 0 : (int)st.k[s];
+    const bool everything = B >= T;
+    const int ns = everything ? T : (int)st.n_sink[s], nr = everything ? 0 : (int)st.n_recent[s], k = everything ? 0 : (int)st.k[s];
     const int M = T - ns - nr;
-    if (M > nc * kSelCapCta) return;                         // the streaming kernel owns this stream
+    const float* first = scores + st.cu_T[s] + ns;
     int32_t* out = idx + st.cu_B[s];
+    grid_dep_wait();
+    if (trigger_late) grid_dep_launch_dependents();
+    // cluster-uniform exits (before any cluster barrier)
+    if (B == 0) return;
+    if (M > nc * kSelCapCta) return;                         // the streaming kernel owns this stream
+
+    // this CTA's candidates: [j_lo, j_lo + n) of the stream's M
+    const int per_cta = ((M + nc - 1) / nc + 31) / 32 * 32;
+    const int j_lo = rank * per_cta;
+    const int n = max(0, min(M - j_lo, per_cta));
+    if (k > 0) {
+        const int step = M / kSelThreads;                    // 0: every candidate is in the sample
+        const int js = step > 0 ? tid * step : tid;
+        const float sample = js < M && tid < kSelThreads ? __ldg(first + js) : __uint_as_float(0x7fc00000u);
+        for (int j0 = tid; j0 < n; j0 += threads * kSelBatch) {
+            float v[kSelBatch];
+#pragma unroll
+            for (int u = 0; u < kSelBatch; ++u) v[u] = j0 + u * threads < n ? __ldg(first + j_lo + j0 + u * threads) : 0.f;
+#pragma unroll
+            for (int u = 0; u < kSelBatch; ++u)
+                if (j0 + u * threads < n) keys[j0 + u * threads] = score_key(v[u]);
+        }
+        // the finite samples' range
+        const uint32_t ks = score_key(sample);
+        const bool finite = ks >= 0x00800000u && ks <= 0xff7fffffu;
+        const uint32_t lo_w = __reduce_min_sync(0xffffffffu, finite ? ks : 0xffffffffu), hi_w = __reduce_max_sync(0xffffffffu, finite ? ks : 0u);
+        if (lane == 0) { sh.lo[warp] = lo_w; sh.hi[warp] = hi_w; }
+    }
     // always-kept tokens (spread over the cluster): position p < ns is token p, position ns + k + i is token T - nr + i
-    for (int p = rank * kSelThreads + tid; p < ns + nr; p += nc * kSelThreads) {
+    for (int p = rank * threads + tid; p < ns + nr; p += nc * threads) {
         if (p < ns) out[p] = p; else out[p + k] = T - (ns + nr) + p;
     }
     if (k == 0) return;
-
-    // this CTA's candidates: [j_lo, j_lo + n) of the stream's M, a whole number of rounds per CTA
-    const int per_cta = (M + nc * kSelThreads - 1) / (nc * kSelThreads) * kSelThreads;
-    const int j_lo = rank * per_cta;
-    const int n = max(0, min(M - j_lo, per_cta));
-    const float* sc = scores + st.cu_T[s] + ns + j_lo;
-    uint32_t* keys = reinterpret_cast<uint32_t*>(sel_smem);
-    uint32_t* list = reinterpret_cast<uint32_t*>(sel_smem + keys_bytes);
-    int* hist0 = reinterpret_cast<int*>(sel_smem + keys_bytes + kSelListCap * 4);
-    int* hist1 = hist0 + kSelHistBins;
-    for (int j0 = tid; j0 < n; j0 += kSelThreads * kSelBatch) {
-        float v[kSelBatch];
-#pragma unroll
-        for (int u = 0; u < kSelBatch; ++u) {
-            const int j = j0 + u * kSelThreads;
-            v[u] = j < n ? __ldg(sc + j) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < kSelBatch; ++u) {
-            const int j = j0 + u * kSelThreads;
-            if (j < n) keys[j] = score_key(v[u]);
-        }
-    }
-    if (tid == 0) sh.list_n = 0;
     __syncthreads();
-
-    // ---- the key of the k-th largest candidate
+    uint32_t klo = 0u, khi = 0xffffffffu;                    // the keys still in question
+    float lo = 0.f, scale = 0.f;                             // how they are divided: equal steps of the score,
+    int shift = -1;                                          // or of the key (>= 0)
+    auto steps = [&](uint32_t a, uint32_t b) {               // between the finite scores of keys a < b
+        lo = key_score(a);
+        scale = (float)kSelBins / (key_score(b) - lo);
+        if (!(scale <= 3.0e38f)) scale = 0.f;                // a range of a few denormals
+    };
+    {
+        const uint32_t a = __reduce_min_sync(0xffffffffu, sh.lo[lane & (kSelWarps - 1)]), b = __reduce_max_sync(0xffffffffu, sh.hi[lane & (kSelWarps - 1)]);
+        if (a < b) steps(a, b);                              // at least two finite values
+    }
+    // Monotone in the key: rounding is, and so are the clamps; infinities end up in the end bins, NaN (lowest) in bin 0, and with
+    // scale = 0 everything in bin 0.
+    auto bin_of = [&](uint32_t key) {
+        int b = shift >= 0 ? (int)((key - klo) >> shift)
+                           : min(max(__float2int_rz(__fmul_rn(__fsub_rn(key_score(key), lo), scale)), 0), kSelBins - 1);
+        if (key < klo) b = -1;
+        if (key > khi) b = kSelBins;
+        return b;
+    };
+    // each warp's stretch of the candidates: whole groups of 32
+    const int per_warp = ((n + 31) / 32 + warps - 1) / warps * 32;
+    const int w0 = min(n, warp * per_warp), w1 = min(n, w0 + per_warp);
+    const unsigned lt = (1u << lane) - 1u;
     uint32_t thr = 0u;
     int need_eq = k, eq_total = 0;
-    radix_pass(cluster, sh, hist0, n, 21, 11, thr, need_eq, eq_total,
-               [&](int j, uint32_t& key) { key = keys[j]; return true; });
-    // this CTA's survivors go to its short list if they fit (any order: only their values matter now)
-    int n_mine = 0;
-    {
-        const uint32_t top = thr >> 21;
-        for (int j0 = 0; j0 < n; j0 += kSelThreads) {
-            const int j = j0 + tid;
-            const uint32_t kx = j < n ? keys[j] : 0u;
-            const bool hit = j < n && (kx >> 21) == top;
-            const unsigned b = __ballot_sync(0xffffffffu, hit);
-            if (b != 0u) {
-                int base = 0;
-                if (lane == 0) base = atomicAdd(&sh.list_n, __popc(b));
-                base = __shfl_sync(0xffffffffu, base, 0);
-                const int slot = base + __popc(b & ((1u << lane) - 1u));
-                if (hit && slot < kSelListCap) list[slot] = kx;
+    int gt_before = 0, eq_before = 0;                        // in the CTAs before this one
+    bool ranked = true;
+#pragma unroll 1
+    for (int level = 0;; ++level) {                          // cluster-uniform
+        int* h = hist + (level & 1) * kSelBins;              // (every CTA is past its reads of the level before last)
+        if (level > 0) {
+            if (tid < kSelThreads) *reinterpret_cast<int4*>(h + 4 * tid) = make_int4(0, 0, 0, 0);
+            __syncthreads();
+        }
+#pragma unroll 4
+        for (int j = tid; j < n; j += threads) {
+            const int b = bin_of(keys[j]);
+            if ((unsigned)b < (unsigned)kSelBins) atomicAdd(h + b, 1);
+        }
+        find_bin(cluster, nc, sh, h, need_eq);
+        need_eq = sh.k_rem; eq_total = sh.bin_count;
+        // ranking m keys costs a warp m / 32 turns of m comparisons, narrowing down two more sweeps over the CTA's share
+        if (eq_total <= max(256, min(kSelList, per_cta / 32))) break;
+        // ---- too many: what lies between the smallest and the largest of them
+        const int bin = sh.bin;
+        int above = 0, in = 0;
+        uint32_t mn = 0xffffffffu, mx = 0u;
+        for (int j0 = w0; j0 < w1; j0 += 32) {
+            const uint32_t key = j0 + lane < w1 ? keys[j0 + lane] : 0u;
+            const int b = j0 + lane < w1 ? bin_of(key) : -1;
+            above += __popc(__ballot_sync(0xffffffffu, b > bin));
+            in += __popc(__ballot_sync(0xffffffffu, b == bin));
+            if (b == bin) { mn = min(mn, key); mx = max(mx, key); }
+        }
+        mn = __reduce_min_sync(0xffffffffu, mn); mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) { sh.lo[warp] = mn; sh.hi[warp] = mx; sh.warp_gt[warp] = above; sh.warp_eq[warp] = in; }
+        __syncthreads();
+        if (warp == 0) {
+            const int a = __reduce_add_sync(0xffffffffu, lane < warps ? sh.warp_gt[lane] : 0), i = __reduce_add_sync(0xffffffffu, lane < warps ? sh.warp_eq[lane] : 0);
+            mn = __reduce_min_sync(0xffffffffu, lane < warps ? sh.lo[lane] : 0xffffffffu); mx = __reduce_max_sync(0xffffffffu, lane < warps ? sh.hi[lane] : 0u);
+            if (lane < nc) {
+                SelShared* remote = cluster.map_shared_rank(&sh, lane);
+                remote->in_bin[rank] = i; remote->above[rank] = a; remote->cta_lo[rank] = mn; remote->cta_hi[rank] = mx;
             }
+        }
+        sel_barrier(cluster, nc);
+        mn = __reduce_min_sync(0xffffffffu, lane < nc ? sh.cta_lo[lane] : 0xffffffffu); mx = __reduce_max_sync(0xffffffffu, lane < nc ? sh.cta_hi[lane] : 0u);
+        if (mn == mx) {                                      // all equal
+            thr = mn;
+            gt_before = __reduce_add_sync(0xffffffffu, lane < rank ? sh.above[lane] : 0);
+            eq_before = __reduce_add_sync(0xffffffffu, lane < rank ? sh.in_bin[lane] : 0);
+            ranked = false;
+            break;
+        }
+        klo = mn; khi = mx;
+        const bool finite = klo >= 0x00800000u && khi <= 0xff7fffffu;
+        if (level == 0 && finite) steps(klo, khi);
+        else shift = max(0, 22 - __clz(khi - klo));
+    }
+    if (ranked) {
+        // ---- the bin's candidates, to segment `rank` of every CTA's list (any order: only their values matter now)
+        const int bin = sh.bin, k_rem = need_eq;
+        int above = 0;
+#pragma unroll 4
+        for (int j0 = w0; j0 < w1; j0 += 32) {
+            const uint32_t key = j0 + lane < w1 ? keys[j0 + lane] : 0u;
+            const int b = j0 + lane < w1 ? bin_of(key) : -1;
+            above += __popc(__ballot_sync(0xffffffffu, b > bin));
+            if (b == bin) {
+                const int at = atomicAdd(&sh.list_n, 1);
+                for (int r = 0; r < nc; ++r) cluster.map_shared_rank(list, r)[rank * kSelList + at] = key;
+            }
+        }
+        if (lane == 0) sh.warp_gt[warp] = above;
+        __syncthreads();
+        if (warp == 0) {
+            const int a = __reduce_add_sync(0xffffffffu, lane < warps ? sh.warp_gt[lane] : 0);
+            if (lane < nc) {
+                SelShared* remote = cluster.map_shared_rank(&sh, lane);
+                remote->in_bin[rank] = sh.list_n; remote->above[rank] = a;
+            }
+        }
+        sel_barrier(cluster, nc);
+        // ---- side by side, in the CTAs' order
+        const int in_bin = lane < nc ? sh.in_bin[lane] : 0;
+        const int n_all = __reduce_add_sync(0xffffffffu, in_bin), n_before = __reduce_add_sync(0xffffffffu, lane < rank ? in_bin : 0);
+        gt_before = __reduce_add_sync(0xffffffffu, lane < rank ? sh.above[lane] : 0);
+        uint32_t* flat = nc > 1 ? all : list;
+        if (nc > 1 && warp < nc) {
+            const int at = __reduce_add_sync(0xffffffffu, lane < warp ? in_bin : 0), m = sh.in_bin[warp];
+            for (int i = lane; i < m; i += 32) all[at + i] = list[warp * kSelList + i];
+        }
+        if (nc > 1) __syncthreads();
+        // ---- the key of the k_rem-th largest of them: every thread ranks its own
+        for (int i = tid; i < n_all; i += threads) {
+            const uint32_t key = flat[i];
+            int gt = 0, eq = 0;
+            int e = 0;
+#pragma unroll 2
+            for (; e + 4 <= n_all; e += 4) {
+                const uint4 o = *reinterpret_cast<const uint4*>(flat + e);
+                gt += (o.x > key) + (o.y > key) + (o.z > key) + (o.w > key);
+                eq += (o.x == key) + (o.y == key) + (o.z == key) + (o.w == key);
+            }
+            for (; e < n_all; ++e) { gt += flat[e] > key; eq += flat[e] == key; }
+            if (gt < k_rem && k_rem <= gt + eq) { sh.thr = key; sh.need_eq = k_rem - gt; sh.eq_total = eq; }   // equal keys write the same
         }
         __syncthreads();
-        n_mine = sh.list_n;
-    }
-    const bool listed = n_mine <= kSelListCap;               // block-uniform (each CTA decides for itself)
-    const int n_rest = listed ? n_mine : n;
-    {
-        const uint32_t pf1 = thr;
-        radix_pass(cluster, sh, hist1, n_rest, 10, 11, thr, need_eq, eq_total, [&](int j, uint32_t& key) {
-            key = listed ? list[j] : keys[j];
-            return (key & 0xffe00000u) == pf1;
-        });
-        const uint32_t pf2 = thr;
-        radix_pass(cluster, sh, hist0, n_rest, 0, 10, thr, need_eq, eq_total, [&](int j, uint32_t& key) {
-            key = listed ? list[j] : keys[j];
-            return (key & 0xfffffc00u) == pf2;
-        });
+        thr = sh.thr; need_eq = sh.need_eq; eq_total = sh.eq_total;
+        // what the CTAs before this one keep of them (every warp for itself)
+        for (int i0 = 0; i0 < n_before; i0 += 32) {
+            const bool in = i0 + lane < n_before;
+            const uint32_t key = in ? flat[i0 + lane] : 0u;
+            gt_before += __popc(__ballot_sync(0xffffffffu, in && key > thr));
+            eq_before += __popc(__ballot_sync(0xffffffffu, in && key == thr));
+        }
     }
 
-    // ---- ordered emission.  Own candidate j = (round * NW + warp) * 32 + lane; per (round, warp)
-    // pair the counts of candidates above the threshold and equal to it (one byte each) go to shared
-    // memory, scans over the pairs and the CTAs' totals turn them into output slots.  hist1 and the
-    // list are free now (hist0 may still be read by other CTAs).
+    // ---- ordered emission
     const bool ties = need_eq != eq_total;                   // cluster-uniform: some equal candidates stay out
-    const int rounds = (n + kSelThreads - 1) / kSelThreads, n_pairs = rounds * NW;
-    uint16_t* cnt = reinterpret_cast<uint16_t*>(hist1);      // [n_pairs]: above | equal << 8
-    int* slot = reinterpret_cast<int*>(list);                // [n_pairs]: kept before the pair | equal ones taken << 24
-    // a thread's candidates' classes stay in registers as bit masks (rounds <= 44)
-    uint32_t gtb[2], eqb[2];
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk) {
-        uint32_t g = 0u, e = 0u;
-        const int i_end = min(rounds, (blk + 1) * 32);
-        for (int i = blk * 32; i < i_end; ++i) {
-            const int j = i * kSelThreads + tid;
-            const uint32_t kx = j < n ? keys[j] : 0u;
-            const bool is_gt = j < n && kx > thr, is_eq = j < n && kx == thr;
-            const unsigned bg = __ballot_sync(0xffffffffu, is_gt), be = __ballot_sync(0xffffffffu, is_eq);
-            if (lane == 0) cnt[i * NW + warp] = (uint16_t)(__popc(bg) | (__popc(be) << 8));
-            g |= (uint32_t)is_gt << (i & 31);
-            e |= (uint32_t)is_eq << (i & 31);
-        }
-        gtb[blk] = g; eqb[blk] = e;
+    int gt = 0, eq = 0;
+#pragma unroll 4
+    for (int j0 = w0; j0 < w1; j0 += 32) {
+        const uint32_t key = j0 + lane < w1 ? keys[j0 + lane] : 0u;
+        gt += __popc(__ballot_sync(0xffffffffu, j0 + lane < w1 && key > thr));
+        eq += __popc(__ballot_sync(0xffffffffu, j0 + lane < w1 && key == thr));
     }
+    __syncthreads();                                         // the last reads of warp_gt are complete
+    if (lane == 0) { sh.warp_gt[warp] = gt; sh.warp_eq[warp] = eq; }
     __syncthreads();
-    // thread t owns pairs [t * per, (t + 1) * per)
-    const int per = (n_pairs + kSelThreads - 1) / kSelThreads;
-    const int p0 = min(n_pairs, tid * per), p1 = min(n_pairs, p0 + per);
-    int my_gt = 0, my_eq = 0;
-    for (int p = p0; p < p1; ++p) { my_gt += cnt[p] & 0xff; my_eq += cnt[p] >> 8; }
-    int gt_cta, eq_cta;
-    const int gt_before_t = sel_exclusive_scan(my_gt, sh.warp_sums, &gt_cta);
-    const int eq_before_t = sel_exclusive_scan(my_eq, sh.warp_sums, &eq_cta);
-    if (tid < nc) {                                          // this CTA's totals, to every CTA of the cluster
-        int* remote = &cluster.map_shared_rank(&sh, tid)->tot[rank][0];
-        remote[0] = gt_cta; remote[1] = eq_cta;
-    }
-    cluster.sync();
-    // candidates kept in the CTAs before this one, and equal ones seen there
-    int kept_before = 0, eq_before = 0;
-    for (int r = 0; r < rank; ++r) {
-        const int take = ties ? min(sh.tot[r][1], max(0, need_eq - eq_before)) : sh.tot[r][1];
-        kept_before += sh.tot[r][0] + take;
-        eq_before += sh.tot[r][1];
-    }
-    {
-        // kept before this thread's pairs inside the CTA: the ones above the threshold, and of the
-        // equal ones those that still fit
-        int e = eq_before + eq_before_t;
-        const int taken_before_t = ties ? min(eq_before_t, max(0, need_eq - eq_before)) : eq_before_t;
-        int pos = kept_before + gt_before_t + taken_before_t;
-        for (int p = p0; p < p1; ++p) {
-            const int g = cnt[p] & 0xff, q = cnt[p] >> 8;
-            const int take = ties ? min(q, max(0, need_eq - e)) : q;
-            slot[p] = pos | (take << 24);                    // take <= 32; pos < 2^24
-            e += q;
-            pos += g + take;
+    gt_before += __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp_gt[lane] : 0);
+    eq_before += __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp_eq[lane] : 0);
+    int pos = ns + gt_before + (ties ? min(eq_before, need_eq) : eq_before);
+#pragma unroll 4
+    for (int j0 = w0; j0 < w1; j0 += 32) {
+        const uint32_t key = j0 + lane < w1 ? keys[j0 + lane] : 0u;
+        const bool is_eq = j0 + lane < w1 && key == thr;
+        bool keep = j0 + lane < w1 && key >= thr;
+        if (ties) {
+            const unsigned be = __ballot_sync(0xffffffffu, is_eq);
+            keep = keep && (!is_eq || eq_before + __popc(be & lt) < need_eq);
+            eq_before += __popc(be);
         }
-    }
-    __syncthreads();
-    const unsigned lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk) {
-        const int i_end = min(rounds, (blk + 1) * 32);
-        for (int i = blk * 32; i < i_end; ++i) {
-            const bool is_gt = (gtb[blk] >> (i & 31)) & 1u, is_eq = (eqb[blk] >> (i & 31)) & 1u;
-            const int sl = slot[i * NW + warp];
-            bool keep = is_gt || is_eq;
-            if (ties) {
-                const unsigned be = __ballot_sync(0xffffffffu, is_eq);
-                keep = is_gt || (is_eq && __popc(be & lt) < (sl >> 24));
-            }
-            const unsigned bk = __ballot_sync(0xffffffffu, keep);
-            if (keep) out[ns + (sl & 0xffffff) + __popc(bk & lt)] = ns + j_lo + i * kSelThreads + tid;
-        }
+        const unsigned bk = __ballot_sync(0xffffffffu, keep);
+        if (keep) out[pos + __popc(bk & lt)] = ns + j_lo + j0 + lane;
+        pos += __popc(bk);
     }
 }
 
 // Streams with more candidates than a cluster's shared memory holds: keys are re-read from L2 in every pass
 // (4 passes of 8 bits), and each thread emits a contiguous token range.
-__global__ void __launch_bounds__(kSelThreads)
+__global__ void __launch_bounds__(kSelStreamThreads)
 select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* __restrict__ idx, int trigger_late) {
     if (!trigger_late) grid_dep_launch_dependents();
     grid_dep_wait();
@@ -340,14 +409,14 @@ select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* 
             const int shift = 24 - 8 * pass;
             if (tid < 256) hist[tid] = 0;
             __syncthreads();
-            for (int t0 = c0 + tid; t0 < c1; t0 += kSelThreads * kSelBatch) {
+            for (int t0 = c0 + tid; t0 < c1; t0 += kSelStreamThreads * kSelBatch) {
                 float v[kSelBatch];                      // the batch's loads are in flight together
 #pragma unroll
-                for (int u = 0; u < kSelBatch; ++u) v[u] = t0 + u * kSelThreads < c1 ? __ldg(sc + t0 + u * kSelThreads) : 0.f;
+                for (int u = 0; u < kSelBatch; ++u) v[u] = t0 + u * kSelStreamThreads < c1 ? __ldg(sc + t0 + u * kSelStreamThreads) : 0.f;
 #pragma unroll
                 for (int u = 0; u < kSelBatch; ++u) {
                     const uint32_t key = score_key(v[u]);
-                    if (t0 + u * kSelThreads < c1 && (key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
+                    if (t0 + u * kSelStreamThreads < c1 && (key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
                 }
             }
             __syncthreads();
@@ -383,7 +452,7 @@ select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* 
     }
 
     // ---- ordered emission
-    const int per = (T + kSelThreads - 1) / kSelThreads;
+    const int per = (T + kSelStreamThreads - 1) / kSelStreamThreads;
     const int t0 = min(T, tid * per), t1 = min(T, t0 + per);
     int eqc = 0;
     for (int t = max(t0, c0); t < min(t1, c1); ++t) eqc += (score_key(sc[t]) == thr);
@@ -414,14 +483,14 @@ select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* 
 
 namespace {
 constexpr size_t kSelSmemMax = 227 * 1024 - 1024;            // dynamic shared memory a CTA may ask for (static part left out)
-static_assert((size_t)kSelCapCta * 4 + kSelListCap * 4 + kSelHistBins * 4 * 2 <= kSelSmemMax, "a CTA's share does not fit");
-// (round, warp) pairs of the emission: two bytes each in one histogram buffer, one int each in the list
-static_assert((kSelCapCta / kSelThreads) * (kSelThreads / 32) * 2 <= kSelHistBins * 4 &&
-              (kSelCapCta / kSelThreads) * (kSelThreads / 32) <= kSelListCap && kSelCapCta / kSelThreads <= 64,
-              "pair tables outgrow their buffers");
+constexpr size_t kSelFixedBytes = (size_t)(2 * kSelBins + (kSelCluster + 1) * kSelList) * 4;
+static_assert((size_t)kSelCapCta * 4 + kSelFixedBytes <= kSelSmemMax, "a CTA's share does not fit");
 }  // namespace
 
 namespace {
+// Candidates a CTA: most before the cluster doubles, and most for a block of 256 threads (2000 candidates: 6.9 us in 256 threads, 5.8 in 1024; 444:
+// 4.3 and 8.5).
+constexpr int64_t kSelShare = 4096, kSelShort = 1024;
 struct SelLaunch {
     bool any_cluster = false, any_stream = false;
     int nc = 1;
@@ -438,11 +507,11 @@ SelLaunch plan_select(const StreamTable& st) {
         pl.any_cluster = true;
         if (M > m_max) m_max = M;
     }
-    // CTAs per stream.  A barrier across CTAs and the trip through distributed shared memory cost
-    // more than a few rounds over the candidates: one CTA up to 24 rounds (24 576 candidates: the
-    // 28 080-token cache), then as many as keep a CTA's share near 16 rounds.
-    while (pl.nc < kSelCluster && m_max > (int64_t)pl.nc * (pl.nc == 1 ? 24576 : 16384)) pl.nc *= 2;
-    pl.per_cta = (m_max + pl.nc * kSelThreads - 1) / (pl.nc * kSelThreads) * kSelThreads;
+    // CTAs per stream.  A histogram of 1024 candidates costs a CTA some 400 clocks (13 an add and warp, whether or not its
+    // lanes collide), the barriers across CTAs and the trips through distributed shared memory two to three thousand: 7800 candidates
+    // 9.4 us on one CTA, 7.9 on two, 7.4 on four; 16 000 10.2 on two, 8.4 on four.
+    while (pl.nc < kSelCluster && m_max > (int64_t)pl.nc * kSelShare) pl.nc *= 2;
+    pl.per_cta = ((m_max + pl.nc - 1) / pl.nc + 31) / 32 * 32;
     return pl;
 }
 }  // namespace
@@ -462,13 +531,14 @@ pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* i
             }))
             return PAFU_ERR_CUDA;
         const int32_t keys_bytes = (int32_t)(pl.per_cta * 4);
-        const size_t smem = (size_t)keys_bytes + kSelListCap * 4 + kSelHistBins * 4 * 2;
-        if (launch_dependent(select_cluster_kernel, dim3((unsigned)(st.n_streams * pl.nc)), dim3(kSelThreads), smem, stream,
+        const size_t smem = (size_t)keys_bytes + kSelFixedBytes;
+        if (launch_dependent(select_cluster_kernel, dim3((unsigned)(st.n_streams * pl.nc)),
+                             dim3(pl.per_cta <= kSelShort ? kSelThreads : kSelThreadsMax), smem, stream,
                              (unsigned)pl.nc, scores, st, keys_bytes, idx, trigger_late) != cudaSuccess)
             return PAFU_ERR_CUDA;
     }
     if (pl.any_stream &&
-        launch_dependent(select_stream_kernel, dim3((unsigned)st.n_streams), dim3(kSelThreads), 0, stream, 1, scores, st,
+        launch_dependent(select_stream_kernel, dim3((unsigned)st.n_streams), dim3(kSelStreamThreads), 0, stream, 1, scores, st,
                          idx, trigger_late) != cudaSuccess)
         return PAFU_ERR_CUDA;
     return PAFU_OK;

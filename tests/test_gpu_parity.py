@@ -164,6 +164,34 @@ def test_select_bit_exact(kind):
             assert np.array_equal(got[cu_B[st]:cu_B[st + 1]], want), (kind, ci, st)
 
 
+@pytest.mark.parametrize("kind", ["steps", "equal", "outlier", "two_values", "one_bin_256", "one_bin_257", "denormal", "infinite"])
+def test_select_histogram_routes(kind):
+    """Sizes around what one warp, one block and 1, 2, 4, 8 CTAs take, with scores that spread over the value histogram, that
+    fall into one bin of it (as many as are ranked directly, and one more), and that leave it no finite range."""
+    rng = np.random.default_rng(11)
+    for M in (1, 2, 31, 33, 255, 257, 600, 1024, 1025, 4096, 4097, 8193, 16385, 33000):
+        s = rng.standard_normal(M + 5).astype(np.float32)
+        if kind == "equal":
+            s[:] = 0.25
+        elif kind == "outlier":
+            s[::256] = 1e30
+        elif kind == "two_values":
+            s = np.where(s > 0, np.float32(1), np.float32(-1))
+        elif kind.startswith("one_bin"):
+            s = (100 * np.sign(s) + s).astype(np.float32)
+            n = min(int(kind[-3:]), M)
+            s[3 + rng.permutation(M)[:n]] = (0.01 * rng.standard_normal(n)).astype(np.float32)
+        elif kind == "denormal":
+            s *= np.float32(1e-44)
+        elif kind == "infinite":
+            s = rng.choice(np.array([np.inf, -np.inf, np.nan, 3.4e38, -3.4e38], np.float32), M + 5)
+        for k in sorted({1, M // 3, M // 2, M - 1} - {0}):
+            shape = pafu.Shape(1, 64, [0, M + 5], None)
+            idx = torch.full((k + 5,), -1, dtype=torch.int32, device="cuda")
+            pafu.pafu_select(torch.from_numpy(s).cuda(), shape, pafu.make_policy(3, 2, [k + 5], 1), idx)
+            assert np.array_equal(idx.cpu().numpy(), oracle.select(s, 3, 2, k + 5)), (kind, M, k)
+
+
 # ------------------------------------------------------------------------------- compact
 @pytest.mark.parametrize("w", SMALL + [wl.Workload("odd_dm", 7, 5, 8, (77, 9), (30, 9), 2, 3, (4, 4), 32)],
                          ids=lambda w: "%s-dm%d" % (w.name, w.d_model))
