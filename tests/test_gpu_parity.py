@@ -268,6 +268,37 @@ def test_attention_segment_edge_cases():
             close(LSE.cpu().numpy(), wl_, "edge LSE")
 
 
+@pytest.mark.parametrize("kind", ["one_run", "runs", "steps_of_two", "unsorted", "ragged_run"])
+def test_indexed_attention_takes_runs_tiled(kind):
+    """Tiles of neighbouring cache rows are loaded tiled, all others row by row: the same bits as on gathered rows."""
+    g = torch.Generator(device="cuda"); g.manual_seed(7)
+    N, D, Lq = 3, 128, (200, 300)
+    T = (900, 700)
+    rn = lambda n: torch.randn(n, N, D, generator=g, device="cuda").to(torch.bfloat16)
+    K, V, Q, Kq, Vq = rn(sum(T)), rn(sum(T)), rn(sum(Lq)), rn(sum(Lq)), rn(sum(Lq))
+    ar = lambda a, b: torch.arange(a, b, device="cuda")
+    lists = []
+    for t in T:
+        lists.append({"one_run": ar(37, 37 + 512), "runs": torch.cat([ar(0, 100), ar(130, 400), ar(401, 430)]),
+                      "steps_of_two": ar(0, 256) * 2, "unsorted": torch.cat([ar(300, 428), ar(0, 64).flip(0), ar(64, 128)]),
+                      "ragged_run": ar(t - 421, t)}[kind])
+    cu_B = np.concatenate([[0], np.cumsum([len(i) for i in lists])])
+    idx = torch.cat(lists).to(torch.int32)
+    rows = torch.cat([lists[0], lists[1] + T[0]])
+    shape = pafu.Shape(N, D, np.concatenate([[0], np.cumsum(T)]), np.concatenate([[0], np.cumsum(Lq)]))
+    ws = torch.zeros(pafu.pafu_workspace_bytes(shape), dtype=torch.uint8, device="cuda")
+    out = []
+    for indexed in (False, True):
+        O, LSE = torch.zeros_like(Q), torch.zeros(N, sum(Lq), device="cuda")
+        if indexed:
+            pafu.pafu_chunk_attn_indexed(Q, K, V, idx, cu_B, Kq, Vq, shape, 0.0, O, LSE, ws)
+        else:
+            pafu.pafu_chunk_attn(Q, K[rows].contiguous(), V[rows].contiguous(), cu_B, Kq, Vq, shape, 0.0, O, LSE, ws)
+        assert pafu.pafu_workspace_status(ws) == 0
+        out.append((O, LSE))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
 # ---------------------------------- peaked attention: the running maximum has to move (Sec. 3.2)
 def _attention_all_entry_points(d, N, D, Lq, nB, what, seed=0):
     """One set of inputs through pafu_chunk_attn, pafu_chunk_attn_indexed (the retained rows
