@@ -43,6 +43,38 @@ __device__ __forceinline__ void copy_kv_row(const uint4* __restrict__ K, const u
     if (SLc != nullptr && lane == 0) SLc[dst_row] = __ldg(SL + src_row);
 }
 
+// The same for `count` rows that are narrower than what a warp keeps in flight, laid end to end: lane l < count knows row l's
+// source and destination, and unit u = i * 32 + lane of the stretch, which belongs to row u / chunks_per_row (bits 5 i .. 5 i + 4 of
+// `row_of`), takes them from that lane.  (K, V, Kc and Vc hold less than 2^32 units each: the host sees to it.)
+__device__ __forceinline__ uint32_t rows_of_units(int chunks_per_row, int lane) {
+    uint32_t r = 0;
+#pragma unroll
+    for (int i = 0; i < kCompactUnroll; ++i) r |= (uint32_t)min((i * 32 + lane) / chunks_per_row, 31) << (5 * i);
+    return r;
+}
+__device__ __forceinline__ void copy_kv_rows(const uint4* __restrict__ K, const uint4* __restrict__ V,
+                                             const float* __restrict__ SL, int64_t src_row, int64_t dst_row, int count,
+                                             int chunks_per_row, uint4* __restrict__ Kc, uint4* __restrict__ Vc,
+                                             float* __restrict__ SLc, int lane, uint32_t row_of) {
+    static_assert(kCompactUnroll <= 6, "row_of holds six rows");
+    const int units = count * chunks_per_row;
+    const uint32_t src = (uint32_t)(src_row - lane) * chunks_per_row + lane, dst = (uint32_t)(dst_row - lane) * chunks_per_row + lane;
+    uint4 kb[kCompactUnroll], vb[kCompactUnroll];
+#pragma unroll
+    for (int i = 0; i < kCompactUnroll; ++i) {
+        const int from = (row_of >> (5 * i)) & 31;
+        const uint32_t s = __shfl_sync(0xffffffffu, src, from) - from + lane + i * 32;
+        if (i * 32 + lane < units) { kb[i] = ld_nc_v4(K + s); vb[i] = ld_nc_v4(V + s); }
+    }
+#pragma unroll
+    for (int i = 0; i < kCompactUnroll; ++i) {
+        const int from = (row_of >> (5 * i)) & 31;
+        const uint32_t d = __shfl_sync(0xffffffffu, dst, from) - from + lane + i * 32;
+        if (i * 32 + lane < units) { Kc[d] = kb[i]; Vc[d] = vb[i]; }
+    }
+    if (SLc != nullptr && lane < count) SLc[dst_row] = __ldg(SL + src_row);
+}
+
 // always_first = 0: wait for the preceding kernel, then copy every kept row through the index list.
 // always_first = 1 (inside a layer step, directly behind the selection kernels, which let their
 // dependents start at once): the rows that are kept whatever the scores say - sink and recent
@@ -52,7 +84,7 @@ __device__ __forceinline__ void copy_kv_row(const uint4* __restrict__ K, const u
 // not read by them, so the early part touches nothing the predecessor produces.  (SL is the
 // score array in a step: all of its entries are copied after the wait.)
 // When the selection occupies more than kStaticSelect SMs, rows are handed out through two counters in the
-// workspace header (`work`: early rows, late rows, finished blocks), one row per claim with the
+// workspace header (`work`: early rows, late rows, finished blocks), a row or a group per claim with the
 // next claim under way during the copy: the blocks that only get an SM when the selection's CTAs
 // leave simply find less work left, instead of starting a fixed share late (that tail cost 40 us
 // at the batch-4 size); the last block to finish puts the counters back to zero.  With a selection
@@ -60,31 +92,49 @@ __device__ __forceinline__ void copy_kv_row(const uint4* __restrict__ K, const u
 // selection and gather of the 28 080-token cache, selected by eight CTAs, 39.6 us with claiming, 31.4 with shares; of the
 // 93 600-token one 33.5 and 29.3; four streams, 32 CTAs: no difference).
 constexpr int kStaticSelect = 8;
-constexpr int kCompactClaim = 1;
 
 // A claim in two halves: lane 0 issues the add; its result is fetched (and shared with the warp)
 // only when the rows are needed, so the trip to L2 overlaps the copying in between.
-__device__ __forceinline__ int claim_issue(int* counter, int lane) {
-    return lane == 0 ? atomicAdd(counter, kCompactClaim) : 0;
+__device__ __forceinline__ int claim_issue(int* counter, int group, int lane) {
+    return lane == 0 ? atomicAdd(counter, group) : 0;
 }
 __device__ __forceinline__ int64_t claim_get(int pending) { return __shfl_sync(0xffffffffu, pending, 0); }
 
-__global__ void __launch_bounds__(kCompactWarpsPerBlock * 32)
+// GROUPS: a warp copies `rows_at_once` narrow rows at a time.  A narrow row alone leaves most of a warp's batch empty: 48 000 rows
+// of 256 bytes, selected from 76 000 in four streams, selection and gather together 56 us, in groups of 12 rows 29.4; 24 000
+// rows of 1280 bytes 45.7 and 39.6.
+template <bool GROUPS>
+__global__ void __launch_bounds__(kCompactWarpsPerBlock * 32, 3)
 compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
                     const float* __restrict__ SL, const int32_t* idx,
                     const __grid_constant__ StreamTable st, int32_t chunks_per_row,
                     uint4* __restrict__ Kc, uint4* __restrict__ Vc, float* __restrict__ SLc,
-                    int64_t n_rows, int* __restrict__ work, int early_static) {
+                    int64_t n_rows, int* __restrict__ work, int early_static, int rows_at_once) {
+    const int group = GROUPS ? rows_at_once : 1;
     const int lane = threadIdx.x & 31;
+    const uint32_t row_of = GROUPS ? rows_of_units(chunks_per_row, lane) : 0u;
     const int64_t warp0 = (int64_t)blockIdx.x * kCompactWarpsPerBlock + (threadIdx.x >> 5);
     const int64_t n_warps = (int64_t)gridDim.x * kCompactWarpsPerBlock;
+    // rows [base, base + group) of n: `where` says where row i comes from and goes to
+    auto copy = [&](int64_t base, int64_t n, auto where, const float* from, float* to) {
+        int64_t src, dst;
+        if constexpr (!GROUPS) {
+            where(base, src, dst);
+            copy_kv_row(K, V, from, src, dst, chunks_per_row, Kc, Vc, to, lane);
+        } else {
+            const int count = (int)(n - base < group ? n - base : group);
+            where(base + (lane < count ? lane : 0), src, dst);
+            copy_kv_rows(K, V, from, src, dst, count, chunks_per_row, Kc, Vc, to, lane, row_of);
+        }
+    };
     if (work == nullptr) {
         grid_dep_wait();
-        for (int64_t r = warp0; r < n_rows; r += n_warps) {
+        auto kept = [&](int64_t r, int64_t& src, int64_t& dst) {
             int s = 0;
             while (s + 1 < st.n_streams && r >= st.cu_B[s + 1]) ++s;
-            copy_kv_row(K, V, SL, st.cu_T[s] + (int64_t)ld_index(idx + r), r, chunks_per_row, Kc, Vc, SLc, lane);
-        }
+            src = st.cu_T[s] + (int64_t)ld_index(idx + r); dst = r;
+        };
+        for (int64_t r = warp0 * group; r < n_rows; r += n_warps * group) copy(r, n_rows, kept, SL, SLc);
         return;
     }
     // part 1: always-kept rows, enumerated stream by stream (A_s = n_sink + n_recent of them, or all T)
@@ -93,7 +143,7 @@ compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
         const int64_t T = st.cu_T[s + 1] - st.cu_T[s], B = st.cu_B[s + 1] - st.cu_B[s];
         n_always += B >= T ? T : st.n_sink[s] + st.n_recent[s];
     }
-    auto copy_always = [&](int64_t a) {
+    auto always = [&](int64_t a, int64_t& src, int64_t& dst) {
         int s = 0;
         int64_t p = a;
         for (;; ++s) {
@@ -105,15 +155,14 @@ compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
         const int64_t T = st.cu_T[s + 1] - st.cu_T[s], B = st.cu_B[s + 1] - st.cu_B[s];
         const int64_t ns = B >= T ? T : st.n_sink[s], k = B >= T ? 0 : st.k[s], A = B >= T ? T : ns + st.n_recent[s];
         // position p < ns is token p; position ns + k + i is token T - n_recent + i
-        const int64_t pos = p < ns ? p : p + k, tok = p < ns ? p : T - A + p;
-        copy_kv_row(K, V, nullptr, st.cu_T[s] + tok, st.cu_B[s] + pos, chunks_per_row, Kc, Vc, nullptr, lane);
+        src = st.cu_T[s] + (p < ns ? p : T - A + p); dst = st.cu_B[s] + (p < ns ? p : p + k);
     };
-    auto copy_top = [&](int64_t q) {
+    auto top = [&](int64_t q, int64_t& src, int64_t& dst) {
         int s = 0;
         int64_t p = q;
         for (; p >= st.k[s]; ++s) p -= st.k[s];
-        const int64_t r = st.cu_B[s] + st.n_sink[s] + p;
-        copy_kv_row(K, V, SL, st.cu_T[s] + (int64_t)ld_index(idx + r), r, chunks_per_row, Kc, Vc, SLc, lane);
+        dst = st.cu_B[s] + st.n_sink[s] + p;
+        src = st.cu_T[s] + (int64_t)ld_index(idx + dst);
     };
     int64_t n_top = 0;
     for (int s = 0; s < st.n_streams; ++s) n_top += st.k[s];
@@ -128,24 +177,24 @@ compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
     };
     if (early_static) {
         // every block is resident from the start (the launcher sized the grid for it): fixed shares
-        for (int64_t a = warp0; a < n_always; a += n_warps) copy_always(a);
+        for (int64_t a = warp0 * group; a < n_always; a += n_warps * group) copy(a, n_always, always, nullptr, nullptr);
         grid_dep_wait();
         fill_always_sl();
-        for (int64_t q = warp0; q < n_top; q += n_warps) copy_top(q);
+        for (int64_t q = warp0 * group; q < n_top; q += n_warps * group) copy(q, n_top, top, SL, SLc);
         return;
     }
-    int pending = claim_issue(work + 0, lane);
+    int pending = claim_issue(work + 0, group, lane);
     for (int64_t base = claim_get(pending); base < n_always; base = claim_get(pending)) {
-        pending = claim_issue(work + 0, lane);
-        for (int64_t a = base; a < base + kCompactClaim && a < n_always; ++a) copy_always(a);
+        pending = claim_issue(work + 0, group, lane);
+        copy(base, n_always, always, nullptr, nullptr);
     }
     // part 2: the selection's result
     grid_dep_wait();
     fill_always_sl();
-    pending = claim_issue(work + 1, lane);
+    pending = claim_issue(work + 1, group, lane);
     for (int64_t base = claim_get(pending); base < n_top; base = claim_get(pending)) {
-        pending = claim_issue(work + 1, lane);
-        for (int64_t q = base; q < base + kCompactClaim && q < n_top; ++q) copy_top(q);
+        pending = claim_issue(work + 1, group, lane);
+        copy(base, n_top, top, SL, SLc);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -322,7 +371,6 @@ pafu_status launch_compact(const uint16_t* K, const uint16_t* V, const float* SL
     const int64_t n_rows = st.cu_B[st.n_streams];
     if (n_rows == 0) return PAFU_OK;
     const int32_t chunks = d_model / 8;
-    int64_t blocks = (n_rows + kCompactWarpsPerBlock - 1) / kCompactWarpsPerBlock;
     // A few resident waves, larger inputs loop.  With the early part the grid is what the device
     // holds at once (three blocks fit on an SM): a block must not queue behind blocks that are
     // waiting for the selection.  Fixed shares: the selection's SMs are left out of the count.
@@ -330,11 +378,19 @@ pafu_status launch_compact(const uint16_t* K, const uint16_t* V, const float* SL
     int sms = device_sm_count() - (early_static ? select_ctas : 0);
     if (sms < 1) sms = 1;
     const int64_t max_blocks = work != nullptr ? (int64_t)sms * 3 : 148 * 8 * 4;
+    // Rows a warp copies at once: as many as fill its batch, but no more than leave every warp some, and one where a warp has but one
+    // or two (10 280 rows of 512 bytes in pairs: 48.5 us a step, one by one 47.7).
+    const int64_t resident = (int64_t)device_sm_count() * 3 * kCompactWarpsPerBlock;
+    int64_t group = kCompactUnroll * 32 / chunks;
+    if (group > n_rows / resident) group = n_rows / resident;
+    if (group > 32) group = 32;
+    if (group < 1 || n_rows < 3 * resident || st.cu_T[st.n_streams] * chunks >= (int64_t)1 << 32) group = 1;   // (32-bit unit numbers in groups)
+    int64_t blocks = (n_rows + kCompactWarpsPerBlock * group - 1) / (kCompactWarpsPerBlock * group);
     if (blocks > max_blocks) blocks = max_blocks;
-    return cuda_ok(launch_dependent(compact_rows_kernel, dim3((unsigned)blocks), dim3(kCompactWarpsPerBlock * 32), 0, stream, 1,
+    return cuda_ok(launch_dependent(group > 1 ? compact_rows_kernel<true> : compact_rows_kernel<false>, dim3((unsigned)blocks), dim3(kCompactWarpsPerBlock * 32), 0, stream, 1,
                                     reinterpret_cast<const uint4*>(K), reinterpret_cast<const uint4*>(V), SL, idx, st,
                                     chunks, reinterpret_cast<uint4*>(Kc), reinterpret_cast<uint4*>(Vc), SLc, n_rows, work,
-                                    early_static));
+                                    early_static, (int)group));
 }
 
 }  // namespace pafu

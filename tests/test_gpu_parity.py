@@ -220,6 +220,26 @@ def test_compact_bit_exact(w):
     assert np.array_equal(bf16_to_bits(K), d["K"]) and np.array_equal(bf16_to_bits(V), d["V"])
 
 
+@pytest.mark.parametrize("d_head,n_heads,T,B", [
+    (64, 1, (47000,), (45000,)),                            # rows of 8 pieces: 12 at once, one selecting cluster
+    (64, 1, (9000, 700, 9, 40000), (9000, 650, 0, 39999)),  # four streams, one kept whole, one empty: rows are claimed
+    (64, 3, (12000,), (11111,)),                            # 24 pieces, the last group short
+    (128, 6, (11000,), (10700,)),                           # 96 pieces: one row at a time
+], ids=lambda v: str(v) if isinstance(v, int) else "x".join(map(str, v)))
+def test_gather_of_narrow_rows(d_head, n_heads, T, B):
+    """The row gather's groups of rows, behind the selection inside a step and by itself: every kept row and score is a copy."""
+    w = wl.Workload("narrow", 8, n_heads, d_head, T, B, 7, 9, (64,) * len(T), 32)
+    L = Layer(w, wl.make_layer_device(w, seed=3))
+    L.step(); L.check_status()
+    cuT, cuB = w.cu("T"), L.cu_B
+    idx = torch.cat([L.idx[cuB[s]:cuB[s + 1]].long() + int(cuT[s]) for s in range(len(T))])
+    for again in range(2):
+        assert torch.equal(L.Kc[:L.nB], L.K[idx]) and torch.equal(L.Vc[:L.nB], L.V[idx])
+        assert torch.equal(L.SLc[:L.nB], L.scores[idx])
+        L.Kc.zero_(); L.Vc.zero_(); L.SLc.zero_()
+        L.compact()
+
+
 # ----------------------------------------------------------------------------- attention
 @pytest.mark.parametrize("w", SMALL, ids=lambda w: "%s-d%d" % (w.name, w.d_head))
 def test_attention_matches_oracle_everywhere(w):
