@@ -447,10 +447,14 @@ static pafu_status step_impl(const pafu_step_args* a, void* const* ev, void* str
         // once the indices exist.  No event may sit between the two launches, so in the timed
         // variant the "after select" stamp is taken before them.
         if (!mark(2)) return PAFU_ERR_CUDA;
-        e = launch_select(a->scores, st, a->idx, cs);
-        if (e != PAFU_OK) return e;
-        e = launch_compact(a->K, a->V, a->SLc ? a->scores : nullptr, a->idx, st, (int32_t)dm, a->Kc, a->Vc, a->SLc, cs,
-                           static_cast<int*>(a->ws) + kStatusWordGatherWork, select_cta_count(st));
+        bool done = false;
+        e = launch_select_compact(a->K, a->V, a->scores, st, (int32_t)dm, a->idx, a->Kc, a->Vc, a->SLc, cs, &done);
+        if (e == PAFU_OK && !done) {
+            e = launch_select(a->scores, st, a->idx, cs);
+            if (e == PAFU_OK)
+                e = launch_compact(a->K, a->V, a->SLc ? a->scores : nullptr, a->idx, st, (int32_t)dm, a->Kc, a->Vc, a->SLc, cs,
+                                   static_cast<int*>(a->ws) + kStatusWordGatherWork, select_cta_count(st));
+        }
         if (e != PAFU_OK) return e;
     } else {
         e = pafu_select(a->scores, &a->shape, a->policy, a->idx, a->ws, a->ws_bytes, stream);

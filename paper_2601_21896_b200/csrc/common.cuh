@@ -123,6 +123,9 @@ pafu_status launch_score(const pafu_head& head, const uint16_t* const* X, int n_
 // selection is complete
 pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx,
                           cudaStream_t stream, int trigger_late = 0);
+// Selection and row gather of a small step in one launch; *done = false: the step is not small, nothing was launched.
+pafu_status launch_select_compact(const uint16_t* K, const uint16_t* V, const float* scores, const StreamTable& st, int32_t d_model, int32_t* idx,
+                                  uint16_t* Kc, uint16_t* Vc, float* SLc, cudaStream_t stream, bool* done);
 int select_cta_count(const StreamTable& st);      // CTAs launch_select's kernels occupy for this geometry
 // work != nullptr (three zeroed words of the workspace header): the rows that are kept whatever
 // the scores say are copied before the kernel waits for its predecessor (only valid when that

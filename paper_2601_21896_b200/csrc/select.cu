@@ -81,6 +81,12 @@ __device__ __forceinline__ int sel_exclusive_scan(int v, int* warp_sums, int* to
     return warp_sums[warp] + inc - v;
 }
 
+namespace {
+constexpr size_t kSelSmemMax = 227 * 1024 - 1024;            // dynamic shared memory a CTA may ask for (static part left out)
+constexpr size_t kSelFixedBytes = (size_t)(2 * kSelBins + (kSelCluster + 1) * kSelList) * 4;
+static_assert((size_t)kSelCapCta * 4 + kSelFixedBytes <= kSelSmemMax, "a CTA's share does not fit");
+}  // namespace
+
 // The score a key stands for (a NaN for key 0).
 __device__ __forceinline__ float key_score(uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); }
 
@@ -143,16 +149,16 @@ __device__ __forceinline__ void find_bin(cg::cluster_group& cluster, int nc, Sel
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSelThreadsMax, 1)
-select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ StreamTable st, int32_t keys_bytes,
-                      int32_t* __restrict__ idx, int trigger_late) {
-    extern __shared__ __align__(16) unsigned char sel_smem[];
-    __shared__ SelShared sh;
-    if (!trigger_late) grid_dep_launch_dependents();
+// The selection of stream s by the CTAs of a cluster, or (ALONE) by one CTA for itself: `copies` CTAs then select the same stream
+// side by side, number `copy` of them writes its share of the always-kept indices, number 0 the top-k ones, and every one
+// leaves the top-k tokens in its shared memory (`top`).
+template <bool ALONE>
+__device__ __forceinline__ void select_stream(const float* __restrict__ scores, const StreamTable& st, int s, int copy, int copies, int32_t keys_bytes,
+                                              int32_t* __restrict__ idx, int trigger_late, unsigned char* sel_smem, SelShared& sh, int* top) {
+    if (!ALONE && !trigger_late) grid_dep_launch_dependents();
     cg::cluster_group cluster = cg::this_cluster();
-    const int nc = (int)cluster.num_blocks();                // 1, 2, 4 or 8: the host's choice for this launch
-    const int s = blockIdx.x / nc;
-    const int rank = (int)cluster.block_rank();
+    const int nc = ALONE ? 1 : (int)cluster.num_blocks();    // 1, 2, 4 or 8: the host's choice for this launch
+    const int rank = ALONE ? 0 : (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int threads = (int)blockDim.x, warps = threads >> 5;
     uint32_t* keys = reinterpret_cast<uint32_t*>(sel_smem);
@@ -169,7 +175,7 @@ select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ 
     const float* first = scores + st.cu_T[s] + ns;
     int32_t* out = idx + st.cu_B[s];
     grid_dep_wait();
-    if (trigger_late) grid_dep_launch_dependents();
+    if (!ALONE && trigger_late) grid_dep_launch_dependents();
     // cluster-uniform exits (before any cluster barrier)
     if (B == 0) return;
     if (M > nc * kSelCapCta) return;                         // the streaming kernel owns this stream
@@ -196,8 +202,8 @@ select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ 
         const uint32_t lo_w = __reduce_min_sync(0xffffffffu, finite ? ks : 0xffffffffu), hi_w = __reduce_max_sync(0xffffffffu, finite ? ks : 0u);
         if (lane == 0) { sh.lo[warp] = lo_w; sh.hi[warp] = hi_w; }
     }
-    // always-kept tokens (spread over the cluster): position p < ns is token p, position ns + k + i is token T - nr + i
-    for (int p = rank * threads + tid; p < ns + nr; p += nc * threads) {
+    // always-kept tokens (spread over the cluster, or the CTAs side by side): position p < ns is token p, position ns + k + i is token T - nr + i
+    for (int p = (ALONE ? copy : rank) * threads + tid; p < ns + nr; p += (ALONE ? copies : nc) * threads) {
         if (p < ns) out[p] = p; else out[p + k] = T - (ns + nr) + p;
     }
     if (k == 0) return;
@@ -368,9 +374,66 @@ select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ 
             eq_before += __popc(be);
         }
         const unsigned bk = __ballot_sync(0xffffffffu, keep);
-        if (keep) out[pos + __popc(bk & lt)] = ns + j_lo + j0 + lane;
+        if (keep) {
+            if (ALONE) top[pos - ns + __popc(bk & lt)] = ns + j0 + lane;
+            if (!ALONE || copy == 0) out[pos + __popc(bk & lt)] = ns + j_lo + j0 + lane;
+        }
         pos += __popc(bk);
     }
+}
+
+__global__ void __launch_bounds__(kSelThreadsMax, 1)
+select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ StreamTable st, int32_t keys_bytes,
+                      int32_t* __restrict__ idx, int trigger_late) {
+    extern __shared__ __align__(16) unsigned char sel_smem[];
+    __shared__ SelShared sh;
+    select_stream<false>(scores, st, blockIdx.x / cg::this_cluster().num_blocks(), 0, 1, keys_bytes, idx, trigger_late, sel_smem, sh, nullptr);
+}
+
+// Selection and row gather of a small layer step in one launch: `copies` CTAs per stream all make the stream's whole selection (a
+// few microseconds, whoever does it) and then copy a share of its rows each, without a word between them.  What it
+// saves is the second kernel's start: a step of 2 heads x 64 over 512 tokens 19.0 -> 17.2 us, 4 x 64 over 600 25.5 -> 23.8, 5 x 128 over 1800 +
+// 2500 37.5 -> 37.0, 12 x 128 over 3000 (18 MB in and out) 54.1 -> 53.1.  Larger steps keep two launches: their always-kept rows are
+// copied while the selection runs.
+constexpr int kSelCopyBatch = 4;            // 16-byte pieces of K and of V a thread has in flight
+__global__ void __launch_bounds__(kSelThreadsMax, 1)
+select_copy_kernel(const float* __restrict__ scores, const __grid_constant__ StreamTable st, int32_t keys_bytes,
+                   int32_t* __restrict__ idx, int copies, const uint4* __restrict__ K, const uint4* __restrict__ V,
+                   int chunks_per_row, uint4* __restrict__ Kc, uint4* __restrict__ Vc, float* __restrict__ SLc) {
+    extern __shared__ __align__(16) unsigned char sel_smem[];
+    __shared__ SelShared sh;
+    const int s = blockIdx.x / copies, copy = blockIdx.x % copies, threads = (int)blockDim.x;
+    int* top = reinterpret_cast<int*>(sel_smem + keys_bytes + kSelFixedBytes);
+    select_stream<true>(scores, st, s, copy, copies, keys_bytes, idx, 0, sel_smem, sh, top);
+    __syncthreads();
+    const int T = (int)(st.cu_T[s + 1] - st.cu_T[s]), B = (int)(st.cu_B[s + 1] - st.cu_B[s]);
+    const bool everything = B >= T;
+    const int ns = everything ? T : (int)st.n_sink[s], k = everything ? 0 : (int)st.k[s];
+    auto token = [&](int r) { return r < ns ? r : r < ns + k ? top[r - ns] : T - B + r; };
+    const uint4* Ks = K + st.cu_T[s] * chunks_per_row;
+    const uint4* Vs = V + st.cu_T[s] * chunks_per_row;
+    uint4* Kd = Kc + st.cu_B[s] * chunks_per_row;
+    uint4* Vd = Vc + st.cu_B[s] * chunks_per_row;
+    const int units = B * chunks_per_row, step = copies * threads;
+    for (int u0 = copy * threads + (int)threadIdx.x; u0 < units; u0 += step * kSelCopyBatch) {
+        uint4 kb[kSelCopyBatch], vb[kSelCopyBatch];
+#pragma unroll
+        for (int i = 0; i < kSelCopyBatch; ++i) {
+            const int u = u0 + i * step;
+            if (u < units) {
+                const int row = u / chunks_per_row;
+                const int64_t src = (int64_t)token(row) * chunks_per_row + (u - row * chunks_per_row);
+                kb[i] = __ldg(Ks + src); vb[i] = __ldg(Vs + src);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kSelCopyBatch; ++i) {
+            const int u = u0 + i * step;
+            if (u < units) { Kd[u] = kb[i]; Vd[u] = vb[i]; }
+        }
+    }
+    if (SLc != nullptr)
+        for (int r = copy * threads + (int)threadIdx.x; r < B; r += step) SLc[st.cu_B[s] + r] = __ldg(scores + st.cu_T[s] + token(r));
 }
 
 // Streams with more candidates than a cluster's shared memory holds: keys are re-read from L2 in every pass
@@ -482,15 +545,10 @@ select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* 
 }
 
 namespace {
-constexpr size_t kSelSmemMax = 227 * 1024 - 1024;            // dynamic shared memory a CTA may ask for (static part left out)
-constexpr size_t kSelFixedBytes = (size_t)(2 * kSelBins + (kSelCluster + 1) * kSelList) * 4;
-static_assert((size_t)kSelCapCta * 4 + kSelFixedBytes <= kSelSmemMax, "a CTA's share does not fit");
-}  // namespace
-
-namespace {
 // Candidates a CTA: most before the cluster doubles, and most for a block of 256 threads (2000 candidates: 6.9 us in 256 threads, 5.8 in 1024; 444:
 // 4.3 and 8.5).
 constexpr int64_t kSelShare = 4096, kSelShort = 1024;
+constexpr int64_t kSelCopyBytes = 64 << 20;
 struct SelLaunch {
     bool any_cluster = false, any_stream = false;
     int nc = 1;
@@ -519,6 +577,32 @@ SelLaunch plan_select(const StreamTable& st) {
 int select_cta_count(const StreamTable& st) {
     const SelLaunch pl = plan_select(st);
     return (pl.any_cluster ? st.n_streams * pl.nc : 0) + (pl.any_stream ? st.n_streams : 0);
+}
+
+// A step is small when one CTA selects each stream and the rows, K and V in and out, are kSelCopyBytes at most.
+pafu_status launch_select_compact(const uint16_t* K, const uint16_t* V, const float* scores, const StreamTable& st, int32_t d_model, int32_t* idx,
+                                  uint16_t* Kc, uint16_t* Vc, float* SLc, cudaStream_t stream, bool* done) {
+    const SelLaunch pl = plan_select(st);
+    const int64_t chunks = d_model / 8, B = st.cu_B[st.n_streams];
+    *done = !pl.any_stream && pl.any_cluster && pl.nc == 1 && B * chunks * 64 <= kSelCopyBytes;
+    if (!*done) return PAFU_OK;
+    static bool attr[kMaxDevices] = {};
+    if (!once_per_device(attr, [] {
+            return cudaFuncSetAttribute(select_copy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmemMax) == cudaSuccess;
+        }))
+        return PAFU_ERR_CUDA;
+    const int threads = pl.per_cta <= kSelShort ? kSelThreads : kSelThreadsMax;
+    int64_t longest = 0;
+    for (int s = 0; s < st.n_streams; ++s) longest = longest > st.cu_B[s + 1] - st.cu_B[s] ? longest : st.cu_B[s + 1] - st.cu_B[s];
+    // as many CTAs a stream as its rows keep busy with one batch each, as far as the GPU holds them at once
+    int64_t copies = (longest * chunks + threads * kSelCopyBatch - 1) / (threads * kSelCopyBatch);
+    const int64_t most = device_sm_count() / st.n_streams > 0 ? device_sm_count() / st.n_streams : 1;
+    if (copies > most) copies = most;
+    const int32_t keys_bytes = (int32_t)(pl.per_cta * 4);
+    return cuda_ok(launch_dependent(select_copy_kernel, dim3((unsigned)(st.n_streams * copies)), dim3(threads),
+                                    (size_t)keys_bytes * 2 + kSelFixedBytes, stream, 1, scores, st, keys_bytes, idx, (int)copies,
+                                    reinterpret_cast<const uint4*>(K), reinterpret_cast<const uint4*>(V), (int)chunks,
+                                    reinterpret_cast<uint4*>(Kc), reinterpret_cast<uint4*>(Vc), SLc));
 }
 
 pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx, cudaStream_t stream, int trigger_late) {

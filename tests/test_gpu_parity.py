@@ -240,6 +240,30 @@ def test_gather_of_narrow_rows(d_head, n_heads, T, B):
         L.compact()
 
 
+@pytest.mark.parametrize("d_head,n_heads,T,B,sink,recent,slc", [
+    (64, 1, (3, 1), (2, 1), 0, 0, True),                        # smaller than a warp; a stream kept whole
+    (64, 2, (1100, 40, 9), (1, 40, 0), 0, 0, False),            # one row, everything, nothing; no salience list
+    (64, 3, (1024 + 30, 1025 + 30), (300, 30), 10, 20, True),   # candidates around a small block's; no top-k row at all
+    (128, 2, (4096 + 7, 2000), (4000, 1999), 3, 4, True),       # the most one CTA selects
+    (128, 2, (4097 + 7, 2000), (4000, 1999), 3, 4, True),       # one more: two launches
+    (128, 3, (30000,), (29000,), 27000, 100, True),             # few candidates, many rows
+], ids=lambda v: str(v) if not isinstance(v, tuple) else "x".join(map(str, v)))
+def test_small_step_selects_and_copies_in_one_launch(d_head, n_heads, T, B, sink, recent, slc):
+    """The same indices, rows and scores as the separate calls."""
+    w = wl.Workload("small", 9, n_heads, d_head, T, B, sink, recent, (64,) * len(T), 32)
+    d = wl.make_layer_device(w, seed=5)
+    A, S = Layer(w, d, want_slc=slc), Layer(w, d, want_slc=slc)
+    for t in (A.idx, S.idx):
+        t.fill_(-1)
+    for t in (A.Kc, A.Vc, S.Kc, S.Vc):
+        t.zero_()
+    A.step(); A.check_status()
+    S.score(); S.select(); S.compact(); S.attn(); S.check_status()
+    assert torch.equal(A.idx, S.idx) and torch.equal(A.Kc, S.Kc) and torch.equal(A.Vc, S.Vc)
+    assert not slc or torch.equal(A.SLc[:A.nB], S.SLc[:S.nB])
+    assert torch.equal(A.O, S.O)
+
+
 # ----------------------------------------------------------------------------- attention
 @pytest.mark.parametrize("w", SMALL, ids=lambda w: "%s-d%d" % (w.name, w.d_head))
 def test_attention_matches_oracle_everywhere(w):
