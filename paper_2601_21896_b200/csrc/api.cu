@@ -690,9 +690,11 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
         for (const uint16_t* x : parts)
             apart = apart || ranges_overlap(x, (size_t)chunk * dm * 2, c->K[to][l] + first * dm, (size_t)(dst0 + chunk - first) * dm * 2) ||
                     ranges_overlap(x, (size_t)chunk * dm * 2, c->V[to][l] + first * dm, (size_t)(dst0 + chunk - first) * dm * 2);
+    // rows in and out, at the copies' rate (6.2 TB/s)
+    const bool share = !apart && head_shares_sms(*head, (double)(chunk + keep) * (double)dm * 8.0 * c->n_layers / 6.2e6);
     auto copy_rows = [&](int64_t n_new, int64_t n_keep, int sel) {
         return launch_cache_rows(Knew, Vnew, n_new, c->K[from], c->V[from], c->SL[from], c->idx, n_keep, dst0, c->K[to], c->V[to],
-                                 c->SL[to], c->n_layers, (int32_t)dm, sel, cs);
+                                 c->SL[to], c->n_layers, (int32_t)dm, sel, share, cs);
     };
     e = apart && keep == 0 ? PAFU_OK : copy_rows(apart ? 0 : chunk, keep, select_ctas);
     if (e != PAFU_OK) return e;
@@ -701,7 +703,7 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
     c->T = dst0;
     if (pruned != nullptr && prune) *pruned = 1;
     // 3. the chunk's salience scores go straight to the tail of SL
-    e = launch_score(*head, parts, 3, chunk, dm, c->SL[to] + dst0, ws, ws_bytes, cs, apart ? 0 : 1);
+    e = launch_score(*head, parts, 3, chunk, dm, c->SL[to] + dst0, ws, ws_bytes, cs, apart ? 0 : share ? 2 : 1);
     if (e != PAFU_OK) return e;
     if (apart) {
         e = copy_rows(chunk, 0, 0);

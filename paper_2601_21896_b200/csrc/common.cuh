@@ -91,15 +91,17 @@ __device__ __forceinline__ int32_t ld_index(const int32_t* p) {
     return v;
 }
 #endif
+// carveout >= 0: that share (per cent) of an SM's L1 and shared memory is to be shared memory while the kernel runs, so that a kernel
+// with dynamic shared memory can join it.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                    cudaStream_t stream, unsigned cluster_x, Args... args) {
+inline cudaError_t launch_dependent_carveout(int carveout, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                             cudaStream_t stream, unsigned cluster_x, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 1;
@@ -110,13 +112,23 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
+    if (carveout >= 0) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs].val.sharedMemCarveout = (unsigned)carveout;
+        ++cfg.numAttrs;
+    }
     cfg.attrs = attr;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, unsigned cluster_x, Args... args) {
+    return launch_dependent_carveout(-1, kernel, grid, block, smem, stream, cluster_x, args...);
 }
 
 // Launchers (each enqueues on `stream` and returns the launch status).
 // beside_predecessor = 1: the kernel runs beside the one launched before it, which must be
 // launch_cache_rows (that kernel lets it start only once everything before it is complete), and ends after it.
+// 2: the same, with shared memory that lets it join that kernel's blocks (launched with share_sms).
 pafu_status launch_score(const pafu_head& head, const uint16_t* const* X, int n_parts, int64_t n_tokens, int64_t ldx,
                          float* scores, void* ws, size_t ws_bytes, cudaStream_t stream, int beside_predecessor = 0);
 // trigger_late = 1: the kernel behind it may start early, but not before everything ahead of the
@@ -144,7 +156,9 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
 pafu_status launch_cache_rows(const uint16_t* const* Knew, const uint16_t* const* Vnew, int64_t n_new,
                               const uint16_t* const* Ks, const uint16_t* const* Vs, const float* SL, const int32_t* idx,
                               int64_t keep, int64_t dst0, uint16_t* const* Kd, uint16_t* const* Vd, float* SLd, int32_t n_layers,
-                              int32_t d_model, int select_ctas, cudaStream_t stream);
+                              int32_t d_model, int select_ctas, bool share_sms, cudaStream_t stream);
+// Whether the salience head should share the SMs with row copies that take about copy_us.
+bool head_shares_sms(const pafu_head& head, double copy_us);
 pafu_status launch_attn(const uint16_t* Q, const uint16_t* Kc, const uint16_t* Vc,
                         const uint16_t* Kq, const uint16_t* Vq, const StreamTable& st,
                         int32_t n_heads, int32_t d_head, float scale, uint16_t* O, float* LSE,

@@ -279,7 +279,10 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
 // A rolling-cache update's copies: the chunk's new rows of every layer, then the kept rows through the
 // index list.  The new rows need nothing that the selection ahead produces, so they are copied while
 // it runs; and the kernel lets the one behind it start at once: that is the salience head of the chunk,
-// tensor-bound work on one CTA an SM, which this kernel leaves registers for (one block of 256 threads an SM).
+// tensor-bound work on one CTA an SM, which this kernel leaves registers for (one block of 256 threads an SM), and where head_shares_sms()
+// says so shared memory too.  (Without that the head starts on an SM only when its block has ended.  Tried for long copies: the head on 13, 19 or
+// 37 SMs of its own, 30 layers of 12 heads 586 -> 610, 601 and 593 us, since the copies miss those SMs and slow the head's weight reads down;
+// all of the L1 but 28 KB given to the head's block 677.)
 //
 // Bound by memory.  What one block an SM reaches is set by its bytes in flight, so a warp's batch is a stretch of
 // kCompactUnroll x 32 sixteen-byte units of a layer's rows laid end to end, whatever the row width, and the
@@ -288,6 +291,7 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
 // 117, 305, 588 and 781; as select, gather, head and append one after the other, many blocks an SM, 140, 164, 324,
 // 612 and 807.  With the indices fetched before the batch's loads instead of behind them 618 at 3072 bytes.)
 constexpr int kCacheSeg = kCompactUnroll * 32;     // units of a warp's batch
+constexpr int kCacheCarveout = 72;                 // per cent of 228 KB: 164 KB of shared memory for the salience head's block
 
 // One batch: unit dst + 32 i comes from src[i]; `between` runs while its loads are under way.
 template <typename Between>
@@ -349,14 +353,14 @@ cache_rows_kernel(const __grid_constant__ LayerPtrs add, const __grid_constant__
 pafu_status launch_cache_rows(const uint16_t* const* Knew, const uint16_t* const* Vnew, int64_t n_new,
                               const uint16_t* const* Ks, const uint16_t* const* Vs, const float* SL, const int32_t* idx,
                               int64_t keep, int64_t dst0, uint16_t* const* Kd, uint16_t* const* Vd, float* SLd, int32_t n_layers,
-                              int32_t d_model, int select_ctas, cudaStream_t stream) {
+                              int32_t d_model, int select_ctas, bool share_sms, cudaStream_t stream) {
     const int64_t cpr = d_model / 8;
     const int64_t segs = ((n_new * cpr + kCacheSeg - 1) / kCacheSeg + (keep * cpr + kCacheSeg - 1) / kCacheSeg) * n_layers;
     int64_t blocks = (segs + kCompactWarpsPerBlock - 1) / kCompactWarpsPerBlock;
     // one block an SM, in fixed shares; the selection's SMs are left out
     const int64_t most = device_sm_count() > select_ctas ? device_sm_count() - select_ctas : 1;
     if (blocks > most) blocks = most;
-    return cuda_ok(launch_dependent(cache_rows_kernel, dim3((unsigned)blocks), dim3(kCompactWarpsPerBlock * 32), 0, stream, 1,
+    return cuda_ok(launch_dependent_carveout(share_sms ? kCacheCarveout : -1, cache_rows_kernel, dim3((unsigned)blocks), dim3(kCompactWarpsPerBlock * 32), 0, stream, 1,
                                     layer_ptrs(Knew, Vnew, Kd, Vd, n_layers), layer_ptrs(Ks, Vs, Kd, Vd, n_layers), (uint32_t)n_layers,
                                     (uint32_t)n_new, dst0, SL, idx, (uint32_t)keep, (uint32_t)cpr, SLd, select_ctas > 0 ? 1 : 0));
 }

@@ -13,4 +13,18 @@ pafu_status launch_score(const pafu_head& head, const uint16_t* const* X, int n_
                             reinterpret_cast<int*>(ws) + kStatusWordTimeout, device_sm_count(), stream, beside_predecessor);
 }
 
+// Row copies leave the head no room: they run with the largest L1, and an SM's split changes only when it is idle, so
+// the head starts where they end.  With 164 KB of shared memory set aside it joins them, but their bytes in flight pass
+// through what is left of the L1, and long copies lose more (a seventh) than the head takes.  So they share while the copies
+// take at most kSharePerSlice us for each of the head's reduction slices, of which it needs 0.45 to 1.1 us: 11 layers of 16 heads,
+// 2300 + 700 tokens 126.8 -> 99.6 us; 10 x 12, 4000 + 2000 147.7 -> 133.9; 8 x 12, 4680 + 4680 210.2 -> 200.5; 30 x 6, 2500 + 1500 135.2 -> 130.0.
+// Beyond: 15 x 12, 4680 + 4680 331 both ways; 30 x 12 586 and 607; 25 x 12, 13 000 + 1000 681 and 727.  Narrow heads are over
+// too soon: 10 layers of 2 heads, 5000 + 4000 56.1 and 58.7.
+bool head_shares_sms(const pafu_head& head, double copy_us) {
+    constexpr double kSharePerSlice = 3.5;
+    constexpr int kShareSlices = 24;
+    const int slices = head.d_in / score_tc::kBK;
+    return slices >= kShareSlices && copy_us <= kSharePerSlice * slices;
+}
+
 }  // namespace pafu

@@ -40,7 +40,9 @@ constexpr int kWBytes = kNMax * kBK * 2;        // 32 KiB
 constexpr int kStageBytes = kXBytes + kWBytes;
 constexpr int kMaxHidden = 1024;
 constexpr int kMaxChunks = kMaxHidden / kNMax;
-constexpr int kSmemBytes = kStages * kStageBytes + 2 * kMaxHidden * 4 + 2 * kBM * 4 + kMaxChunks * kBM * 4 + 256 + 1024;
+constexpr int kStagesShared = 3;     // where it shares the SMs with row copies: leaves them an L1 of 92 KB
+constexpr int smem_bytes(int stages) { return stages * kStageBytes + 2 * kMaxHidden * 4 + 2 * kBM * 4 + kMaxChunks * kBM * 4 + 256 + 1024; }
+static_assert(smem_bytes(kStagesShared) + 1024 + 64 <= 164 * 1024, "the copies' shared-memory share (kCacheCarveout) is 164 KB");
 
 struct Params {
     int64_t n_tokens;
@@ -81,11 +83,12 @@ __device__ __forceinline__ float silu(float x) { return x * rcpf(1.0f + ex2f(-x 
 template <int ACT>
 __device__ __forceinline__ float act_fn(float x) { return ACT == PAFU_ACT_GELU ? gelu_erf(x) : silu(x); }
 
-template <int ACT>
+template <int ACT, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap mX, const __grid_constant__ CUtensorMap mX1,
                 const __grid_constant__ CUtensorMap mX2, const __grid_constant__ CUtensorMap mW,
                 const __grid_constant__ CUtensorMap mWt, const __grid_constant__ Params p) {
+    constexpr int kStages = STAGES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t sStage = smem_u32(smem);
@@ -328,7 +331,7 @@ inline pafu_status launch(const pafu_head& head, const uint16_t* const* X, int n
     Params p;
     p.n_tokens = n_tokens; p.d_in = head.d_in; p.d_hidden = head.d_hidden; p.d_out = head.d_out;
     p.act = head.act; p.final = head.final; p.w2 = head.w2; p.b1 = head.b1; p.b2 = head.b2;
-    p.scores = scores; p.status = status; p.beside = beside;
+    p.scores = scores; p.status = status; p.beside = beside != 0;
     p.k_per_part = d_part / kBK;
     const int64_t n_tiles = (n_tokens + kBM - 1) / kBM;
     const int n_chunks = (head.d_hidden + kNMax - 1) / kNMax;
@@ -351,13 +354,20 @@ inline pafu_status launch(const pafu_head& head, const uint16_t* const* X, int n
     const unsigned cluster = p.split ? (unsigned)n_chunks : (p.tail_tiles > 0 ? 2u : 1u);
     static bool attr_set[kMaxDevices] = {};
     if (!once_per_device(attr_set, [] {
-            return cudaFuncSetAttribute(score_tc_kernel<PAFU_ACT_GELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) == cudaSuccess &&
-                   cudaFuncSetAttribute(score_tc_kernel<PAFU_ACT_SILU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) == cudaSuccess;
+            auto opt_in = [](auto* kernel, int stages) {
+                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(stages)) == cudaSuccess;
+            };
+            return opt_in(score_tc_kernel<PAFU_ACT_GELU, kStages>, kStages) && opt_in(score_tc_kernel<PAFU_ACT_SILU, kStages>, kStages) &&
+                   opt_in(score_tc_kernel<PAFU_ACT_GELU, kStagesShared>, kStagesShared) && opt_in(score_tc_kernel<PAFU_ACT_SILU, kStagesShared>, kStagesShared);
         }))
         return PAFU_ERR_CUDA;
-    return cuda_ok(head.act == PAFU_ACT_GELU
-                       ? launch_dependent(score_tc_kernel<PAFU_ACT_GELU>, dim3(grid), dim3(kThreads), kSmemBytes, stream, cluster, mX[0], mX[1], mX[2], mW, mWt, p)
-                       : launch_dependent(score_tc_kernel<PAFU_ACT_SILU>, dim3(grid), dim3(kThreads), kSmemBytes, stream, cluster, mX[0], mX[1], mX[2], mW, mWt, p));
+    auto go = [&](auto* kernel, int stages) {
+        return cuda_ok(launch_dependent(kernel, dim3(grid), dim3(kThreads), smem_bytes(stages), stream, cluster, mX[0], mX[1], mX[2], mW, mWt, p));
+    };
+    const bool shared = beside == 2;
+    if (head.act == PAFU_ACT_GELU)
+        return shared ? go(score_tc_kernel<PAFU_ACT_GELU, kStagesShared>, kStagesShared) : go(score_tc_kernel<PAFU_ACT_GELU, kStages>, kStages);
+    return shared ? go(score_tc_kernel<PAFU_ACT_SILU, kStagesShared>, kStagesShared) : go(score_tc_kernel<PAFU_ACT_SILU, kStages>, kStages);
 }
 
 }  // namespace score_tc

@@ -697,6 +697,41 @@ def test_cache_updates_without_a_synchronisation_between_them(cap, chunk, N):
         assert torch.equal(cache.K[l], K[l]) and torch.equal(cache.V[l], V[l])
 
 
+@pytest.mark.parametrize("layers,N,cap,chunk,hidden", [
+    (1, 8, 700, 130, 1024),       # short copies: the head shares their SMs, (tile, chunk) units in clusters of four
+    (3, 4, 2000, 1900, 640),      # the same with a half-full last accumulator
+    (2, 4, 1000, 700, 64),        # one accumulator: tiles shared by two CTAs
+    (40, 4, 3000, 300, 256),      # copies too long for that
+    (4, 2, 1000, 500, 1024),      # too narrow a head for that
+])
+def test_cache_update_head_beside_the_copies(layers, N, cap, chunk, hidden):
+    """The salience head beside the row copies, on their SMs or not, gives the bits that it gives alone; the rows are copies."""
+    D, keep = 128, cap - chunk
+    g = torch.Generator(device="cuda").manual_seed(layers + hidden)
+    rn = lambda *shape: torch.randn(*shape, generator=g, device="cuda")
+    w = [(rn(*s) / 8).to(torch.bfloat16) for s in ((hidden, 3 * N * D), (hidden,), (12, hidden), (12,))]
+    head = pafu.Head(*w, wl.ACT_SILU, wl.FINAL_NONE)
+    ws = torch.zeros(pafu.pafu_workspace_bytes(pafu.Shape(N, D, [0, cap], [0, chunk]), None, head), dtype=torch.uint8, device="cuda")
+    cache = pafu.Cache(layers, N, D, cap, 50)
+    for l in range(layers):
+        cache.Kb[0][l].copy_(rn(cap, N, D)); cache.Vb[0][l].copy_(rn(cap, N, D))
+    cache.SLb[0].copy_(rn(cap))
+    cache.c.T = cap
+    new = [rn(chunk, N, D).to(torch.bfloat16) for _ in range(3)]
+    want = torch.empty(chunk, device="cuda")
+    pafu.pafu_score_qkv(head, *new, want, ws, ld=N * D)
+    for _ in range(3):                                     # back to back from the same full cache
+        cache.c.T, cache.c.cur = cap, 0
+        pafu.pafu_cache_update(cache, head, *new, [new[1]] * layers, [new[2]] * layers, ws)
+    assert pafu.pafu_workspace_status(ws) == 0
+    assert torch.equal(cache.SL[keep:], want)
+    i = cache.idx[:keep].long()
+    assert torch.equal(cache.SL[:keep], cache.SLb[0][:cap][i])
+    for l in range(layers):
+        assert torch.equal(cache.K[l], torch.cat([cache.Kb[0][l][i], new[1]]))
+        assert torch.equal(cache.V[l], torch.cat([cache.Vb[0][l][i], new[2]]))
+
+
 @pytest.mark.parametrize("T,where", [(300, "append"), (128, "append"), (300, "kept"), (256, "append")])
 def test_cache_update_head_inputs_in_the_idle_buffers(T, where):
     """The head's input rows may lie in buffers that the update writes: in rows that the append overwrites (they are
