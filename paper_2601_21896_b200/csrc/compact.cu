@@ -4,7 +4,7 @@
 // in 16-byte pieces, all loads of a batch issued before the first store so that each warp
 // keeps up to 12 x 512 B in flight.  Rows are contiguous, so every access is fully coalesced;
 // the only indirection is one int32 index per row.
-#include "common.cuh"
+#include "select_plan.cuh"
 
 namespace pafu {
 
@@ -91,8 +91,6 @@ __device__ __forceinline__ void copy_kv_rows(const uint4* __restrict__ K, const 
 // of one cluster the grid leaves its SMs out and every block takes a fixed share (early_static;
 // selection and gather of the 28 080-token cache, selected by eight CTAs, 39.6 us with claiming, 31.4 with shares; of the
 // 93 600-token one 33.5 and 29.3; four streams, 32 CTAs: no difference).
-constexpr int kStaticSelect = 8;
-
 // A claim in two halves: lane 0 issues the add; its result is fetched (and shared with the warp)
 // only when the rows are needed, so the trip to L2 overlaps the copying in between.
 __device__ __forceinline__ int claim_issue(int* counter, int group, int lane) {
@@ -378,7 +376,7 @@ pafu_status launch_compact(const uint16_t* K, const uint16_t* V, const float* SL
     // A few resident waves, larger inputs loop.  With the early part the grid is what the device
     // holds at once (three blocks fit on an SM): a block must not queue behind blocks that are
     // waiting for the selection.  Fixed shares: the selection's SMs are left out of the count.
-        const int early_static = work != nullptr && select_ctas <= kStaticSelect;
+    const int early_static = work != nullptr && select_ctas <= kStaticSelect;
     int sms = device_sm_count() - (early_static ? select_ctas : 0);
     if (sms < 1) sms = 1;
     const int64_t max_blocks = work != nullptr ? (int64_t)sms * 3 : 148 * 8 * 4;

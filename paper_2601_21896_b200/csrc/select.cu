@@ -27,21 +27,12 @@
 // whatever the scores say while the selection runs, and waits for the indices after that.
 #include <cooperative_groups.h>
 
-#include "common.cuh"
+#include "select_plan.cuh"
 
 namespace pafu {
 
 namespace cg = cooperative_groups;
 
-constexpr int kSelThreads = 256;            // block of a CTA with a short share; kSelThreadsMax with a long one
-constexpr int kSelThreadsMax = 1024;
-constexpr int kSelWarps = kSelThreads / 32;
-constexpr int kSelWarpsMax = kSelThreadsMax / 32;
-constexpr int kSelCluster = 8;              // at most this many CTAs cooperate on one stream
-constexpr int kSelCapCta = 45056;           // candidates one CTA holds (176 KiB of keys)
-constexpr int kSelCapCluster = kSelCluster * kSelCapCta;
-constexpr int kSelBins = 1024;
-constexpr int kSelList = 1024;              // most candidates in the bin of the k-th largest one that are ranked directly
 constexpr int kSelBatch = 8;                // independent loads a thread keeps in flight
 constexpr int kSelStreamThreads = 1024;     // the streaming kernel's block
 static_assert(kSelBins == 4 * kSelThreads, "four bins a thread");
@@ -80,12 +71,6 @@ __device__ __forceinline__ int sel_exclusive_scan(int v, int* warp_sums, int* to
     *total = warp_sums[32];
     return warp_sums[warp] + inc - v;
 }
-
-namespace {
-constexpr size_t kSelSmemMax = 227 * 1024 - 1024;            // dynamic shared memory a CTA may ask for (static part left out)
-constexpr size_t kSelFixedBytes = (size_t)(2 * kSelBins + (kSelCluster + 1) * kSelList) * 4;
-static_assert((size_t)kSelCapCta * 4 + kSelFixedBytes <= kSelSmemMax, "a CTA's share does not fit");
-}  // namespace
 
 // The score a key stands for (a NaN for key 0).
 __device__ __forceinline__ float key_score(uint32_t key) { return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key); }
@@ -390,19 +375,26 @@ select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ 
     select_stream<false>(scores, st, blockIdx.x / cg::this_cluster().num_blocks(), 0, 1, keys_bytes, idx, trigger_late, sel_smem, sh, nullptr);
 }
 
-// Selection and row gather of a small layer step in one launch: `copies` CTAs per stream all make the stream's whole selection (a
+// Selection and row gather of a small layer step in one launch: a stream's CTAs all make its whole selection (a
 // few microseconds, whoever does it) and then copy a share of its rows each, without a word between them.  What it
 // saves is the second kernel's start: a step of 2 heads x 64 over 512 tokens 19.0 -> 17.2 us, 4 x 64 over 600 25.5 -> 23.8, 5 x 128 over 1800 +
 // 2500 37.5 -> 37.0, 12 x 128 over 3000 (18 MB in and out) 54.1 -> 53.1.  Larger steps keep two launches: their always-kept rows are
 // copied while the selection runs.
-constexpr int kSelCopyBatch = 4;            // 16-byte pieces of K and of V a thread has in flight
 __global__ void __launch_bounds__(kSelThreadsMax, 1)
-select_copy_kernel(const float* __restrict__ scores, const __grid_constant__ StreamTable st, int32_t keys_bytes,
-                   int32_t* __restrict__ idx, int copies, const uint4* __restrict__ K, const uint4* __restrict__ V,
+select_copy_kernel(const __grid_constant__ CopyShares shares, const float* __restrict__ scores, int32_t keys_bytes,
+                   int32_t* __restrict__ idx, const __grid_constant__ StreamTable st, const uint4* __restrict__ K, const uint4* __restrict__ V,
                    int chunks_per_row, uint4* __restrict__ Kc, uint4* __restrict__ Vc, float* __restrict__ SLc) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     __shared__ SelShared sh;
-    const int s = blockIdx.x / copies, copy = blockIdx.x % copies, threads = (int)blockDim.x;
+    const int b = (int)blockIdx.x, threads = (int)blockDim.x;
+    int s = 0, copy = b, copies = (int)gridDim.x;
+    if (st.n_streams > 1) {                                  // the last stream that begins at or before b
+#pragma unroll
+        for (int d = PAFU_MAX_STREAMS / 2; d > 0; d /= 2)
+            if (s + d < st.n_streams && shares.first[s + d] <= b) s += d;
+        copy -= shares.first[s];
+        copies = shares.first[s + 1] - shares.first[s];
+    }
     int* top = reinterpret_cast<int*>(sel_smem + keys_bytes + kSelFixedBytes);
     select_stream<true>(scores, st, s, copy, copies, keys_bytes, idx, 0, sel_smem, sh, top);
     __syncthreads();
@@ -544,64 +536,26 @@ select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* 
     }
 }
 
-namespace {
-// Candidates a CTA: most before the cluster doubles, and most for a block of 256 threads (2000 candidates: 6.9 us in 256 threads, 5.8 in 1024; 444:
-// 4.3 and 8.5).
-constexpr int64_t kSelShare = 4096, kSelShort = 1024;
-constexpr int64_t kSelCopyBytes = 64 << 20;
-struct SelLaunch {
-    bool any_cluster = false, any_stream = false;
-    int nc = 1;
-    int64_t per_cta = 0;
-};
-SelLaunch plan_select(const StreamTable& st) {
-    SelLaunch pl;
-    int64_t m_max = 0;
-    for (int s = 0; s < st.n_streams; ++s) {
-        const int64_t T = st.cu_T[s + 1] - st.cu_T[s], B = st.cu_B[s + 1] - st.cu_B[s];
-        if (B == 0) continue;
-        const int64_t M = B >= T ? 0 : T - st.n_sink[s] - st.n_recent[s];
-        if (M > kSelCapCluster) { pl.any_stream = true; continue; }
-        pl.any_cluster = true;
-        if (M > m_max) m_max = M;
-    }
-    // CTAs per stream.  A histogram of 1024 candidates costs a CTA some 400 clocks (13 an add and warp, whether or not its
-    // lanes collide), the barriers across CTAs and the trips through distributed shared memory two to three thousand: 7800 candidates
-    // 9.4 us on one CTA, 7.9 on two, 7.4 on four; 16 000 10.2 on two, 8.4 on four.
-    while (pl.nc < kSelCluster && m_max > (int64_t)pl.nc * kSelShare) pl.nc *= 2;
-    pl.per_cta = ((m_max + pl.nc - 1) / pl.nc + 31) / 32 * 32;
-    return pl;
-}
-}  // namespace
-
 int select_cta_count(const StreamTable& st) {
     const SelLaunch pl = plan_select(st);
     return (pl.any_cluster ? st.n_streams * pl.nc : 0) + (pl.any_stream ? st.n_streams : 0);
 }
 
-// A step is small when one CTA selects each stream and the rows, K and V in and out, are kSelCopyBytes at most.
 pafu_status launch_select_compact(const uint16_t* K, const uint16_t* V, const float* scores, const StreamTable& st, int32_t d_model, int32_t* idx,
                                   uint16_t* Kc, uint16_t* Vc, float* SLc, cudaStream_t stream, bool* done) {
-    const SelLaunch pl = plan_select(st);
-    const int64_t chunks = d_model / 8, B = st.cu_B[st.n_streams];
-    *done = !pl.any_stream && pl.any_cluster && pl.nc == 1 && B * chunks * 64 <= kSelCopyBytes;
+    const int chunks = d_model / 8;
+    const SelCopyLaunch cp = plan_select_copy(st, chunks, device_sm_count());
+    *done = cp.small;
     if (!*done) return PAFU_OK;
     static bool attr[kMaxDevices] = {};
     if (!once_per_device(attr, [] {
             return cudaFuncSetAttribute(select_copy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmemMax) == cudaSuccess;
         }))
         return PAFU_ERR_CUDA;
-    const int threads = pl.per_cta <= kSelShort ? kSelThreads : kSelThreadsMax;
-    int64_t longest = 0;
-    for (int s = 0; s < st.n_streams; ++s) longest = longest > st.cu_B[s + 1] - st.cu_B[s] ? longest : st.cu_B[s + 1] - st.cu_B[s];
-    // as many CTAs a stream as its rows keep busy with one batch each, as far as the GPU holds them at once
-    int64_t copies = (longest * chunks + threads * kSelCopyBatch - 1) / (threads * kSelCopyBatch);
-    const int64_t most = device_sm_count() / st.n_streams > 0 ? device_sm_count() / st.n_streams : 1;
-    if (copies > most) copies = most;
-    const int32_t keys_bytes = (int32_t)(pl.per_cta * 4);
-    return cuda_ok(launch_dependent(select_copy_kernel, dim3((unsigned)(st.n_streams * copies)), dim3(threads),
-                                    (size_t)keys_bytes * 2 + kSelFixedBytes, stream, 1, scores, st, keys_bytes, idx, (int)copies,
-                                    reinterpret_cast<const uint4*>(K), reinterpret_cast<const uint4*>(V), (int)chunks,
+    const int32_t keys_bytes = cp.per_cta * 4;
+    return cuda_ok(launch_dependent(select_copy_kernel, dim3((unsigned)cp.shares.first[st.n_streams]), dim3(cp.threads),
+                                    (size_t)keys_bytes * 2 + kSelFixedBytes, stream, 1, cp.shares, scores, keys_bytes, idx, st,
+                                    reinterpret_cast<const uint4*>(K), reinterpret_cast<const uint4*>(V), chunks,
                                     reinterpret_cast<uint4*>(Kc), reinterpret_cast<uint4*>(Vc), SLc));
 }
 
@@ -617,7 +571,7 @@ pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* i
         const int32_t keys_bytes = (int32_t)(pl.per_cta * 4);
         const size_t smem = (size_t)keys_bytes + kSelFixedBytes;
         if (launch_dependent(select_cluster_kernel, dim3((unsigned)(st.n_streams * pl.nc)),
-                             dim3(pl.per_cta <= kSelShort ? kSelThreads : kSelThreadsMax), smem, stream,
+                             dim3(pl.threads()), smem, stream,
                              (unsigned)pl.nc, scores, st, keys_bytes, idx, trigger_late) != cudaSuccess)
             return PAFU_ERR_CUDA;
     }

@@ -246,7 +246,9 @@ def test_gather_of_narrow_rows(d_head, n_heads, T, B):
     (64, 3, (1024 + 30, 1025 + 30), (300, 30), 10, 20, True),   # candidates around a small block's; no top-k row at all
     (128, 2, (4096 + 7, 2000), (4000, 1999), 3, 4, True),       # the most one CTA selects
     (128, 2, (4097 + 7, 2000), (4000, 1999), 3, 4, True),       # one more: two launches
-    (128, 3, (30000,), (29000,), 27000, 100, True),             # few candidates, many rows
+    (128, 3, (30000,), (29000,), 27000, 100, True),             # 89 MB: two launches
+    (128, 3, (13000,), (12600,), 12000, 100, True),             # few candidates, many rows: 38.7 MB in and out in one launch
+    (64, 2, (36000,) + (60, 9) * 15 + (100,), (36000,) + (30, 0) * 15 + (99,), 3, 4, True),   # one stream kept whole beside 31 short ones
 ], ids=lambda v: str(v) if not isinstance(v, tuple) else "x".join(map(str, v)))
 def test_small_step_selects_and_copies_in_one_launch(d_head, n_heads, T, B, sink, recent, slc):
     """The same indices, rows and scores as the separate calls."""
