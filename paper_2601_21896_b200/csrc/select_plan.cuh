@@ -22,6 +22,10 @@ static_assert((size_t)kSelCapCta * 4 + kSelFixedBytes <= kSelSmemMax, "a CTA's s
 // 4.3 and 8.5).
 constexpr int64_t kSelShare = 4096, kSelShort = 1024;
 
+// Clusters of eight, one block an SM, that the GPU holds at once: 15 streams of 21 840 candidates 10.4 us, 16 18.8 (in clusters of four 11.3); 32
+// streams 28.1, in clusters of four 11.6; 31 of 500 candidates beside one of 20 000 23.1 and 10.7; 16 of 45 000 24.1 and 16.4.
+constexpr int kSelRoom8 = 15 * 8;
+
 struct SelLaunch {
     bool any_cluster = false, any_stream = false;
     int nc = 1;
@@ -42,7 +46,9 @@ inline SelLaunch plan_select(const StreamTable& st) {
     // CTAs per stream.  A histogram of 1024 candidates costs a CTA some 400 clocks (13 an add and warp, whether or not its
     // lanes collide), the barriers across CTAs and the trips through distributed shared memory two to three thousand: 7800 candidates
     // 9.4 us on one CTA, 7.9 on two, 7.4 on four; 16 000 10.2 on two, 8.4 on four.
-    while (pl.nc < kSelCluster && m_max > (int64_t)pl.nc * kSelShare) pl.nc *= 2;
+    // They are doubled while all streams' clusters find room on the GPU at once, or one stream's candidates would not fit.
+    auto fits = [&](int nc) { return st.n_streams * nc <= (nc < 8 ? 128 : kSelRoom8); };
+    while (pl.nc < kSelCluster && m_max > pl.nc * (fits(2 * pl.nc) ? kSelShare : (int64_t)kSelCapCta)) pl.nc *= 2;
     pl.per_cta = ((m_max + pl.nc - 1) / pl.nc + 31) / 32 * 32;
     return pl;
 }

@@ -27,3 +27,9 @@ extern "C" void plan_copy(int n, const int64_t* T, const int64_t* B, int64_t sin
     out[0] = cp.small; out[1] = cp.threads; out[2] = cp.per_cta;
     for (int s = 0; cp.small && s <= n; ++s) out[3 + s] = cp.shares.first[s];
 }
+
+// out: [CTAs a stream, candidates a CTA, streaming kernel too]
+extern "C" void plan_selection(int n, const int64_t* T, const int64_t* B, int64_t sink, int64_t recent, int64_t* out) {
+    const SelLaunch pl = plan_select(table(n, T, B, sink, recent));
+    out[0] = pl.nc; out[1] = pl.per_cta; out[2] = pl.any_stream;
+}

@@ -78,3 +78,21 @@ def test_shares_of_many_small_steps(lib):
 ])
 def test_limits_of_small_steps(lib, T, B, sink, chunks, small):
     assert plan_copy(lib, T, B, sink, 0, chunks)[0] == small
+
+
+def plan_selection(lib, M):
+    out = np.zeros(3, dtype=np.int64)
+    T, i64 = [m + 5 for m in M], ctypes.c_int64
+    lib.plan_selection(len(M), arr(T), arr([m // 2 + 5 for m in M]), i64(2), i64(3), out.ctypes.data_as(ctypes.c_void_p))
+    return out.tolist()
+
+
+@pytest.mark.parametrize("M,ctas", [
+    ([4096], 1), ([4097], 2), ([8193], 4), ([16385], 8), ([360448], 8),
+    ([21840] * 15, 8), ([21840] * 16, 4), ([21840] * 32, 4), ([500] * 31 + [20000], 4),       # one wave
+    ([180224] * 32, 4), ([500] * 31 + [180225], 8),                                            # the most four CTAs hold
+])
+def test_selecting_clusters_fit_on_the_gpu_at_once(lib, M, ctas):
+    nc, per_cta, stream = plan_selection(lib, M)
+    assert nc == ctas and not stream and per_cta * nc >= max(M) and per_cta <= 45056
+    assert nc * len(M) <= (120 if nc == 8 else 128) or max(M) > nc // 2 * 45056
