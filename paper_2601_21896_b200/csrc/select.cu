@@ -6,21 +6,26 @@
 // distributed shared memory, and instructions that every warp executes (a scan by 32 warps costs four times the issue slots of
 // one by eight, so short shares run in blocks of 256 threads and eight warps do what is done once).  One CTA, or a
 // cluster of two, four or eight (the host picks by the stream length), works on one stream; CTA r holds the r-th part of the
-// candidates in its shared memory.  Back to back, 444 / 4000 / 7800 / 21 840 / 87 360 candidates: 4.3 / 7.6 / 8.5 / 9.4 / 16.7 us; with
-// three passes over digits of the key (11 + 11 + 10 bits, a tenth of the candidates left after the first), blocks of 1024 and one CTA
-// up to 24 576 candidates 8.4 / 10.1 / 11.8 / 19.6 / 25.4.
+// candidates in its shared memory.  Back to back, 444 / 4000 / 7800 / 21 840 / 87 360 / 200 000 / 360 000 candidates:
+// 4.3 / 8.2 / 8.8 / 9.8 / 17.1 / 24.9 / 37.1 us; with three passes over digits of the key (11 + 11 + 10 bits, a tenth of the candidates left after
+// the first), blocks of 1024 and one CTA up to 24 576 candidates 8.4 / 10.4 / 12.0 / 18.5 / 25.0 / 31.5 / 40.0.
 //   1. fp32 scores map to order-preserving 32-bit keys (-0 folded onto +0, NaN lowest).
 //   2. One histogram of 1024 equal steps between the smallest and the largest of 256 sampled scores (the same sample in
 //      every CTA, so nothing is exchanged for it; values outside fall into the end bins).  One cluster barrier later
 //      every CTA adds up all histograms through distributed shared memory and finds by itself the bin that holds the k-th
 //      largest candidate.  Every CTA sends its few candidates of that bin to all others; one more barrier, and each ranks
 //      them against one another by itself.
+//      Long shares (more than kSelLong candidates a CTA): ranking m candidates costs m^2, and a bin of the whole range holds hundreds; the
+//      adds into the histogram alone take 10 us at 45 000.  So the sample is ranked, and the steps lie between its places three standard
+//      deviations around the k-th largest candidate's: most candidates then fall into the end bins, which are counted in
+//      registers, the bins hold dozens, and an outlier in the sample does no harm (360 000 candidates with steps between the extremes
+//      61 us, with outliers 63; so 37 and 38).
 //   3. A bin that holds too many (ties, a far outlier in the sample) is narrowed down: the smallest and the largest of
 //      its candidates are exchanged, and if they differ another histogram divides what lies between them, first in equal
 //      steps of the score, then of the key (which ends: 2^32 keys, a factor of 1024 each time).
-//   4. Ordered emission: every warp owns a contiguous stretch of the CTA's candidates, counts what it keeps and, once the counts
-//      of the warps and CTAs before it are known, writes it in order: the result is ascending and ties resolve to
-//      the lowest indices.
+//   4. Ordered emission: every warp owns a contiguous stretch of the CTA's candidates.  What it keeps of them is known from the sweep that
+//      found the bin's candidates and from who found which; with the counts of the warps and CTAs before it, it writes them in order:
+//      the result is ascending and ties resolve to the lowest indices.
 // Streams with more candidates than eight CTAs hold (360 448) use one CTA that re-reads L2 in every pass.
 // A kernel launched behind these as a programmatic dependent may start at once (the trigger at
 // their top): inside a layer step that is the row gather, which copies the rows that are kept
@@ -82,7 +87,8 @@ struct SelShared {
     uint32_t thr;
     int need_eq, eq_total;
     int list_n;
-    int warp_gt[kSelWarpsMax], warp_eq[kSelWarpsMax];
+    int warp_gt[kSelWarpsMax], warp_eq[kSelWarpsMax];   // candidates of each warp above the bin (the threshold) and in it (equal to it)
+    uint8_t owner[kSelList];         // whose the CTA's candidates in the bin are
     // from every CTA: its candidates in the bin and above it, and the smallest and largest of those in it
     int in_bin[kSelCluster], above[kSelCluster];
     uint32_t cta_lo[kSelCluster], cta_hi[kSelCluster];
@@ -169,6 +175,7 @@ __device__ __forceinline__ void select_stream(const float* __restrict__ scores, 
     const int per_cta = ((M + nc - 1) / nc + 31) / 32 * 32;
     const int j_lo = rank * per_cta;
     const int n = max(0, min(M - j_lo, per_cta));
+    const bool near_k = !ALONE && per_cta > kSelLong;
     if (k > 0) {
         const int step = M / kSelThreads;                    // 0: every candidate is in the sample
         const int js = step > 0 ? tid * step : tid;
@@ -186,6 +193,7 @@ __device__ __forceinline__ void select_stream(const float* __restrict__ scores, 
         const bool finite = ks >= 0x00800000u && ks <= 0xff7fffffu;
         const uint32_t lo_w = __reduce_min_sync(0xffffffffu, finite ? ks : 0xffffffffu), hi_w = __reduce_max_sync(0xffffffffu, finite ? ks : 0u);
         if (lane == 0) { sh.lo[warp] = lo_w; sh.hi[warp] = hi_w; }
+        if (near_k && tid < kSelThreads && tid % 2 == 0) hist[kSelBins + tid / 2] = (int)ks;
     }
     // always-kept tokens (spread over the cluster, or the CTAs side by side): position p < ns is token p, position ns + k + i is token T - nr + i
     for (int p = (ALONE ? copy : rank) * threads + tid; p < ns + nr; p += (ALONE ? copies : nc) * threads) {
@@ -196,14 +204,42 @@ __device__ __forceinline__ void select_stream(const float* __restrict__ scores, 
     uint32_t klo = 0u, khi = 0xffffffffu;                    // the keys still in question
     float lo = 0.f, scale = 0.f;                             // how they are divided: equal steps of the score,
     int shift = -1;                                          // or of the key (>= 0)
-    auto steps = [&](uint32_t a, uint32_t b) {               // between the finite scores of keys a < b
-        lo = key_score(a);
-        scale = (float)kSelBins / (key_score(b) - lo);
+    auto steps = [&](float a, float b) {                     // between finite scores a < b
+        lo = a;
+        scale = (float)kSelBins / (b - a);
         if (!(scale <= 3.0e38f)) scale = 0.f;                // a range of a few denormals
     };
     {
         const uint32_t a = __reduce_min_sync(0xffffffffu, sh.lo[lane & (kSelWarps - 1)]), b = __reduce_max_sync(0xffffffffu, sh.hi[lane & (kSelWarps - 1)]);
-        if (a < b) steps(a, b);                              // at least two finite values
+        if (a < b) steps(key_score(a), key_score(b));        // at least two finite values
+    }
+    if (near_k) {
+        // Between the places of every other sample three standard deviations around the k-th largest candidate's, and three times as far
+        // out where the sample ends (eight threads rank a sample).
+        constexpr int kRanked = kSelThreads / 2;
+        static_assert(kRanked * 8 == kSelThreadsMax, "eight threads a sample");
+        const float p = (float)k / (float)M * kRanked, d = 3.f * sqrtf(p * (1.f - p / kRanked)) + 1.f;
+        const int r_hi = max(0, (int)(p - d)), r_lo = min(kRanked - 1, (int)(p + d) + 1);
+        const uint32_t* ranked_keys = reinterpret_cast<const uint32_t*>(hist + kSelBins);
+        const uint32_t key = ranked_keys[tid >> 3];
+        int gt = 0, ge = 0;
+#pragma unroll
+        for (int e = 0; e < kRanked / 8; e += 4) {
+            const uint4 o = *reinterpret_cast<const uint4*>(ranked_keys + (tid & 7) * (kRanked / 8) + e);
+            gt += (o.x > key) + (o.y > key) + (o.z > key) + (o.w > key);
+            ge += (o.x >= key) + (o.y >= key) + (o.z >= key) + (o.w >= key);
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) { gt += __shfl_xor_sync(0xffffffffu, gt, o); ge += __shfl_xor_sync(0xffffffffu, ge, o); }
+        if (gt <= r_hi && r_hi < ge) sh.hi[kSelWarps] = key;                 // equal keys write the same
+        if (gt <= r_lo && r_lo < ge) sh.lo[kSelWarps] = key;
+        __syncthreads();
+        const uint32_t l = sh.lo[kSelWarps], h = sh.hi[kSelWarps];
+        if (l >= 0x00800000u && l < h && h <= 0xff7fffffu) {
+            const float a = key_score(l), b = key_score(h), far = 3.f * (b - a);
+            const float x = p < d ? b + far : b, y = p + d > kRanked ? a - far : a;
+            if (x - y <= 3.0e38f) steps(y, x); else steps(a, b);
+        }
     }
     // Monotone in the key: rounding is, and so are the clamps; infinities end up in the end bins, NaN (lowest) in bin 0, and with
     // scale = 0 everything in bin 0.
@@ -229,10 +265,24 @@ __device__ __forceinline__ void select_stream(const float* __restrict__ scores, 
             if (tid < kSelThreads) *reinterpret_cast<int4*>(h + 4 * tid) = make_int4(0, 0, 0, 0);
             __syncthreads();
         }
+        if (near_k && level == 0) {                          // most candidates fall into the end bins: they are counted in registers
+            int low = 0, high = 0;
 #pragma unroll 4
-        for (int j = tid; j < n; j += threads) {
-            const int b = bin_of(keys[j]);
-            if ((unsigned)b < (unsigned)kSelBins) atomicAdd(h + b, 1);
+            for (int j = tid; j < n; j += threads) {
+                const int b = bin_of(keys[j]);
+                low += b == 0;
+                high += b == kSelBins - 1;
+                if (b > 0 && b < kSelBins - 1) atomicAdd(h + b, 1);
+            }
+            low = __reduce_add_sync(0xffffffffu, low);
+            high = __reduce_add_sync(0xffffffffu, high);
+            if (lane == 0) { atomicAdd(h, low); atomicAdd(h + kSelBins - 1, high); }
+        } else {
+#pragma unroll 4
+            for (int j = tid; j < n; j += threads) {
+                const int b = bin_of(keys[j]);
+                if ((unsigned)b < (unsigned)kSelBins) atomicAdd(h + b, 1);
+            }
         }
         find_bin(cluster, nc, sh, h, need_eq);
         need_eq = sh.k_rem; eq_total = sh.bin_count;
@@ -271,7 +321,7 @@ __device__ __forceinline__ void select_stream(const float* __restrict__ scores, 
         }
         klo = mn; khi = mx;
         const bool finite = klo >= 0x00800000u && khi <= 0xff7fffffu;
-        if (level == 0 && finite) steps(klo, khi);
+        if (level == 0 && finite) steps(key_score(klo), key_score(khi));
         else shift = max(0, 22 - __clz(khi - klo));
     }
     if (ranked) {
@@ -285,10 +335,11 @@ __device__ __forceinline__ void select_stream(const float* __restrict__ scores, 
             above += __popc(__ballot_sync(0xffffffffu, b > bin));
             if (b == bin) {
                 const int at = atomicAdd(&sh.list_n, 1);
+                sh.owner[at] = (uint8_t)warp;
                 for (int r = 0; r < nc; ++r) cluster.map_shared_rank(list, r)[rank * kSelList + at] = key;
             }
         }
-        if (lane == 0) sh.warp_gt[warp] = above;
+        if (lane == 0) { sh.warp_gt[warp] = above; sh.warp_eq[warp] = 0; }
         __syncthreads();
         if (warp == 0) {
             const int a = __reduce_add_sync(0xffffffffu, lane < warps ? sh.warp_gt[lane] : 0);
@@ -331,20 +382,16 @@ __device__ __forceinline__ void select_stream(const float* __restrict__ scores, 
             gt_before += __popc(__ballot_sync(0xffffffffu, in && key > thr));
             eq_before += __popc(__ballot_sync(0xffffffffu, in && key == thr));
         }
+        // and what the warps of this one do
+        for (int i = tid; i < sh.list_n; i += threads) {
+            const uint32_t key = list[rank * kSelList + i];
+            if (key >= thr) atomicAdd(key > thr ? &sh.warp_gt[sh.owner[i]] : &sh.warp_eq[sh.owner[i]], 1);
+        }
+        __syncthreads();
     }
 
     // ---- ordered emission
     const bool ties = need_eq != eq_total;                   // cluster-uniform: some equal candidates stay out
-    int gt = 0, eq = 0;
-#pragma unroll 4
-    for (int j0 = w0; j0 < w1; j0 += 32) {
-        const uint32_t key = j0 + lane < w1 ? keys[j0 + lane] : 0u;
-        gt += __popc(__ballot_sync(0xffffffffu, j0 + lane < w1 && key > thr));
-        eq += __popc(__ballot_sync(0xffffffffu, j0 + lane < w1 && key == thr));
-    }
-    __syncthreads();                                         // the last reads of warp_gt are complete
-    if (lane == 0) { sh.warp_gt[warp] = gt; sh.warp_eq[warp] = eq; }
-    __syncthreads();
     gt_before += __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp_gt[lane] : 0);
     eq_before += __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp_eq[lane] : 0);
     int pos = ns + gt_before + (ties ? min(eq_before, need_eq) : eq_before);

@@ -14,10 +14,14 @@ constexpr int kSelCapCta = 45056;           // candidates one CTA holds (176 KiB
 constexpr int kSelCapCluster = kSelCluster * kSelCapCta;
 constexpr int kSelBins = 1024;
 constexpr int kSelList = 1024;              // most candidates in the bin of the k-th largest one that are ranked directly
-constexpr size_t kSelSmemMax = 227 * 1024 - 1024;            // dynamic shared memory a CTA may ask for (static part left out)
+constexpr size_t kSelSmemMax = 227 * 1024 - 2048;            // dynamic shared memory a CTA may ask for (static part left out)
 constexpr size_t kSelFixedBytes = (size_t)(2 * kSelBins + (kSelCluster + 1) * kSelList) * 4;
 static_assert((size_t)kSelCapCta * 4 + kSelFixedBytes <= kSelSmemMax, "a CTA's share does not fit");
 
+// A share beyond this is sorted into bins only near where a sample has the k-th largest candidate.  That takes 0.5 us for ranking the sample and
+// wins from 7500 candidates a CTA on; where a far outlier in the sample makes the plain range sweep twice, no sooner than here is
+// that slower than three digits of the key were.
+constexpr int kSelLong = 11264;
 // Candidates a CTA: most before the cluster doubles, and most for a block of 256 threads (2000 candidates: 6.9 us in 256 threads, 5.8 in 1024; 444:
 // 4.3 and 8.5).
 constexpr int64_t kSelShare = 4096, kSelShort = 1024;

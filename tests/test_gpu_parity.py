@@ -192,6 +192,37 @@ def test_select_histogram_routes(kind):
             assert np.array_equal(idx.cpu().numpy(), oracle.select(s, 3, 2, k + 5)), (kind, M, k)
 
 
+@pytest.mark.parametrize("M", [8 * 11264, 8 * 11264 + 1, 200000, 360448])
+@pytest.mark.parametrize("kind", ["normal", "outlier", "frames", "equal", "one_bin", "one_bin_in_one_cta", "one_bin_too_many", "extremes"])
+def test_select_long_shares(M, kind):
+    """Shares around the length from which the steps lie near the k-th largest candidate, and the longest one; one bin with as many
+    candidates as are ranked directly, spread over the CTAs or all in one's, and one more; k in the tails."""
+    rng = np.random.default_rng(M)
+    s = rng.standard_normal(M).astype(np.float32)
+    ks = [1, M // 700, M // 2, M - M // 50, M - 1]
+    if kind == "outlier":
+        s[::257] = 1e30
+    elif kind == "frames":
+        s = (0.1 * s + np.repeat(rng.standard_normal(M // 1560 + 1), 1560)[:M]).astype(np.float32)
+    elif kind == "equal":
+        s[:] = -3.5
+    elif kind == "extremes":
+        s = rng.choice(np.array([np.inf, -np.inf, np.nan, 3.4e38, -3.4e38, 1e-44, -1e-44, 0.0, -0.0], np.float32), M)
+    elif kind.startswith("one_bin"):
+        per_cta = (-(-M // 8) + 31) // 32 * 32
+        n = max(256, min(1024, per_cta // 32)) + (kind == "one_bin_too_many")
+        s = (100 * np.sign(s) + s).astype(np.float32)
+        at = rng.permutation(M)[:n] if kind != "one_bin_in_one_cta" else per_cta + rng.permutation(per_cta)[:n]
+        s[at] = (0.001 * rng.standard_normal(n)).astype(np.float32)
+        above = int((s > 50).sum())
+        ks = [above, above + 1, above + n // 2, above + n, above + n + 1]
+    d = torch.from_numpy(s).cuda()
+    for k in ks:
+        idx = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+        pafu.pafu_select(d, pafu.Shape(1, 64, [0, M], None), pafu.make_policy(0, 0, [k], 1), idx)
+        assert np.array_equal(idx.cpu().numpy(), oracle.select(s, 0, 0, k)), (kind, M, k)
+
+
 # ------------------------------------------------------------------------------- compact
 @pytest.mark.parametrize("w", SMALL + [wl.Workload("odd_dm", 7, 5, 8, (77, 9), (30, 9), 2, 3, (4, 4), 32)],
                          ids=lambda w: "%s-dm%d" % (w.name, w.d_model))
