@@ -672,9 +672,11 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
             pol.n_sink = c->n_sink; pol.n_recent = 0; pol.budget = keep;
             e = fill_policy(&sh, &pol, &st);
             if (e != PAFU_OK) return e;
-            e = launch_select(c->SL[from], st, c->idx, cs, 1);
+            // the append's rows in and out, at the copies' rate (6.2 TB/s), against one CTA's selection of 24 576 candidates
+            const bool covered = (double)chunk * (double)dm * 8.0 * c->n_layers / 6.2e6 >= 30.0;
+            e = launch_select(c->SL[from], st, c->idx, cs, 1, covered);
             if (e != PAFU_OK) return e;
-            select_ctas = select_cta_count(st);
+            select_ctas = select_cta_count(st, covered);
         }
         prune = true;
     }

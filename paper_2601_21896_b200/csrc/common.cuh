@@ -132,13 +132,13 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 pafu_status launch_score(const pafu_head& head, const uint16_t* const* X, int n_parts, int64_t n_tokens, int64_t ldx,
                          float* scores, void* ws, size_t ws_bytes, cudaStream_t stream, int beside_predecessor = 0);
 // trigger_late = 1: the kernel behind it may start early, but not before everything ahead of the
-// selection is complete
+// selection is complete.  covered: work beside the selection takes longer than it, on the SMs that it leaves
 pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx,
-                          cudaStream_t stream, int trigger_late = 0);
+                          cudaStream_t stream, int trigger_late = 0, bool covered = false);
 // Selection and row gather of a small step in one launch; *done = false: the step is not small, nothing was launched.
 pafu_status launch_select_compact(const uint16_t* K, const uint16_t* V, const float* scores, const StreamTable& st, int32_t d_model, int32_t* idx,
                                   uint16_t* Kc, uint16_t* Vc, float* SLc, cudaStream_t stream, bool* done);
-int select_cta_count(const StreamTable& st);      // CTAs launch_select's kernels occupy for this geometry
+int select_cta_count(const StreamTable& st, bool covered = false);      // CTAs launch_select's kernels occupy for this geometry
 // work != nullptr (three zeroed words of the workspace header): the rows that are kept whatever
 // the scores say are copied before the kernel waits for its predecessor (only valid when that
 // predecessor is launch_select of the same step)

@@ -583,8 +583,8 @@ select_stream_kernel(const float* __restrict__ scores, StreamTable st, int32_t* 
     }
 }
 
-int select_cta_count(const StreamTable& st) {
-    const SelLaunch pl = plan_select(st);
+int select_cta_count(const StreamTable& st, bool covered) {
+    const SelLaunch pl = plan_select(st, covered);
     return (pl.any_cluster ? st.n_streams * pl.nc : 0) + (pl.any_stream ? st.n_streams : 0);
 }
 
@@ -606,9 +606,9 @@ pafu_status launch_select_compact(const uint16_t* K, const uint16_t* V, const fl
                                     reinterpret_cast<uint4*>(Kc), reinterpret_cast<uint4*>(Vc), SLc));
 }
 
-pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx, cudaStream_t stream, int trigger_late) {
+pafu_status launch_select(const float* scores, const StreamTable& st, int32_t* idx, cudaStream_t stream, int trigger_late, bool covered) {
     if (st.n_streams == 0 || st.cu_B[st.n_streams] == 0) return PAFU_OK;
-    const SelLaunch pl = plan_select(st);
+    const SelLaunch pl = plan_select(st, covered);
     if (pl.any_cluster) {
         static bool done[kMaxDevices] = {};
         if (!once_per_device(done, [] {

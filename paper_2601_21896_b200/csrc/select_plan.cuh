@@ -30,13 +30,17 @@ constexpr int64_t kSelShare = 4096, kSelShort = 1024;
 // streams 28.1, in clusters of four 11.6; 31 of 500 candidates beside one of 20 000 23.1 and 10.7; 16 of 45 000 24.1 and 16.4.
 constexpr int kSelRoom8 = 15 * 8;
 
+// Where other work covers the selection but leaves its SMs out (a rolling cache's append copies), its CTAs are kept few: a cache of
+// 18 720 tokens, 30 layers of 12 heads, eight CTAs 1109 us, one 1098; 28 080 tokens 1660, two 1631; 18 720 of 2 heads 210 and 206.
+constexpr int64_t kSelShareCovered = 24576;
+
 struct SelLaunch {
     bool any_cluster = false, any_stream = false;
     int nc = 1;
     int64_t per_cta = 0;
     int threads() const { return per_cta <= kSelShort ? kSelThreads : kSelThreadsMax; }
 };
-inline SelLaunch plan_select(const StreamTable& st) {
+inline SelLaunch plan_select(const StreamTable& st, bool covered = false) {
     SelLaunch pl;
     int64_t m_max = 0;
     for (int s = 0; s < st.n_streams; ++s) {
@@ -52,7 +56,7 @@ inline SelLaunch plan_select(const StreamTable& st) {
     // 9.4 us on one CTA, 7.9 on two, 7.4 on four; 16 000 10.2 on two, 8.4 on four.
     // They are doubled while all streams' clusters find room on the GPU at once, or one stream's candidates would not fit.
     auto fits = [&](int nc) { return st.n_streams * nc <= (nc < 8 ? 128 : kSelRoom8); };
-    while (pl.nc < kSelCluster && m_max > pl.nc * (fits(2 * pl.nc) ? kSelShare : (int64_t)kSelCapCta)) pl.nc *= 2;
+    while (pl.nc < kSelCluster && m_max > pl.nc * (!fits(2 * pl.nc) ? (int64_t)kSelCapCta : covered ? kSelShareCovered : kSelShare)) pl.nc *= 2;
     pl.per_cta = ((m_max + pl.nc - 1) / pl.nc + 31) / 32 * 32;
     return pl;
 }

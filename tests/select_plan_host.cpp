@@ -29,7 +29,7 @@ extern "C" void plan_copy(int n, const int64_t* T, const int64_t* B, int64_t sin
 }
 
 // out: [CTAs a stream, candidates a CTA, streaming kernel too]
-extern "C" void plan_selection(int n, const int64_t* T, const int64_t* B, int64_t sink, int64_t recent, int64_t* out) {
-    const SelLaunch pl = plan_select(table(n, T, B, sink, recent));
+extern "C" void plan_selection(int n, const int64_t* T, const int64_t* B, int64_t sink, int64_t recent, int covered, int64_t* out) {
+    const SelLaunch pl = plan_select(table(n, T, B, sink, recent), covered != 0);
     out[0] = pl.nc; out[1] = pl.per_cta; out[2] = pl.any_stream;
 }

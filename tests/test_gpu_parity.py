@@ -689,8 +689,10 @@ def test_cache_update_entry_point_over_chunks(chunk, cap, n_sink):
 
 @pytest.mark.parametrize("cap,chunk,N", [
     (1000, 200, 1),                # one selecting CTA
-    (24576 + 16 + 129, 129, 1),    # one candidate more than it takes: two
-    (60001, 700, 1),               # four
+    (4096 + 16 + 129, 129, 1),     # 129 candidates more than it takes: two
+    (9000, 700, 1), (24576 + 16 + 129, 129, 1),    # four, eight
+    (60001, 700, 1),               # eight with longer shares
+    (24592, 8000, 25), (33100, 8000, 25),          # appends that cover the selection: one CTA with the most it takes there, two
     (363001, 800, 1),              # more candidates than a cluster holds: the streaming selection
     # rows of 8, 24, 56 and 200 sixteen-byte units: the 192-unit batches of the row copies hold whole rows, end inside
     # one, or are shorter than one; one row kept or new

@@ -80,10 +80,10 @@ def test_limits_of_small_steps(lib, T, B, sink, chunks, small):
     assert plan_copy(lib, T, B, sink, 0, chunks)[0] == small
 
 
-def plan_selection(lib, M):
+def plan_selection(lib, M, covered=False):
     out = np.zeros(3, dtype=np.int64)
     T, i64 = [m + 5 for m in M], ctypes.c_int64
-    lib.plan_selection(len(M), arr(T), arr([m // 2 + 5 for m in M]), i64(2), i64(3), out.ctypes.data_as(ctypes.c_void_p))
+    lib.plan_selection(len(M), arr(T), arr([m // 2 + 5 for m in M]), i64(2), i64(3), int(covered), out.ctypes.data_as(ctypes.c_void_p))
     return out.tolist()
 
 
@@ -96,3 +96,9 @@ def test_selecting_clusters_fit_on_the_gpu_at_once(lib, M, ctas):
     nc, per_cta, stream = plan_selection(lib, M)
     assert nc == ctas and not stream and per_cta * nc >= max(M) and per_cta <= 45056
     assert nc * len(M) <= (120 if nc == 8 else 128) or max(M) > nc // 2 * 45056
+
+
+@pytest.mark.parametrize("M,ctas", [(16, 1), (17160, 1), (24576, 1), (24577, 2), (49152, 2), (49153, 4), (98305, 8), (360448, 8)])
+def test_covered_selections_leave_few_sms_out(lib, M, ctas):
+    """Beside a rolling cache's append copies, which take longer."""
+    assert plan_selection(lib, [M], covered=True)[0] == ctas
