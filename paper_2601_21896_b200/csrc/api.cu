@@ -693,7 +693,7 @@ pafu_status pafu_cache_update(pafu_cache* c, const pafu_head* head,
             apart = apart || ranges_overlap(x, (size_t)chunk * dm * 2, c->K[to][l] + first * dm, (size_t)(dst0 + chunk - first) * dm * 2) ||
                     ranges_overlap(x, (size_t)chunk * dm * 2, c->V[to][l] + first * dm, (size_t)(dst0 + chunk - first) * dm * 2);
     // rows in and out, at the copies' rate (6.2 TB/s)
-    const bool share = !apart && head_shares_sms(*head, (double)(chunk + keep) * (double)dm * 8.0 * c->n_layers / 6.2e6);
+    const bool share = !apart && head_shares_sms(*head, chunk, (double)(chunk + keep) * (double)dm * 8.0 * c->n_layers / 6.2e6, select_ctas);
     auto copy_rows = [&](int64_t n_new, int64_t n_keep, int sel) {
         return launch_cache_rows(Knew, Vnew, n_new, c->K[from], c->V[from], c->SL[from], c->idx, n_keep, dst0, c->K[to], c->V[to],
                                  c->SL[to], c->n_layers, (int32_t)dm, sel, share, cs);

@@ -157,8 +157,8 @@ pafu_status launch_cache_rows(const uint16_t* const* Knew, const uint16_t* const
                               const uint16_t* const* Ks, const uint16_t* const* Vs, const float* SL, const int32_t* idx,
                               int64_t keep, int64_t dst0, uint16_t* const* Kd, uint16_t* const* Vd, float* SLd, int32_t n_layers,
                               int32_t d_model, int select_ctas, bool share_sms, cudaStream_t stream);
-// Whether the salience head should share the SMs with row copies that take about copy_us.
-bool head_shares_sms(const pafu_head& head, double copy_us);
+// Whether the salience head of n_tokens should share the SMs with row copies that take about copy_us and leave select_ctas SMs to the selection.
+bool head_shares_sms(const pafu_head& head, int64_t n_tokens, double copy_us, int select_ctas);
 pafu_status launch_attn(const uint16_t* Q, const uint16_t* Kc, const uint16_t* Vc,
                         const uint16_t* Kq, const uint16_t* Vq, const StreamTable& st,
                         int32_t n_heads, int32_t d_head, float scale, uint16_t* O, float* LSE,

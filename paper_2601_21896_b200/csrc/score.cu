@@ -19,11 +19,13 @@ pafu_status launch_score(const pafu_head& head, const uint16_t* const* X, int n_
 // take at most kSharePerSlice us for each of the head's reduction slices, of which it needs 0.45 to 1.1 us: 11 layers of 16 heads,
 // 2300 + 700 tokens 126.8 -> 99.6 us; 10 x 12, 4000 + 2000 147.7 -> 133.9; 8 x 12, 4680 + 4680 210.2 -> 200.5; 30 x 6, 2500 + 1500 135.2 -> 130.0.
 // Beyond: 15 x 12, 4680 + 4680 331 both ways; 30 x 12 586 and 607; 25 x 12, 13 000 + 1000 681 and 727.  Narrow heads are over
-// too soon: 10 layers of 2 heads, 5000 + 4000 56.1 and 58.7.
-bool head_shares_sms(const pafu_head& head, double copy_us) {
+// too soon: 10 layers of 2 heads, 5000 + 4000 56.1 and 58.7.  A head of few CTAs runs on the SMs that the copies leave to the selection: 128 tokens, 16 hidden
+// units (one CTA) beside 20 layers of 12 heads, 4000 tokens, 173 us sharing, 159 so; four CTAs beside 6 layers, 12 000 tokens, 162.6 and 151.3.
+bool head_shares_sms(const pafu_head& head, int64_t n_tokens, double copy_us, int select_ctas) {
     constexpr double kSharePerSlice = 3.5;
     constexpr int kShareSlices = 24;
     const int slices = head.d_in / score_tc::kBK;
+    if (score_tc::plan(head, n_tokens, device_sm_count()).grid <= select_ctas) return false;
     return slices >= kShareSlices && copy_us <= kSharePerSlice * slices;
 }
 

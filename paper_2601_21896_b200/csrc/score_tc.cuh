@@ -317,6 +317,27 @@ score_tc_kernel(const __grid_constant__ CUtensorMap mX, const __grid_constant__ 
     if (p.beside) grid_dep_wait();    // what waits for this kernel relies on the one before it as well
 }
 
+// How n_tokens are handed to CTAs.
+struct Work {
+    int split, tail_tiles, grid;
+    unsigned cluster;
+};
+inline Work plan(const pafu_head& head, int64_t n_tokens, int sm_count) {
+    Work w;
+    const int64_t n_tiles = (n_tokens + kBM - 1) / kBM;
+    const int n_chunks = (head.d_hidden + kNMax - 1) / kNMax;
+    // few tokens and a wide head: one CTA per (tile, chunk), clusters of n_chunks CTAs
+    w.split = (n_chunks > 1 && n_tiles * n_chunks <= 2 * (int64_t)sm_count) ? 1 : 0;
+    // tiles that fill at most half of the last round of CTAs (220 tiles on 148 SMs leave 72): each
+    // is shared by the two CTAs of a cluster, half of the hidden units each
+    const int64_t rest = n_tiles % sm_count;
+    w.tail_tiles = !w.split && n_chunks == 1 && head.d_hidden % 32 == 0 && sm_count % 2 == 0 && rest > 0 && 2 * rest <= sm_count ? (int)rest : 0;
+    w.grid = w.split ? (int)(n_tiles * n_chunks) : (int)(n_tiles < sm_count ? n_tiles : sm_count);
+    if (w.tail_tiles > 0 && n_tiles < sm_count) w.grid = 2 * w.tail_tiles;    // no full round at all
+    w.cluster = w.split ? (unsigned)n_chunks : (w.tail_tiles > 0 ? 2u : 1u);
+    return w;
+}
+
 // X[0..n_parts) are the matrices whose rows, side by side, form a token's d_in features
 // (n_parts = 1: a plain [n_tokens, d_in] matrix; 3: query, key and value rows of d_in / 3 each).
 inline pafu_status launch(const pafu_head& head, const uint16_t* const* X, int n_parts, int64_t n_tokens, int64_t ldx,
@@ -333,25 +354,12 @@ inline pafu_status launch(const pafu_head& head, const uint16_t* const* X, int n
     p.act = head.act; p.final = head.final; p.w2 = head.w2; p.b1 = head.b1; p.b2 = head.b2;
     p.scores = scores; p.status = status; p.beside = beside != 0;
     p.k_per_part = d_part / kBK;
-    const int64_t n_tiles = (n_tokens + kBM - 1) / kBM;
-    const int n_chunks = (head.d_hidden + kNMax - 1) / kNMax;
-    // few tokens and a wide head: one CTA per (tile, chunk), clusters of n_chunks CTAs
-    p.split = (n_chunks > 1 && n_tiles * n_chunks <= 2 * (int64_t)sm_count) ? 1 : 0;
-    // tiles that fill at most half of the last round of CTAs (220 tiles on 148 SMs leave 72): each
-    // is shared by the two CTAs of a cluster, half of the hidden units each
-    p.tail_tiles = 0; p.tail_width = 0;
-    const int64_t rest = n_tiles % sm_count;
-    if (!p.split && n_chunks == 1 && head.d_hidden % 32 == 0 && sm_count % 2 == 0 && rest > 0 && 2 * rest <= sm_count) {
-        p.tail_tiles = (int)rest;
-        p.tail_width = head.d_hidden / 2;
-    }
+    const Work w = plan(head, n_tokens, sm_count);
+    p.split = w.split; p.tail_tiles = w.tail_tiles; p.tail_width = w.tail_tiles > 0 ? head.d_hidden / 2 : 0;
     CUtensorMap mWt = mW;
     if (p.tail_tiles > 0 &&
         !TmapEncoder::matrix(&mWt, head.w1, (uint64_t)head.d_hidden, (uint64_t)head.d_in, (uint64_t)head.d_in, (uint32_t)p.tail_width))
         return PAFU_ERR_CUDA;
-    int grid = p.split ? (int)(n_tiles * n_chunks) : (int)(n_tiles < sm_count ? n_tiles : sm_count);
-    if (p.tail_tiles > 0 && n_tiles < sm_count) grid = 2 * p.tail_tiles;      // no full round at all
-    const unsigned cluster = p.split ? (unsigned)n_chunks : (p.tail_tiles > 0 ? 2u : 1u);
     static bool attr_set[kMaxDevices] = {};
     if (!once_per_device(attr_set, [] {
             auto opt_in = [](auto* kernel, int stages) {
@@ -362,7 +370,7 @@ inline pafu_status launch(const pafu_head& head, const uint16_t* const* X, int n
         }))
         return PAFU_ERR_CUDA;
     auto go = [&](auto* kernel, int stages) {
-        return cuda_ok(launch_dependent(kernel, dim3(grid), dim3(kThreads), smem_bytes(stages), stream, cluster, mX[0], mX[1], mX[2], mW, mWt, p));
+        return cuda_ok(launch_dependent(kernel, dim3(w.grid), dim3(kThreads), smem_bytes(stages), stream, w.cluster, mX[0], mX[1], mX[2], mW, mWt, p));
     };
     const bool shared = beside == 2;
     if (head.act == PAFU_ACT_GELU)

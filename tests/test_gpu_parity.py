@@ -738,6 +738,9 @@ def test_cache_updates_without_a_synchronisation_between_them(cap, chunk, N):
     (2, 4, 1000, 700, 64),        # one accumulator: tiles shared by two CTAs
     (40, 4, 3000, 300, 256),      # copies too long for that
     (4, 2, 1000, 500, 1024),      # too narrow a head for that
+    (3, 12, 4000, 128, 16),       # one CTA on the SM that selects
+    (3, 12, 12000, 130, 64), (2, 12, 12000, 128, 1024),    # four on those of a selecting cluster
+    (3, 12, 12000, 257, 64),      # more than those
 ])
 def test_cache_update_head_beside_the_copies(layers, N, cap, chunk, hidden):
     """The salience head beside the row copies, on their SMs or not, gives the bits that it gives alone; the rows are copies."""
