@@ -125,6 +125,9 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
     return launch_dependent_carveout(-1, kernel, grid, block, smem, stream, cluster_x, args...);
 }
 
+// Shared memory of an SM that row copies leave to a salience head beside them, a split that the hardware has; 92 KB of L1 stay.
+constexpr int kHeadSmemBeside = 164 * 1024;
+
 // Launchers (each enqueues on `stream` and returns the launch status).
 // beside_predecessor = 1: the kernel runs beside the one launched before it, which must be
 // launch_cache_rows (that kernel lets it start only once everything before it is complete), and ends after it.

@@ -289,7 +289,7 @@ pafu_status launch_compact_layers(const uint16_t* const* K, const uint16_t* cons
 // 117, 305, 588 and 781; as select, gather, head and append one after the other, many blocks an SM, 140, 164, 324,
 // 612 and 807.  With the indices fetched before the batch's loads instead of behind them 618 at 3072 bytes.)
 constexpr int kCacheSeg = kCompactUnroll * 32;     // units of a warp's batch
-constexpr int kCacheCarveout = 72;                 // per cent of 228 KB: 164 KB of shared memory for the salience head's block
+constexpr int kCacheCarveout = kHeadSmemBeside * 100 / (228 * 1024);     // per cent, which the driver rounds up to the next split: of 72 % it makes 196 KB
 
 // One batch: unit dst + 32 i comes from src[i]; `between` runs while its loads are under way.
 template <typename Between>

@@ -42,7 +42,7 @@ constexpr int kMaxHidden = 1024;
 constexpr int kMaxChunks = kMaxHidden / kNMax;
 constexpr int kStagesShared = 3;     // where it shares the SMs with row copies: leaves them an L1 of 92 KB
 constexpr int smem_bytes(int stages) { return stages * kStageBytes + 2 * kMaxHidden * 4 + 2 * kBM * 4 + kMaxChunks * kBM * 4 + 256 + 1024; }
-static_assert(smem_bytes(kStagesShared) + 1024 + 64 <= 164 * 1024, "the copies' shared-memory share (kCacheCarveout) is 164 KB");
+static_assert(smem_bytes(kStagesShared) + 1024 + 64 <= kHeadSmemBeside, "the head does not fit beside the row copies");
 
 struct Params {
     int64_t n_tokens;
