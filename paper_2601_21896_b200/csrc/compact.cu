@@ -100,7 +100,7 @@ __device__ __forceinline__ int64_t claim_get(int pending) { return __shfl_sync(0
 
 // GROUPS: a warp copies `rows_at_once` narrow rows at a time.  A narrow row alone leaves most of a warp's batch empty: 48 000 rows
 // of 256 bytes, selected from 76 000 in four streams, selection and gather together 56 us, in groups of 12 rows 29.4; 24 000
-// rows of 1280 bytes 45.7 and 39.6.
+// rows of 1280 bytes 45.7 and 39.6.  (At the 80 registers of three blocks an SM the instantiation in groups spills 28 bytes; the other one nothing.)
 template <bool GROUPS>
 __global__ void __launch_bounds__(kCompactWarpsPerBlock * 32, 3)
 compact_rows_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,

@@ -22,8 +22,10 @@ static_assert((size_t)kSelCapCta * 4 + kSelFixedBytes <= kSelSmemMax, "a CTA's s
 // wins from 7500 candidates a CTA on; where a far outlier in the sample makes the plain range sweep twice, no sooner than here is
 // that slower than three digits of the key were.
 constexpr int kSelLong = 11264;
-// Candidates a CTA: most before the cluster doubles, and most for a block of 256 threads (2000 candidates: 6.9 us in 256 threads, 5.8 in 1024; 444:
-// 4.3 and 8.5).
+// Candidates a CTA: most before the cluster doubles, and most for a block of 256 threads.  Doubling from 2048 / 4096 / 8192 on: 4096 candidates 8.5 / 8.4 /
+// 8.4 us, 6000 8.5 / 8.5 / 9.1, 7800 8.6 / 9.2 / 10.2, 10 000 8.6 / 8.5 / 9.7, 16 000 9.2 / 9.4 / 11.3, 30 000 10.6 / 10.6 / 11.9; up to 4096 one CTA also lets a
+// small step select and copy in one launch.  From 6500 to 8192 four CTAs would be the better choice by 0.7 us.  In 256 threads and in
+// 1024: 444 candidates 4.3 and 8.5 us, 2000 6.9 and 5.8; blocks of 512 were not tried.
 constexpr int64_t kSelShare = 4096, kSelShort = 1024;
 
 // Clusters of eight, one block an SM, that the GPU holds at once: 15 streams of 21 840 candidates 10.4 us, 16 18.8 (in clusters of four 11.3); 32
@@ -52,8 +54,7 @@ inline SelLaunch plan_select(const StreamTable& st, bool covered = false) {
         if (M > m_max) m_max = M;
     }
     // CTAs per stream.  A histogram of 1024 candidates costs a CTA some 400 clocks (13 an add and warp, whether or not its
-    // lanes collide), the barriers across CTAs and the trips through distributed shared memory two to three thousand: 7800 candidates
-    // 9.4 us on one CTA, 7.9 on two, 7.4 on four; 16 000 10.2 on two, 8.4 on four.
+    // lanes collide), the barriers across CTAs and the trips through distributed shared memory two to three thousand.
     // They are doubled while all streams' clusters find room on the GPU at once, or one stream's candidates would not fit.
     auto fits = [&](int nc) { return st.n_streams * nc <= (nc < 8 ? 128 : kSelRoom8); };
     while (pl.nc < kSelCluster && m_max > pl.nc * (!fits(2 * pl.nc) ? (int64_t)kSelCapCta : covered ? kSelShareCovered : kSelShare)) pl.nc *= 2;

@@ -141,9 +141,9 @@ def test_select_bit_exact(kind):
              ((4097,), 0, 0, (1,)), ((4097,), 0, 0, (4096,)), ((3000,), 100, 200, (250,)),
              ((3000,), 5000, 0, (1000,)), ((1, 2, 3), 1, 1, (0, 1, 2)), ((28080,), 1560, 4680, (14040,)),
              ((93600,), 1560, 4680, (9360,)),
-             # around the capacities of the two shared-memory key formats (53 248 whole keys, 106 496 upper halves)
+             # longer streams, selected by clusters of eight
              ((53248 + 30,), 10, 20, (20000,)), ((53249 + 30,), 10, 20, (20000,)), ((106496 + 7,), 3, 4, (106000,)),
-             # beyond them: the kernel that re-reads L2 in every pass; and all three paths in one call
+             # shares that look near the k-th largest candidate only; and long and short streams in one call
              ((106497 + 7,), 3, 4, (555,)), ((200000,), 1560, 4680, (20000,)),
              ((1000, 40000, 90000, 200000, 64), 10, 100, (500, 9000, 30000, 50000, 64))]
     for ci, (T, ns, nr, Bs) in enumerate(cases):
@@ -255,7 +255,8 @@ def test_compact_bit_exact(w):
     (64, 1, (47000,), (45000,)),                            # rows of 8 pieces: 12 at once, one selecting cluster
     (64, 1, (9000, 700, 9, 40000), (9000, 650, 0, 39999)),  # four streams, one kept whole, one empty: rows are claimed
     (64, 3, (12000,), (11111,)),                            # 24 pieces, the last group short
-    (128, 6, (11000,), (10700,)),                           # 96 pieces: one row at a time
+    (128, 6, (11000,), (10700,)),                           # 96 pieces: two rows at once
+    (128, 6, (11000,), (10600,)),                           # fewer than three rows a warp: one at a time
 ], ids=lambda v: str(v) if isinstance(v, int) else "x".join(map(str, v)))
 def test_gather_of_narrow_rows(d_head, n_heads, T, B):
     """The row gather's groups of rows, behind the selection inside a step and by itself: every kept row and score is a copy."""
@@ -295,6 +296,34 @@ def test_small_step_selects_and_copies_in_one_launch(d_head, n_heads, T, B, sink
     assert torch.equal(A.idx, S.idx) and torch.equal(A.Kc, S.Kc) and torch.equal(A.Vc, S.Vc)
     assert not slc or torch.equal(A.SLc[:A.nB], S.SLc[:S.nB])
     assert torch.equal(A.O, S.O)
+
+
+@pytest.mark.parametrize("kind", ["equal", "two_values", "not_finite"])
+@pytest.mark.parametrize("T,B", [((700, 333), (300, 100)), ((4096,), (1500,)), ((4000, 30), (3999, 7))], ids=str)
+def test_small_step_with_ties_and_scores_that_are_not_finite(T, B, kind):
+    """Bins that have to be narrowed down, in the launch that selects and copies: the oracle's indices on its scores, and copies."""
+    w = wl.Workload("tied", 9, 2, 64, T, B, 3, 5, (64,) * len(T), 32, final=wl.FINAL_SIGMOID if kind == "two_values" else wl.FINAL_NONE)
+    d = wl.make_layer_device(w, seed=5)
+    if kind == "equal":
+        d["w2"] = torch.zeros_like(d["w2"])
+    elif kind == "two_values":
+        d["w2"] = d["w2"] * 8192.0                               # the sigmoid saturates
+    else:
+        d["w1"][:, 0] = 3.0e38; d["w2"] = d["w2"].abs()          # infinities, NaN (0 x -inf) and zeros of both signs
+    L = Layer(w, d)
+    L.step(); L.check_status()
+    scores, cuT, cuB = L.scores.cpu().numpy(), w.cu("T"), L.cu_B
+    if kind == "two_values":
+        assert np.mean((scores[:cuT[-1]] == 0) | (scores[:cuT[-1]] == 1)) > 0.9
+    elif kind == "not_finite":
+        assert 0.1 < np.mean(~np.isfinite(scores[:cuT[-1]])) < 0.9
+    for s in range(len(T)):
+        ids = oracle.select(scores[cuT[s]:cuT[s + 1]], 3, 5, B[s])
+        assert np.array_equal(L.idx[cuB[s]:cuB[s + 1]].cpu().numpy(), ids)
+        rows = torch.from_numpy(ids.astype(np.int64)).cuda() + int(cuT[s])
+        for got, want in ((L.Kc, L.K), (L.Vc, L.V), (L.SLc, L.scores)):
+            bits = torch.int16 if got.dtype == torch.bfloat16 else torch.int32
+            assert torch.equal(got[cuB[s]:cuB[s + 1]].view(bits), want[rows].view(bits))
 
 
 # ----------------------------------------------------------------------------- attention
@@ -1207,7 +1236,7 @@ def test_full_size_paper_native_point():
 
 
 def test_full_size_long_horizon():
-    # 93 600-token cache pruned to 9360: the streaming select kernel and heavy-tailed scores
+    # 93 600-token cache pruned to 9360: a cluster of eight selects, heavy-tailed scores
     _full_size_check(wl.long_horizon(), n_rows=256, score_rows=8192)
 
 
