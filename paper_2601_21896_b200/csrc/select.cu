@@ -428,18 +428,22 @@ select_cluster_kernel(const float* __restrict__ scores, const __grid_constant__ 
 // 2500 37.5 -> 37.0, 12 x 128 over 3000 (18 MB in and out) 54.1 -> 53.1.  Larger steps keep two launches: their always-kept rows are
 // copied while the selection runs.
 __global__ void __launch_bounds__(kSelThreadsMax, 1)
-select_copy_kernel(const __grid_constant__ CopyShares shares, const float* __restrict__ scores, int32_t keys_bytes,
-                   int32_t* __restrict__ idx, const __grid_constant__ StreamTable st, const uint4* __restrict__ K, const uint4* __restrict__ V,
+select_copy_kernel(const float* __restrict__ scores, const __grid_constant__ StreamTable st, int32_t keys_bytes,
+                   int32_t* __restrict__ idx, const __grid_constant__ CopyShares shares, const uint4* __restrict__ K, const uint4* __restrict__ V,
                    int chunks_per_row, uint4* __restrict__ Kc, uint4* __restrict__ Vc, float* __restrict__ SLc) {
     extern __shared__ __align__(16) unsigned char sel_smem[];
     __shared__ SelShared sh;
     const int b = (int)blockIdx.x, threads = (int)blockDim.x;
-    int s = 0, copy = b, copies = (int)gridDim.x;
-    if (st.n_streams > 1) {                                  // the last stream that begins at or before b
+    int s, copy, copies = shares.equal;
+    if (copies > 0) {
+        s = b / copies;
+        copy = b - s * copies;
+    } else {
+        s = 0;                                               // the last stream that begins at or before b
 #pragma unroll
         for (int d = PAFU_MAX_STREAMS / 2; d > 0; d /= 2)
             if (s + d < st.n_streams && shares.first[s + d] <= b) s += d;
-        copy -= shares.first[s];
+        copy = b - shares.first[s];
         copies = shares.first[s + 1] - shares.first[s];
     }
     int* top = reinterpret_cast<int*>(sel_smem + keys_bytes + kSelFixedBytes);
@@ -601,7 +605,7 @@ pafu_status launch_select_compact(const uint16_t* K, const uint16_t* V, const fl
         return PAFU_ERR_CUDA;
     const int32_t keys_bytes = cp.per_cta * 4;
     return cuda_ok(launch_dependent(select_copy_kernel, dim3((unsigned)cp.shares.first[st.n_streams]), dim3(cp.threads),
-                                    (size_t)keys_bytes * 2 + kSelFixedBytes, stream, 1, cp.shares, scores, keys_bytes, idx, st,
+                                    (size_t)keys_bytes * 2 + kSelFixedBytes, stream, 1, scores, st, keys_bytes, idx, cp.shares,
                                     reinterpret_cast<const uint4*>(K), reinterpret_cast<const uint4*>(V), chunks,
                                     reinterpret_cast<uint4*>(Kc), reinterpret_cast<uint4*>(Vc), SLc));
 }

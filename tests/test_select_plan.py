@@ -42,7 +42,8 @@ def check_shares(lib, T, B, sink, recent, chunks):
         return False
     units = np.minimum(T, B) * chunks
     ctas = np.diff(first)
-    assert first[0] == 0 and np.all((ctas > 0) == (units > 0)) and first[-1] <= SMS
+    assert first[0] == 0 and np.all(ctas[units > 0] > 0) and first[-1] <= SMS
+    assert np.all(ctas == ctas[0]) or np.all(ctas[units == 0] == 0)
     # shares grow by a 64th until all fit; they fit at the latest when the even share leaves one more CTA a stream
     even = max(threads * BATCH, units.sum() / (SMS - len(T)))
     assert max(u / c for u, c in zip(units, ctas) if c) <= even * 65 / 64 + 1
